@@ -156,7 +156,7 @@ wr_status wr_set_sigma_leaf(wr_ctx *ctx, int64_t orders);
  * lane width, with and without the hints) on that matrix's two layouts (a few
  * launches each, CUDA events) and keeps the
  * fastest, per matrix, layout and block width; smaller matrices and autotune
- * off use the default (2 residues for n <= 8, 4 above).  wr_set_lane_width
+ * off use the default (2 residues for n <= 4, 4 above).  wr_set_lane_width
  * forces one (0 = tuned or default).  Results never depend on it. */
 wr_status wr_set_autotune(wr_ctx *ctx, int32_t on);
 /* Route the context's device allocations through the caller's allocator

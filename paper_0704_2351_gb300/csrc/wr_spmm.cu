@@ -251,14 +251,18 @@ template <int NV, int WL>
 void launch_spmm_kernel(wr_ctx *ctx, const SellView &A, const uint32_t *x, uint32_t *y, const uint32_t *scale,
                         unsigned long long *acc64, const ModP &mp, int *term_counter, bool cs,
                         const MultiEpi *me, int part) {
-    const int64_t vblocks = (A.nseg + 7) / 8;
-    const int64_t lblocks = (A.nchunks * Lanes<NV, WL>::G + 7) / 8;
+    const int64_t vblocks = (A.nseg + SPMM_WARPS - 1) / SPMM_WARPS;
+    const int64_t lwork = (A.nchunks * Lanes<NV, WL>::G + SPMM_WARPS - 1) / SPMM_WARPS;
+    // up to four pieces a block once two waves of blocks remain (1.9M rows: 630
+    // us with one piece a block, 580 with four, 582 with eight)
+    const int pieces = (int)std::clamp<int64_t>(lwork / (2 * (int64_t)ctx->num_sms * Tile<NV, WL>::MINB), 1, 4);
+    const int64_t lblocks = (lwork + pieces - 1) / pieces;
     const int64_t blocks = std::max<int64_t>(vblocks + lblocks, term_counter ? 1 : 0);
     if (blocks <= 0) return;
     const MultiEpi one{};
 #define WR_SPMM_LAUNCH(WIDEV, CSV, MULTIV)                                                                     \
-    k_spmm<NV, WL, WIDEV, CSV, MULTIV><<<(unsigned)blocks, 256, 0, ctx->stream>>>(                             \
-        A, x, y, scale, acc64, mp, term_counter, vblocks, me ? *me : one, part)
+    k_spmm<NV, WL, WIDEV, CSV, MULTIV><<<(unsigned)blocks, 32 * SPMM_WARPS, 0, ctx->stream>>>(                 \
+        A, x, y, scale, acc64, mp, term_counter, vblocks, pieces, me ? *me : one, part)
     if constexpr (NV >= 16) {
         if (me && me->jobs > 1) {
             if (A.wvals) {
