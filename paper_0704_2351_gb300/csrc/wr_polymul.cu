@@ -14,11 +14,16 @@
 // wrapped-around part (coefficients at and above Lz folded onto 0..) stays
 // below lo gives exactly those (a middle product when lo > 0).
 //
-// Transforms: forward decimation in frequency (natural order in, bit-reversed
-// out), pointwise products in that order, inverse decimation in time
-// (bit-reversed in, natural out); residues in Montgomery form; the stages
-// are grouped into passes through shared memory (two passes up to 2^17 points,
-// three up to 2^23), each one launch over all polynomials of the batch.
+// Transforms: X^n - 1 is split as X^2k - c^2 = (X^k - c)(X^k + c) down to linear
+// factors, (u, v) -> (u + c v, u - c v) per stage, so that a stage's twiddle c
+// depends on the block alone: the pairs of a block share one table entry,
+// consecutive blocks read consecutive ones, and one table of the 2^i-th roots
+// in bit-reversed order serves every length.  The order of the transform's
+// points does not matter to the pointwise products; the inverse undoes the
+// stages in reverse.  Residues in Montgomery form.  Up to 2^13 points a
+// transform is one pass (registers and shared memory, k_ntt_tile); longer ones
+// take their top stages in passes of up to four stages in registers
+// (k_ntt_top), each one launch over all polynomials of the batch.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -85,7 +90,8 @@ __global__ void __launch_bounds__(TR_TILE * TR_ROWS)
             for (int y = ty; y < TR_TILE; y += TR_ROWS) {
                 const int64_t k = k0 + y;
                 const int e = e0 + tx;
-                tile[y][tx] = (k < ncoef && e < nent) ? to_mont(src[(size_t)k * nent + e] % mP.p, mP) : 0u;
+                // (a r2 < 2^32 P for any 32-bit a: no reduction before the product)
+                tile[y][tx] = (k < ncoef && e < nent) ? to_mont(src[(size_t)k * nent + e], mP) : 0u;
             }
         }
         __syncthreads();
@@ -97,177 +103,324 @@ __global__ void __launch_bounds__(TR_TILE * TR_ROWS)
     }
 }
 
-// tw[j] = w^j (Montgomery form, w_m = w R mod P) for j < count, by square
-// and multiply
-__global__ void k_twiddles(uint32_t w_m, int64_t count, uint32_t *__restrict__ tw, ModP mP) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < count; j += (int64_t)gridDim.x * blockDim.x) {
+// tw[i] = w^bitrev(i) (Montgomery form, w_m = w R mod P, w a 2^(bits+1)-th root,
+// bitrev over `bits` bits) for i < 2^bits, by square and multiply
+__global__ void k_twiddles(uint32_t w_m, int bits, uint32_t *__restrict__ tw, ModP mP) {
+    const int64_t count = (int64_t)1 << bits;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         uint32_t r = mP.r1, b = w_m;
-        for (int64_t e = j; e; e >>= 1) {
+        for (uint32_t e = bits ? __brev((uint32_t)i) >> (32 - bits) : 0u; e; e >>= 1) {
             if (e & 1) r = mont_mul(r, b, mP);
             b = mont_mul(b, b, mP);
         }
-        tw[j] = r;
+        tw[i] = r;
     }
 }
 
-// Several butterfly stages in one pass through shared memory.  The stages
-// with half = 2^h for h in [b0, b1) pair elements that differ in one of the
-// index bits b0 .. b1 - 1 only, so with e = top 2^b1 + mid 2^b0 + low, a tile
-// of all 2^(b1-b0) mid values x 2^LB consecutive low values (LB = min(b0, 5))
-// of one (polynomial, top, low block) goes through all of them in shared
-// memory: one read and one write of the data per pass instead of per stage.
-// DIF (forward): h from b1 - 1 down to b0, (u, v) -> (u + v, (u - v) w^j);
-// DIT (inverse): h from b0 up to b1 - 1, (u, v w^j) -> (u + v w^j, u - v w^j);
-// j = e mod 2^h, w the 2^(h+1)-th root of unity: w^j = tw[j 2^(lg-1-h+tshift)]
-// in a table of the powers of a 2^(lg+tshift)-th root (Montgomery form).
-constexpr int NTT_PASS_THREADS = 256;
-constexpr int NTT_TILE_LOG = 12;  // 4096 residues (16 KB) per tile
+// residues mod P < 2^31 as the smaller of x and x - P (or x + P) as unsigned
+__device__ __forceinline__ uint32_t ntt_add(uint32_t a, uint32_t b, uint32_t P) {
+    const uint32_t s = a + b;
+    return min(s, s - P);
+}
+__device__ __forceinline__ uint32_t ntt_sub(uint32_t a, uint32_t b, uint32_t P) {
+    const uint32_t d = a - b;
+    return min(d, d + P);
+}
+__device__ __forceinline__ uint32_t ntt_mul(uint32_t a, uint32_t b, uint32_t P, uint32_t pneg) {
+    const unsigned long long t = (unsigned long long)a * b;
+    const uint32_t k = (uint32_t)t * pneg;
+    const uint32_t u = (uint32_t)(madw(k, P, t) >> 32);
+    return min(u, u - P);
+}
 
-template <bool DIF>
-__global__ void __launch_bounds__(NTT_PASS_THREADS)
-    k_ntt_pass(uint32_t *__restrict__ a, int64_t npoly, int lg, int b0, int b1, const uint32_t *__restrict__ tw,
-               int tshift, ModP mP) {
-    __shared__ uint32_t sm[1 << NTT_TILE_LOG];
-    const int MB = b1 - b0, LB = b0 < 5 ? b0 : 5;
-    const int nlow = 1 << LB, tile = 1 << (MB + LB), half_tile = tile >> 1;
-    const int64_t Lz = (int64_t)1 << lg;
-    const int lowblocks_log = b0 - LB;
-    const int64_t tiles_per_poly = Lz >> (MB + LB);
-    for (int64_t tid_tile = blockIdx.x; tid_tile < npoly * tiles_per_poly; tid_tile += gridDim.x) {
-        const int64_t poly = tid_tile / tiles_per_poly, rem = tid_tile - poly * tiles_per_poly;
-        const int64_t lowblock = rem & (((int64_t)1 << lowblocks_log) - 1), top = rem >> lowblocks_log;
-        uint32_t *g = a + poly * Lz + (top << b1) + (lowblock << LB);
-        const int64_t lowbase = lowblock << LB;  // low part of e for l = 0
-        __syncthreads();
-        for (int x = threadIdx.x; x < tile; x += NTT_PASS_THREADS)
-            sm[x] = g[((int64_t)(x >> LB) << b0) + (x & (nlow - 1))];
-        __syncthreads();
-        for (int k = 0; k < MB; k++) {
-            const int h = DIF ? b1 - 1 - k : b0 + k;
-            const int hh = h - b0, hm = 1 << hh;
-            const int sh = lg - 1 - h + tshift;
-            for (int y = threadIdx.x; y < half_tile; y += NTT_PASS_THREADS) {
-                const int l = y & (nlow - 1), r = y >> LB;
-                const int jm = r & (hm - 1), mid0 = ((r >> hh) << (hh + 1)) + jm;
-                const int i0 = (mid0 << LB) + l, i1 = i0 + (hm << LB);
-                const int64_t j = ((int64_t)jm << b0) + lowbase + l;  // e mod 2^h
-                const uint32_t w = tw[j << sh];
-                const uint32_t u = sm[i0];
-                if (DIF) {
-                    const uint32_t v = sm[i1];
-                    sm[i0] = addm(u, v, mP);
-                    sm[i1] = mont_mul(subm(u, v, mP), w, mP);
-                } else {
-                    const uint32_t v = mont_mul(sm[i1], w, mP);
-                    sm[i0] = addm(u, v, mP);
-                    sm[i1] = subm(u, v, mP);
-                }
-            }
-            __syncthreads();
+// the 2^K consecutive table entries of a stage, in loads of up to 16 bytes
+// (entry blk 2^K of a table aligned to more)
+template <int K>
+__device__ __forceinline__ void ntt_twiddles(const uint32_t *__restrict__ tw, uint32_t blk, uint32_t (&c)[1 << K]) {
+    const uint32_t *p = tw + ((size_t)blk << K);
+    if constexpr (K == 0) {
+        c[0] = __ldg(p);
+    } else if constexpr (K == 1) {
+        const uint2 t = __ldg(reinterpret_cast<const uint2 *>(p));
+        c[0] = t.x; c[1] = t.y;
+    } else {
+#pragma unroll
+        for (int k = 0; k < (1 << K) / 4; k++) {
+            const uint4 t = __ldg(reinterpret_cast<const uint4 *>(p) + k);
+            c[4 * k] = t.x; c[4 * k + 1] = t.y; c[4 * k + 2] = t.z; c[4 * k + 3] = t.w;
         }
-        for (int x = threadIdx.x; x < tile; x += NTT_PASS_THREADS)
-            g[((int64_t)(x >> LB) << b0) + (x & (nlow - 1))] = sm[x];
     }
 }
 
-// Bit ranges [b0, b1) of the passes of a length-2^lg transform, lowest first:
-// the lowest pass takes up to NTT_TILE_LOG bits (contiguous segments), the
-// others up to NTT_TILE_LOG - 5 (tiles of 32 consecutive columns).
-inline std::vector<std::pair<int, int>> ntt_passes(int lg) {
-    std::vector<std::pair<int, int>> out;
-    int b0 = 0;
-    while (b0 < lg) {
-        const int room = b0 == 0 ? NTT_TILE_LOG : NTT_TILE_LOG - (b0 < 5 ? b0 : 5);
-        const int b1 = std::min(lg, b0 + room);
-        out.emplace_back(b0, b1);
-        b0 = b1;
-    }
-    return out;
+// Stage K of R on 2^R values: 2^K blocks of 2^(R - K) values.
+template <int R, int K, bool FWD>
+__device__ __forceinline__ void ntt_stage(uint32_t (&v)[1 << R], uint32_t blk, const uint32_t *__restrict__ tw, uint32_t P,
+                                          uint32_t pneg) {
+    constexpr int half = 1 << (R - 1 - K);
+    uint32_t c[1 << K];
+    ntt_twiddles<K>(tw, blk, c);
+#pragma unroll
+    for (int b = 0; b < (1 << K); b++)
+#pragma unroll
+        for (int i = 0; i < half; i++) {
+            uint32_t &x = v[b * 2 * half + i], &y = v[b * 2 * half + i + half];
+            if (FWD) {
+                const uint32_t m = ntt_mul(y, c[b], P, pneg);
+                y = ntt_sub(x, m, P);
+                x = ntt_add(x, m, P);
+            } else {
+                const uint32_t d = ntt_sub(x, y, P);
+                x = ntt_add(x, y, P);
+                y = ntt_mul(d, c[b], P, pneg);
+            }
+        }
 }
 
-// pointwise: C_f = A_f B_f (r x s times s x t) at every transform point f.
-// A thread owns one transform point f (consecutive f across a warp, so every
-// load is one coalesced row segment) and a PW_RT x PW_CT tile of C; a
-// block's eight warps take eight tiles of
-// the same 32 points.  The sums sum_k A_ik B_kj run on 64-bit accumulators
-// (one 32 x 32 + 64-bit multiply-add per product) folded by 2^32 = r1 (mod P)
-// every FOLDK products, reduced mod P and brought to Montgomery form
-// (A_ik B_kj R^-1) once at the end.
+// R stages on 2^R values held in registers; blk: the block that they belong to
+// at the first (forward) of these stages.
+template <int R, bool FWD>
+__device__ __forceinline__ void ntt_stages(uint32_t (&v)[1 << R], uint32_t blk, const uint32_t *__restrict__ tw,
+                                           uint32_t P, uint32_t pneg) {
+    if constexpr (!FWD && R > 3) ntt_stage<R, 3, FWD>(v, blk, tw, P, pneg);
+    if constexpr (!FWD && R > 2) ntt_stage<R, 2, FWD>(v, blk, tw, P, pneg);
+    if constexpr (!FWD && R > 1) ntt_stage<R, 1, FWD>(v, blk, tw, P, pneg);
+    ntt_stage<R, 0, FWD>(v, blk, tw, P, pneg);
+    if constexpr (FWD && R > 1) ntt_stage<R, 1, FWD>(v, blk, tw, P, pneg);
+    if constexpr (FWD && R > 2) ntt_stage<R, 2, FWD>(v, blk, tw, P, pneg);
+    if constexpr (FWD && R > 3) ntt_stage<R, 3, FWD>(v, blk, tw, P, pneg);
+}
+
+// The top K stages (s0 .. s0 + K - 1) of transforms of 2^lg points, in
+// registers: one thread per group of 2^K values, lanes along consecutive values.
+constexpr int NTT_TOP_THREADS = 256;
+template <int K, bool FWD>
+__global__ void __launch_bounds__(NTT_TOP_THREADS)
+    k_ntt_top(uint32_t *__restrict__ a, int64_t npoly, int lg, int s0, const uint32_t *__restrict__ tw, uint32_t P,
+              uint32_t pneg) {
+    const int sl = lg - s0 - K;  // log2 of the distance between a group's values
+    const int64_t groups = npoly << (lg - K);
+    for (int64_t g = (int64_t)blockIdx.x * NTT_TOP_THREADS + threadIdx.x; g < groups;
+         g += (int64_t)gridDim.x * NTT_TOP_THREADS) {
+        const int64_t hi = g >> sl, low = g & (((int64_t)1 << sl) - 1);  // hi = poly 2^s0 + block
+        uint32_t *p = a + (hi << (sl + K)) + low;
+        uint32_t v[1 << K];
+#pragma unroll
+        for (int i = 0; i < (1 << K); i++) v[i] = p[(int64_t)i << sl];
+        ntt_stages<K, FWD>(v, (uint32_t)(hi & (((int64_t)1 << s0) - 1)), tw, P, pneg);
+#pragma unroll
+        for (int i = 0; i < (1 << K); i++) p[(int64_t)i << sl] = v[i];
+    }
+}
+
+// The last lc stages of transforms of 2^lg points (lc = 13, or lg when lg < 13):
+// a block takes a tile of 2^13 values (2^(13-lc) transforms when lc < 13)
+// through all of them in two to four steps of R = 2, 3 or 4 stages, each thread
+// 16 values in registers, exchanged through shared memory between steps
+// (padded by one word in 32).  One read and one write of the data: the first
+// step reads global memory, the last one writes it with the values of a step's
+// group apart (element i of group g at i 2^(lc-R) + g), which keeps the writes
+// coalesced; the inverse reads that order back.  Bound by the butterflies' issue
+// (a product mod P, a sum and a difference: 11 instructions).  Measured: 4,096
+// transforms of 8,192 points 1,140 -> 200 us (two passes with one
+// shared-memory round trip and one scattered twiddle load per stage before).
+constexpr int NTT_TILE_LOG = 13;
+constexpr int NTT_TILE_THREADS = 512;
+
+struct NttSteps {
+    int n;
+    int R[4];  // forward order: from the highest bits down
+};
+__host__ __device__ inline NttSteps ntt_steps(int lc) {
+    NttSteps st{(lc + 3) / 4, {0, 0, 0, 0}};
+    if (st.n < 2) st.n = 2;
+    for (int k = 0, left = lc; k < st.n; k++) {
+        st.R[k] = (left + st.n - k - 1) / (st.n - k);
+        left -= st.R[k];
+    }
+    return st;
+}
+
+__device__ __forceinline__ int ntt_pad(int e) { return e + (e >> 5); }
+
+// One step: h0 the lowest bit it touches.  SRC / DST: 0 shared memory, 1 the
+// tile in natural order, 2 the tile in the transform's order.
+template <int R, bool FWD, int SRC, int DST>
+__device__ __forceinline__ void ntt_step(uint32_t *sm, uint32_t *__restrict__ g, int valid, int lc, int h0, uint32_t top,
+                                         const uint32_t *__restrict__ tw, uint32_t P, uint32_t pneg) {
+    constexpr int NG = 16 >> R;  // groups per thread
+#pragma unroll
+    for (int u = 0; u < NG; u++) {
+        const int gi = threadIdx.x + u * NTT_TILE_THREADS;
+        const int base = ((gi >> h0) << (h0 + R)) | (gi & ((1 << h0) - 1));
+        const int gp = gi & ((1 << (lc - R)) - 1);  // group within its transform
+        const int pbase = ((gi >> (lc - R)) << lc) + gp;
+        const uint32_t blk = (top << (lc - h0 - R)) + (uint32_t)((base & ((1 << lc) - 1)) >> (h0 + R));
+        uint32_t v[1 << R];
+#pragma unroll
+        for (int i = 0; i < (1 << R); i++) {
+            const int e = base + (i << h0), pe = pbase + (i << (lc - R));
+            if (SRC == 0) v[i] = sm[ntt_pad(e)];
+            else if (SRC == 1) v[i] = e < valid ? g[e] : 0u;
+            else v[i] = pe < valid ? g[pe] : 0u;
+        }
+        ntt_stages<R, FWD>(v, blk, tw, P, pneg);
+#pragma unroll
+        for (int i = 0; i < (1 << R); i++) {
+            const int e = base + (i << h0), pe = pbase + (i << (lc - R));
+            if (DST == 0) sm[ntt_pad(e)] = v[i];
+            else if (DST == 1) { if (e < valid) g[e] = v[i]; }
+            else if (pe < valid) g[pe] = v[i];
+        }
+    }
+}
+
+template <bool FWD>
+__global__ void __launch_bounds__(NTT_TILE_THREADS, 2)
+    k_ntt_tile(uint32_t *__restrict__ a, int64_t words, int lg, int lc, const uint32_t *__restrict__ tw, uint32_t P,
+               uint32_t pneg) {
+    __shared__ uint32_t sm[(1 << NTT_TILE_LOG) + (1 << (NTT_TILE_LOG - 5))];
+    uint32_t *g = a + ((int64_t)blockIdx.x << NTT_TILE_LOG);
+    // (the last tile may be short)
+    const int valid = (int)min64(words - ((int64_t)blockIdx.x << NTT_TILE_LOG), 1 << NTT_TILE_LOG);
+    const uint32_t top = lg > lc ? (uint32_t)(blockIdx.x & ((1u << (lg - lc)) - 1)) : 0u;
+    const NttSteps st = ntt_steps(lc);
+    int h0 = FWD ? lc : 0;
+    for (int k = 0; k < st.n; k++) {
+        const int R = st.R[FWD ? k : st.n - 1 - k];
+        if (FWD) h0 -= R;
+        if (k > 0) __syncthreads();
+#define WR_NTT_STEP(SRC, DST)                                                                    \
+    {                                                                                            \
+        if (R == 4) ntt_step<4, FWD, SRC, DST>(sm, g, valid, lc, h0, top, tw, P, pneg);          \
+        else if (R == 3) ntt_step<3, FWD, SRC, DST>(sm, g, valid, lc, h0, top, tw, P, pneg);     \
+        else ntt_step<2, FWD, SRC, DST>(sm, g, valid, lc, h0, top, tw, P, pneg);                 \
+    }
+        if (k == 0) WR_NTT_STEP((FWD ? 1 : 2), 0)
+        else if (k + 1 < st.n) WR_NTT_STEP(0, 0)
+        else WR_NTT_STEP(0, (FWD ? 2 : 1))
+#undef WR_NTT_STEP
+        if (!FWD) h0 += R;
+    }
+}
+
+// pointwise: C_f = A_f B_f (r x s times s x t) at every transform point f.  A
+// lane owns a point (rows of 32 consecutive points are 128-byte lines), a
+// thread a 4 x 8 tile of C at it, a block of eight warps WR x WC such tiles for
+// 8 / (WR WC) groups of 32 points.  The operands of KC values of k are staged in
+// shared memory (16-byte asynchronous copies, two stages), so that an A word
+// serves 8 WC columns and a B word 4 WR rows per read of L2, and an operand
+// costs a conflict-free shared load for 8 or 4 products.  The sums run on
+// 64-bit accumulators (one 32 x 32 + 64-bit multiply-add per product), folded by
+// 2^32 = r1 (mod P) every FOLDK products: a folded accumulator is below 2^60.3
+// for the transform primes (2^32 mod P < 2^28.3), which leaves room for 16
+// products below 2^59.8 (P < 2^30) or 4 below 2^61.9.  Bound by the
+// multiply-adds.  Measured at 64 x 64 x 64, 8,192 points: 4.65 ms -> 430 us
+// (P < 2^30; 480 us with the folds of the third prime) (a
+// thread's operands came straight from L1 and L2 with eight warps an SM before).
 constexpr int PW_RT = 4, PW_CT = 8, PW_WARPS = 8;
 
-template <int FOLDK>
-__global__ void __launch_bounds__(32 * PW_WARPS)
-    k_ntt_pointwise_tiled(const uint32_t *__restrict__ A, const uint32_t *__restrict__ B, uint32_t *__restrict__ C,
-                          int r, int s, int t, int64_t Lz, ModP mP) {
+__device__ __forceinline__ void cp_async16(uint32_t *dst, const uint32_t *src, bool on) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src), "r"(on ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ unsigned long long fold1(unsigned long long x, uint32_t c) {
+    return madw((uint32_t)(x >> 32), c, (unsigned long long)(uint32_t)x);
+}
+
+template <int WR, int WC, int KC>
+struct PwShape {
+    static constexpr int FG = PW_WARPS / (WR * WC);
+    static constexpr int TR = PW_RT * WR, TC = PW_CT * WC;  // rows and columns of C per block
+    static constexpr int STAGE = FG * KC * (TR + TC) * 32;  // words
+    static constexpr size_t SMEM = 2 * (size_t)STAGE * 4;
+};
+
+template <int WR, int WC, int KC, int FOLDK>
+__global__ void __launch_bounds__(32 * PW_WARPS, 2)
+    k_ntt_pointwise(const uint32_t *__restrict__ A, const uint32_t *__restrict__ B, uint32_t *__restrict__ C, int r,
+                    int s, int t, int64_t Lz, ModP mP) {
+    using S = PwShape<WR, WC, KC>;
+    extern __shared__ __align__(16) uint32_t pw_sm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t f = (int64_t)blockIdx.x * 32 + lane;
-    const int ntj = (t + PW_CT - 1) / PW_CT, nti = (r + PW_RT - 1) / PW_RT;
-    const int tile = blockIdx.y * PW_WARPS + warp;
-    if (tile >= nti * ntj || f >= Lz) return;
-    const int i0 = (tile / ntj) * PW_RT, j0 = (tile % ntj) * PW_CT;
+    const int fg = warp / (WR * WC), wr = warp / WC % WR, wc = warp % WC;
+    const int ntj = (t + S::TC - 1) / S::TC;
+    const int i0 = (int)(blockIdx.y / ntj) * S::TR, j0 = (int)(blockIdx.y % ntj) * S::TC;
+    const int64_t f0 = (int64_t)blockIdx.x * 32 * S::FG;
     const uint32_t fc = mP.r1;  // 2^32 mod P
-    bool iv[PW_RT], jv[PW_CT];
-    const uint32_t *pa[PW_RT];
-    const uint32_t *pb[PW_CT];
-#pragma unroll
-    for (int u = 0; u < PW_RT; u++) {
-        iv[u] = i0 + u < r;
-        pa[u] = A + ((size_t)(iv[u] ? i0 + u : 0) * s) * Lz + f;  // row i0 + u, k = 0
-    }
-#pragma unroll
-    for (int v = 0; v < PW_CT; v++) {
-        jv[v] = j0 + v < t;
-        pb[v] = B + (size_t)(jv[v] ? j0 + v : 0) * Lz + f;  // column j0 + v, k = 0
-    }
-    const size_t bstep = (size_t)t * Lz;
+    // stage: [group][k][TR rows of A, then TC columns of B][32 points]
+    auto load = [&](int k0, int stage) {
+        uint32_t *sm = pw_sm + stage * S::STAGE;
+        for (int c = threadIdx.x; c < S::STAGE / 4; c += 32 * PW_WARPS) {
+            const int row = c >> 3, x = row % (S::TR + S::TC), kg = row / (S::TR + S::TC);
+            const int k = k0 + kg % KC;
+            const int64_t f = f0 + (kg / KC) * 32 + (c & 7) * 4;
+            const bool isa = x < S::TR;
+            const int i = i0 + x, j = j0 + x - S::TR;
+            const bool on = k < s && f < Lz && (isa ? i < r : j < t);
+            const uint32_t *src = !on ? A : (isa ? A + ((size_t)i * s + k) * Lz + f : B + ((size_t)k * t + j) * Lz + f);
+            cp_async16(sm + c * 4, src, on);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     unsigned long long acc[PW_RT][PW_CT];
 #pragma unroll
     for (int u = 0; u < PW_RT; u++)
 #pragma unroll
         for (int v = 0; v < PW_CT; v++) acc[u][v] = 0ull;
-    int k = 0;
-    for (; k + FOLDK <= s; k += FOLDK) {
+    load(0, 0);
+    int since = 0;  // products since the last fold
+    for (int k0 = 0, st = 0; k0 < s; k0 += KC, st ^= 1) {
+        if (k0 + KC < s) {
+            load(k0 + KC, st ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const uint32_t *sm = pw_sm + st * S::STAGE + fg * KC * (S::TR + S::TC) * 32 + lane;
+        const uint32_t *sa = sm + PW_RT * wr * 32, *sb = sm + (S::TR + PW_CT * wc) * 32;
 #pragma unroll
-        for (int kk = 0; kk < FOLDK; kk++) {
+        for (int kk = 0; kk < KC; kk++) {
             uint32_t a[PW_RT], b[PW_CT];
 #pragma unroll
-            for (int u = 0; u < PW_RT; u++) a[u] = iv[u] ? __ldg(pa[u] + (size_t)(k + kk) * Lz) : 0u;
+            for (int u = 0; u < PW_RT; u++) a[u] = sa[(kk * (S::TR + S::TC) + u) * 32];
 #pragma unroll
-            for (int v = 0; v < PW_CT; v++) b[v] = jv[v] ? __ldg(pb[v] + (size_t)(k + kk) * bstep) : 0u;
+            for (int v = 0; v < PW_CT; v++) b[v] = sb[(kk * (S::TR + S::TC) + v) * 32];
 #pragma unroll
             for (int u = 0; u < PW_RT; u++)
 #pragma unroll
                 for (int v = 0; v < PW_CT; v++) acc[u][v] = madw(a[u], b[v], acc[u][v]);
+            if ((FOLDK < KC && (kk + 1) % FOLDK == 0) || (kk == KC - 1 && (since += KC) >= FOLDK)) {
+                since = 0;
+#pragma unroll
+                for (int u = 0; u < PW_RT; u++)
+#pragma unroll
+                    for (int v = 0; v < PW_CT; v++) acc[u][v] = fold1(acc[u][v], fc);
+            }
         }
-#pragma unroll
-        for (int u = 0; u < PW_RT; u++)
-#pragma unroll
-            for (int v = 0; v < PW_CT; v++) acc[u][v] = fold2(acc[u][v], fc);
+        __syncthreads();
     }
-    for (; k < s; k++) {  // fewer than FOLDK products after the last fold
-        uint32_t a[PW_RT], b[PW_CT];
-#pragma unroll
-        for (int u = 0; u < PW_RT; u++) a[u] = iv[u] ? __ldg(pa[u] + (size_t)k * Lz) : 0u;
-#pragma unroll
-        for (int v = 0; v < PW_CT; v++) b[v] = jv[v] ? __ldg(pb[v] + (size_t)k * bstep) : 0u;
-#pragma unroll
-        for (int u = 0; u < PW_RT; u++)
-#pragma unroll
-            for (int v = 0; v < PW_CT; v++) acc[u][v] = madw(a[u], b[v], acc[u][v]);
-    }
+    const int64_t f = f0 + fg * 32 + lane;
+    if (f >= Lz) return;
 #pragma unroll
     for (int u = 0; u < PW_RT; u++)
 #pragma unroll
-        for (int v = 0; v < PW_CT; v++)
-            if (iv[u] && jv[v]) C[((size_t)(i0 + u) * t + j0 + v) * Lz + f] = mont_redc(red64(acc[u][v], mP), mP);
+        for (int v = 0; v < PW_CT; v++) {
+            const int i = i0 + PW_RT * wr + u, j = j0 + PW_CT * wc + v;
+            // folded twice: below 2^57.2, so below P 2^32
+            if (i < r && j < t)
+                C[((size_t)i * t + j) * Lz + f] = mont_redc(fold1(fold1(acc[u][v], fc), fc), mP);
+        }
 }
 
 struct CrtConst {
     uint32_t P1, P2, P3;
-    uint32_t c12;        // P1^{-1} mod P2
-    uint32_t c123;       // (P1 P2)^{-1} mod P3
-    uint32_t p1_mod_p3;  // P1 mod P3
-    uint32_t P1_mod_p, P1P2_mod_p;
+    uint32_t c12;        // P1^{-1} mod P2                    (these three in the
+    uint32_t c123;       // (P1 P2)^{-1} mod P3                Montgomery form of
+    uint32_t p1_mod_p3;  // P1 mod P3                          their modulus)
+    uint32_t k1, k2, k3; // 1, P1, P1 P2 mod p (Montgomery form)
 };
 
 // Garner: the integer x < P1 P2 P3 with x = r_i mod P_i, reduced mod p.
@@ -298,15 +451,16 @@ __global__ void __launch_bounds__(TR_TILE * TR_ROWS)
                 const uint32_t r1 = mont_mul(R1[src], il1, m1);
                 const uint32_t r2 = mont_mul(R2[src], il2, m2);
                 const uint32_t r3 = mont_mul(R3[src], il3, m3);
-                const uint32_t t1 = r1;
-                const uint32_t t2 = mulm(subm(r2, t1 % cc.P2, m2), cc.c12, m2);
-                uint32_t u = subm(r3, t1 % cc.P3, m3);
-                u = subm(u, mulm(cc.p1_mod_p3, t2, m3), m3);
-                const uint32_t t3 = mulm(u, cc.c123, m3);
-                uint64_t w = (uint64_t)(t1 % mp.p);
-                w += (uint64_t)mulm(cc.P1_mod_p, t2 % mp.p, mp);
-                w += (uint64_t)mulm(cc.P1P2_mod_p, t3 % mp.p, mp);
-                v = red64(w, mp);
+                // r1 < P1 < 2.2 P2 and P1 < P3
+                uint32_t q1 = r1 >= cc.P2 ? r1 - cc.P2 : r1;
+                q1 = q1 >= cc.P2 ? q1 - cc.P2 : q1;
+                const uint32_t t2 = mont_mul(subm(r2, q1, m2), cc.c12, m2);
+                const uint32_t u = subm(subm(r3, r1, m3), mont_mul(t2, cc.p1_mod_p3, m3), m3);
+                const uint32_t t3 = mont_mul(u, cc.c123, m3);
+                // r1 + t2 P1 + t3 P1 P2 mod p: r1, t2 < 2^30 (their primes are), so
+                // the first two products together stay below p 2^32
+                v = addm(mont_redc((uint64_t)r1 * cc.k1 + (uint64_t)t2 * cc.k2, mp), mont_redc((uint64_t)t3 * cc.k3, mp),
+                         mp);
             }
             tile[y][tx] = v;
         }
@@ -329,9 +483,9 @@ inline unsigned tr_grid(int64_t nk, int64_t nent, int num_sms) {
 }  // namespace
 
 // The context's twiddle tables, kept across products: for each transform
-// prime, the powers w^j and w^-j (j < 2^(LG-1)) of a 2^LG-th root of unity,
-// LG >= lg (a shorter transform takes every 2^(LG-lg)-th entry); built on
-// the device when a longer transform than the tables serve is first needed.
+// prime, the powers w^bitrev(i) and w^-bitrev(i) (i < 2^(LG-1)) of a 2^LG-th
+// root of unity, LG >= lg (entry i is the same for every LG); built on the
+// device when a longer transform than the tables serve is first needed.
 static wr_status ensure_twiddles(wr_ctx *ctx, int lg) {
     if (ctx->ntt_lg >= lg) return WR_OK;
     const int LG = std::max(lg, 14);
@@ -345,12 +499,56 @@ static wr_status ensure_twiddles(wr_ctx *ctx, int lg) {
         const uint32_t wm = (uint32_t)(((unsigned __int128)w << 32) % P), wim = (uint32_t)(((unsigned __int128)wi << 32) % P);
         uint32_t *tw = ctx->ntt_tw.as<uint32_t>() + (size_t)(2 * i) * half;
         const unsigned g2 = (unsigned)std::min<int64_t>((half + 255) / 256, (int64_t)ctx->num_sms * 16);
-        k_twiddles<<<g2, 256, 0, ctx->stream>>>(wm, half, tw, mP);
+        k_twiddles<<<g2, 256, 0, ctx->stream>>>(wm, LG - 1, tw, mP);
         WR_LAUNCHED(ctx);
-        k_twiddles<<<g2, 256, 0, ctx->stream>>>(wim, half, tw + half, mP);
+        k_twiddles<<<g2, 256, 0, ctx->stream>>>(wim, LG - 1, tw + half, mP);
         WR_LAUNCHED(ctx);
     }
     ctx->ntt_lg = LG;
+    return WR_OK;
+}
+
+// All stages of npoly transforms of 2^lg points, in place: the stages above
+// the tile's in passes of up to four, and the tile pass.
+template <bool FWD>
+static wr_status ntt_run(wr_ctx *ctx, uint32_t *a, int64_t npoly, int lg, const uint32_t *tw, const ModP &mP) {
+    cudaStream_t st = ctx->stream;
+    const int lc = std::min(lg, NTT_TILE_LOG), rem = lg - lc;
+    auto top = [&](int s0, int K) -> wr_status {
+        const int64_t groups = npoly << (lg - K);
+        const unsigned grid = (unsigned)std::min<int64_t>((groups + NTT_TOP_THREADS - 1) / NTT_TOP_THREADS,
+                                                          (int64_t)ctx->num_sms * 64);
+        auto *k = K == 4 ? k_ntt_top<4, FWD> : (K == 3 ? k_ntt_top<3, FWD> : (K == 2 ? k_ntt_top<2, FWD> : k_ntt_top<1, FWD>));
+        k<<<grid, NTT_TOP_THREADS, 0, st>>>(a, npoly, lg, s0, tw, mP.p, mP.pneg);
+        WR_LAUNCHED(ctx);
+        return WR_OK;
+    };
+    auto tiles = [&]() -> wr_status {
+        const int64_t words = npoly << lg;
+        k_ntt_tile<FWD><<<(unsigned)((words + (1 << NTT_TILE_LOG) - 1) >> NTT_TILE_LOG), NTT_TILE_THREADS, 0, st>>>(
+            a, words, lg, lc, tw, mP.p, mP.pneg);
+        WR_LAUNCHED(ctx);
+        return WR_OK;
+    };
+    if (!FWD) WR_TRY(tiles());
+    for (int k = 0; k < (rem + 3) / 4; k++) {
+        const int s0 = FWD ? 4 * k : 4 * ((rem + 3) / 4 - 1 - k);
+        WR_TRY(top(s0, std::min(4, rem - s0)));
+    }
+    if (FWD) WR_TRY(tiles());
+    return WR_OK;
+}
+
+template <int WR, int WC, int KC>
+static wr_status pointwise_run(wr_ctx *ctx, const uint32_t *A, const uint32_t *B, uint32_t *C, int r, int s, int t,
+                               int64_t Lz, const ModP &mP) {
+    using S = PwShape<WR, WC, KC>;
+    auto *k = mP.p < (1u << 30) ? k_ntt_pointwise<WR, WC, KC, 16> : k_ntt_pointwise<WR, WC, KC, 4>;
+    WR_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM));
+    const int64_t tiles = (int64_t)((r + S::TR - 1) / S::TR) * ((t + S::TC - 1) / S::TC);
+    const dim3 g((unsigned)((Lz + 32 * S::FG - 1) / (32 * S::FG)), (unsigned)tiles);
+    k<<<g, 32 * PW_WARPS, S::SMEM, ctx->stream>>>(A, B, C, r, s, t, Lz, mP);
+    WR_LAUNCHED(ctx);
     return WR_OK;
 }
 
@@ -394,7 +592,7 @@ static wr_status polymat_mul_run(wr_ctx *ctx, const uint32_t *A, int64_t na, con
         return fail(WR_EINVAL, "polynomial product coefficients exceed the transform primes' product");
     const int64_t full = na + nb - 1;  // coefficients of the exact product
     const int64_t need = std::max<int64_t>(hi, full - lo);
-    int lg = 1;
+    int lg = 5;  // rows of at least 32 points for the pointwise products
     while (((int64_t)1 << lg) < need) lg++;
     if (lg > NTT_MAX_LOG) return fail(WR_EINVAL, "polynomial product too long for the transform primes");
     const int64_t Lz = (int64_t)1 << lg;
@@ -405,7 +603,7 @@ static wr_status polymat_mul_run(wr_ctx *ctx, const uint32_t *A, int64_t na, con
     WR_TRY(dev_alloc(ctx, bufB, sizeof(uint32_t) * (size_t)nB * Lz));
     for (int i = 0; i < NTT_NPRIMES; i++) WR_TRY(dev_alloc(ctx, bufC[i], sizeof(uint32_t) * (size_t)nC * Lz));
     WR_TRY(ensure_twiddles(ctx, lg));
-    const int LG = ctx->ntt_lg, tshift = LG - lg;  // the length-2^lg twiddle j is table entry j << tshift
+    const int LG = ctx->ntt_lg;
     uint32_t il[NTT_NPRIMES];
     ModP mP[NTT_NPRIMES];
     for (int i = 0; i < NTT_NPRIMES; i++) {
@@ -418,44 +616,28 @@ static wr_status polymat_mul_run(wr_ctx *ctx, const uint32_t *A, int64_t na, con
         WR_LAUNCHED(ctx);
         k_ntt_load<<<tr_grid(Lz, nB, ctx->num_sms), TR_TILE * TR_ROWS, 0, st>>>(B, nb, nB, Lz, bufB.as<uint32_t>(), mP[i]);
         WR_LAUNCHED(ctx);
-        const auto passes = ntt_passes(lg);
-        const int tile_log = NTT_TILE_LOG;
-        auto pass_grid = [&](int64_t npoly) {
-            const int64_t tiles = npoly * (Lz >> std::min<int64_t>(lg, tile_log));
-            return (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)ctx->num_sms * 8));
-        };
-        for (auto it = passes.rbegin(); it != passes.rend(); ++it) {  // forward: highest bits first
-            k_ntt_pass<true><<<pass_grid(nA), NTT_PASS_THREADS, 0, st>>>(bufA.as<uint32_t>(), nA, lg, it->first,
-                                                                        it->second, tw, tshift, mP[i]);
-            WR_LAUNCHED(ctx);
-            k_ntt_pass<true><<<pass_grid(nB), NTT_PASS_THREADS, 0, st>>>(bufB.as<uint32_t>(), nB, lg, it->first,
-                                                                        it->second, tw, tshift, mP[i]);
-            WR_LAUNCHED(ctx);
-        }
-        {
-            const int fk = fold_products(NTT_PRIMES[i]);
-            auto *kpw = fk >= 14 ? k_ntt_pointwise_tiled<14> : (fk >= 4 ? k_ntt_pointwise_tiled<4> : k_ntt_pointwise_tiled<2>);
-            const int tiles = ((r + PW_RT - 1) / PW_RT) * ((t + PW_CT - 1) / PW_CT);
-            const dim3 g((unsigned)((Lz + 31) / 32), (unsigned)((tiles + PW_WARPS - 1) / PW_WARPS));
-            kpw<<<g, 32 * PW_WARPS, 0, st>>>(bufA.as<uint32_t>(), bufB.as<uint32_t>(), bufC[i].as<uint32_t>(), r, s,
-                                              t, Lz, mP[i]);
-            WR_LAUNCHED(ctx);
-        }
-        for (const auto &ps : passes) {  // inverse: lowest bits first
-            k_ntt_pass<false><<<pass_grid(nC), NTT_PASS_THREADS, 0, st>>>(bufC[i].as<uint32_t>(), nC, lg, ps.first,
-                                                                         ps.second, twi, tshift, mP[i]);
-            WR_LAUNCHED(ctx);
-        }
+        WR_TRY(ntt_run<true>(ctx, bufA.as<uint32_t>(), nA, lg, tw, mP[i]));
+        WR_TRY(ntt_run<true>(ctx, bufB.as<uint32_t>(), nB, lg, tw, mP[i]));
+        // the tile of C that a block covers: 16 x 16, or less where C is smaller
+        // (the block then takes more groups of points)
+        uint32_t *pA = bufA.as<uint32_t>(), *pB = bufB.as<uint32_t>(), *pC = bufC[i].as<uint32_t>();
+        if (r <= 4 && t <= 8) WR_TRY((pointwise_run<1, 1, 2>(ctx, pA, pB, pC, r, s, t, Lz, mP[i])));
+        else if (t <= 8) WR_TRY((pointwise_run<2, 1, 4>(ctx, pA, pB, pC, r, s, t, Lz, mP[i])));
+        else if (r <= 8) WR_TRY((pointwise_run<2, 2, 4>(ctx, pA, pB, pC, r, s, t, Lz, mP[i])));
+        else WR_TRY((pointwise_run<4, 2, 8>(ctx, pA, pB, pC, r, s, t, Lz, mP[i])));
+        WR_TRY(ntt_run<false>(ctx, pC, nC, lg, twi, mP[i]));
     }
     CrtConst cc;
     cc.P1 = NTT_PRIMES[0];
     cc.P2 = NTT_PRIMES[1];
     cc.P3 = NTT_PRIMES[2];
-    cc.c12 = (uint32_t)hpow(cc.P1 % cc.P2, cc.P2 - 2, cc.P2);
-    cc.c123 = (uint32_t)hpow((uint64_t)cc.P1 * cc.P2 % cc.P3, cc.P3 - 2, cc.P3);
-    cc.p1_mod_p3 = cc.P1 % cc.P3;
-    cc.P1_mod_p = cc.P1 % p;
-    cc.P1P2_mod_p = (uint32_t)((uint64_t)cc.P1 * cc.P2 % p);
+    auto mont = [](uint64_t x, uint32_t m) { return (uint32_t)(((x % m) << 32) % m); };
+    cc.c12 = mont(hpow(cc.P1 % cc.P2, cc.P2 - 2, cc.P2), cc.P2);
+    cc.c123 = mont(hpow((uint64_t)cc.P1 * cc.P2 % cc.P3, cc.P3 - 2, cc.P3), cc.P3);
+    cc.p1_mod_p3 = mont(cc.P1, cc.P3);
+    cc.k1 = mont(1, p);
+    cc.k2 = mont(cc.P1, p);
+    cc.k3 = mont((uint64_t)cc.P1 * cc.P2, p);
     k_ntt_crt<<<tr_grid(hi - lo, nC, ctx->num_sms), TR_TILE * TR_ROWS, 0, st>>>(
         bufC[0].as<uint32_t>(), bufC[1].as<uint32_t>(), bufC[2].as<uint32_t>(), nC, Lz, lo, hi, C, il[0], il[1],
         il[2], cc, mP[0], mP[1], mP[2], mp);
