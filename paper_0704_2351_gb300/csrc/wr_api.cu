@@ -6,6 +6,7 @@
 #include <chrono>
 #include <cstring>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <thread>
 #include <vector>
@@ -37,8 +38,44 @@ void DevBuf::release() {
     bytes = 0;
 }
 
+DevPool::DevPool(int device) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    uint64_t keep = POOL_KEEP;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+        cudaGetLastError();  // the device's default pool serves
+        pool = nullptr;
+    } else {
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+}
+
+// (memory still in use, a matrix's say, keeps the pool alive until it is freed)
+DevPool::~DevPool() {
+    if (pool) cudaMemPoolDestroy(pool);
+}
+
+std::shared_ptr<DevPool> device_pool(int device) {
+    static std::mutex mu;
+    static std::weak_ptr<DevPool> pools[128];
+    static unsigned long long ids[128];
+    if (device < 0 || device >= 128) return std::make_shared<DevPool>(device);
+    cudaFree(nullptr);  // the device's CUDA context exists from here on
+    const unsigned long long id = current_context_id();
+    std::lock_guard<std::mutex> lk(mu);
+    std::shared_ptr<DevPool> p = pools[device].lock();
+    if (!p || id == 0 || ids[device] != id) {  // (a pool does not outlive a device reset)
+        p = std::make_shared<DevPool>(device);
+        pools[device] = p;
+        ids[device] = id;
+    }
+    return p;
+}
+
 // Device buffers come from the caller's allocator when one is set
-// (wr_set_allocator), else from the stream-ordered pool (cudaMallocAsync);
+// (wr_set_allocator), else from the context's stream-ordered pool;
 // either way they are used on ctx->stream only and returned on it.
 wr_status dev_alloc(wr_ctx *ctx, DevBuf &b, size_t bytes) {
     b.release();
@@ -50,7 +87,8 @@ wr_status dev_alloc(wr_ctx *ctx, DevBuf &b, size_t bytes) {
         b.free_fn = ctx->free_fn;
         b.free_user = ctx->alloc_user;
     } else {
-        cudaError_t e = cudaMallocAsync(&p, bytes, ctx->stream);
+        cudaError_t e = ctx->pool && ctx->pool->pool ? cudaMallocFromPoolAsync(&p, bytes, ctx->pool->pool, ctx->stream)
+                                                     : cudaMallocAsync(&p, bytes, ctx->stream);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(WR_ENOMEM, std::string("device allocation of ") + std::to_string(bytes) +
@@ -189,6 +227,7 @@ extern "C" wr_status wr_create(wr_ctx **out, int device, void *cuda_stream) {
     int optin = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     c->smem_optin = (size_t)optin;
+    c->pool = device_pool(device);
     *out = c;
     return WR_OK;
 }

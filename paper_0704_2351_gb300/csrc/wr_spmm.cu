@@ -1262,7 +1262,7 @@ typedef int (*CtxGetCurrentFn)(void **);
 typedef int (*CtxGetIdFn)(void *, unsigned long long *);
 
 // unique ID of the calling thread's current context, 0 if unknown
-static unsigned long long current_context_id() {
+unsigned long long current_context_id() {
     static CtxGetCurrentFn get_current = nullptr;
     static CtxGetIdFn get_id = nullptr;
     static std::once_flag once;
