@@ -125,9 +125,9 @@ wr_status wr_set_profiling(wr_ctx *ctx, int on);
 wr_status wr_last_timings(const wr_ctx *ctx, wr_timings *out);
 /* Orders per chunk of the blocked sigma-basis (1..64; 0 = automatic).  The
  * result does not depend on it; the time does: each chunk runs its M-Basis
- * steps in one thread block, whose work per order grows with the chunk, while
- * the discrepancy and product kernels around it do the same total work for
- * any chunk size and cost a few launches per chunk. */
+ * steps in one cluster of thread blocks, whose work per order grows with the
+ * chunk, while the discrepancy and product kernels around it do the same total
+ * work for any chunk size and cost a few launches per chunk. */
 wr_status wr_set_sigma_chunk(wr_ctx *ctx, int32_t orders);
 /* Sigma-bases of more than `orders` orders (>= 64) are computed by PM-Basis
  * (Section 2.4): halved recursively down to leaves of at most `orders`
@@ -136,8 +136,8 @@ wr_status wr_set_sigma_chunk(wr_ctx *ctx, int32_t orders);
  * transforms over three FFT primes and the CRT.  The result is the same basis
  * bit for bit; a leaf as large as the sequence turns PM-Basis off.  0
  * (default) = automatic: PM-Basis with 8,192-order leaves for sequences longer
- * than 131,072 orders when m + n <= 32, with 512-order leaves for sequences
- * longer than 2,048 orders when m + n > 32, the blocked M-Basis otherwise.
+ * than 131,072 orders when m + n <= 32, with 256-order leaves for sequences
+ * longer than 1,024 orders when m + n > 32, the blocked M-Basis otherwise.
  * With the pipeline (wr_set_pipeline) PM-Basis trails the sequence in
  * segments, each about half of the orders still to come but at most a
  * quarter of all (down to two leaves): a segment's residual against the

@@ -78,12 +78,13 @@ struct ModP {
 
 ModP make_modp(uint32_t p);
 
-// Products below (p-1)^2 that fit in a 64-bit accumulator on top of what
-// fold2 by c = 2^32 mod p leaves (at most c^2 + 2^32 - 1): the fold interval
-// of the lazily reduced sums (at least 2 for p < 2^31, 14 for p < 2^30).
-inline int fold_products(uint32_t p) {
+// Products of at most (p-1)^2 that fit in a 64-bit accumulator on top of what
+// fold1 by c = 2^32 mod p leaves (at most (c + 1)(2^32 - 1)): at least 12 for
+// p <= 2^30, where c < p; at least 4 below 2^31 (there c is 2^32 - 3p < 2^30 or
+// 2^32 - 2p, which leaves 2p 2^32 >= 4 p^2).
+inline int fold1_products(uint32_t p) {
     const unsigned __int128 c = ((unsigned __int128)1 << 32) % p;
-    const unsigned __int128 after = c * c + (((unsigned __int128)1 << 32) - 1);
+    const unsigned __int128 after = (c + 1) * (((unsigned __int128)1 << 32) - 1);
     const unsigned __int128 room = (((unsigned __int128)1 << 64) - 1) - after;
     const unsigned __int128 prod = (unsigned __int128)(p - 1) * (p - 1);
     return prod ? (int)std::min<unsigned __int128>(room / prod, 1000) : 1000;
@@ -120,6 +121,11 @@ __device__ __forceinline__ unsigned long long madw(uint32_t a, uint32_t b, unsig
 // instead of a reduction mod p.
 __device__ __forceinline__ unsigned long long fold2(unsigned long long x, uint32_t c) {
     x = madw((uint32_t)(x >> 32), c, (unsigned long long)(uint32_t)x);
+    return madw((uint32_t)(x >> 32), c, (unsigned long long)(uint32_t)x);
+}
+
+// the same folded once: at most (c + 1)(2^32 - 1), room for fold1_products(p) more
+__device__ __forceinline__ unsigned long long fold1(unsigned long long x, uint32_t c) {
     return madw((uint32_t)(x >> 32), c, (unsigned long long)(uint32_t)x);
 }
 

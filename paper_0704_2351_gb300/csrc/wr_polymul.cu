@@ -315,8 +315,8 @@ __global__ void __launch_bounds__(NTT_TILE_THREADS, 2)
 // for the transform primes (2^32 mod P < 2^28.3), which leaves room for 16
 // products below 2^59.8 (P < 2^30) or 4 below 2^61.9.  Bound by the
 // multiply-adds.  Measured at 64 x 64 x 64, 8,192 points: 4.65 ms -> 430 us
-// (P < 2^30; 480 us with the folds of the third prime) (a
-// thread's operands came straight from L1 and L2 with eight warps an SM before).
+// (P < 2^30; 480 us with the third prime's folds; before, a
+// thread's operands came straight from L1 and L2, with eight warps an SM).
 constexpr int PW_RT = 4, PW_CT = 8, PW_WARPS = 8;
 
 __device__ __forceinline__ void cp_async16(uint32_t *dst, const uint32_t *src, bool on) {
@@ -325,10 +325,6 @@ __device__ __forceinline__ void cp_async16(uint32_t *dst, const uint32_t *src, b
                  "l"(src), "r"(on ? 16 : 0)
                  : "memory");
 }
-__device__ __forceinline__ unsigned long long fold1(unsigned long long x, uint32_t c) {
-    return madw((uint32_t)(x >> 32), c, (unsigned long long)(uint32_t)x);
-}
-
 template <int WR, int WC, int KC>
 struct PwShape {
     static constexpr int FG = PW_WARPS / (WR * WC);

@@ -43,7 +43,7 @@ size_t rank_device_bytes(const wr_ctx *ctx, const wr_matrix *mat, const Resolved
     const size_t nsplit = (size_t)(mat->a.nsplit + mat->at.nsplit);
     const size_t seq = 4 * N * nv + 4 * M * nv + 4 * (3 * N + 2 * M) + 4 * N * m + 8 * nv * nsplit + 8 * L * m * n;
     const size_t keep = 4 * L * m * n + 4 * (L + 2) * n * q + 4 * q;
-    size_t sigma = 4 * (L + 2) * n * q + 4 * (size_t)(2 * num_sms) * 64 * m * q + 4 * 65 * q * q + 4 * (m * q + 4 * q);
+    size_t sigma = 4 * (L + 2) * n * q + 4 * (size_t)(3 * num_sms) * 64 * m * q + 4 * 65 * q * q + 4 * (m * q + 4 * q);
     if (sigma_uses_pm(ctx, (int64_t)L, (int)m, (int)n)) {
         // PM-Basis: the residual F, three bases of up to L/2 + 2 coefficients
         // (the basis so far, a segment's or half's, their product), one

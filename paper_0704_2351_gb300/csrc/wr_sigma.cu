@@ -14,7 +14,7 @@
 //            last m rows (the only coefficient of those rows that can still
 //            matter: their degree is below the shifted degree <= k0 + 1);
 //   local  : the b orders of M-Basis on the window alone, building the
-//            chunk's transform Mloc (q x q, degree <= b)  (one block);
+//            chunk's transform Mloc (q x q, degree <= b)  (one cluster);
 //   apply  : P <- P Mloc  (many blocks).
 // The transforms are those of the order-by-order algorithm (the product of
 // the same elementary steps), so P and the degrees are bit-identical to it.
@@ -83,121 +83,143 @@ __global__ void k_quiet(const uint32_t *__restrict__ E, int bb, int m, int n, in
     }
 }
 
-// ---- window.  Block b takes coefficients t in [b tper, (b+1) tper) and
-// writes its partial E_i = sum_t S[k0+i-t] P[t] (mod p) for all i < bb into
-// Epart[b]; k_sum_parts adds the partials.
-constexpr int WIN_THREADS = 256;
-constexpr int WIN_IB = 8;  // orders per thread (IB = 4 for chunks of at most 4 orders)
-constexpr int WIN_CB = 4;  // columns per thread
-static_assert(WIN_CB == 4, "the 16-byte loads assume tiles of 4 columns");
+// ---- block-Toeplitz products mod p: the window and the transform product.
+//
+// C[R][c] = sum_{v in [v0, v1), f < nf} A[R][(v, f)] B[v nf + f][c] for R < rows,
+// c < q, with A[R][(v, f)] = M[(R + (off - v) me) nf + f] (0 outside M's mrows rows):
+//   window: R = i m + a, E_i = sum_t S_{k0 + i - t} P_t    (M = S, me = m, off = k0, B = P)
+//   apply : R = t nr + r, P'_t = sum_s P_{t - s} Ml_s       (M = P, me = nr, off = 0, B = Ml)
+// A block computes 4,096 / NC rows x NC columns (NC = 16, 32 or 64 >= q), a thread
+// 4 x 4 of them on 64-bit accumulators; chunks of 16 (v, f) pairs go through double-
+// buffered shared memory (rows of A one word apart, so that a thread's operands are
+// two 16-byte loads for 16 products).  An accumulator is folded by 2^32 mod p after
+// FOLDK products (below p^2 each, on top of a folded value: fold1_products).
+// The window's v range is split over blockIdx.y, one partial sum each, added by
+// k_sum_parts.  Bound by the 64-bit multiply-adds (a quarter of the issue rate).
+// Measured on GB300, average over a whole sigma-basis: q = 64, 4,098 orders in
+// 256-order leaves, 16 orders a chunk 55 us a launch (with 512-order leaves and 4
+// orders a chunk, one block per SM that held its operands' coefficients whole in
+// shared memory, window 141 and product 131 us); q = 16, 11,252 orders, 64 a chunk
+// 69 us (window 85, product 154 us).
+constexpr int TP_THREADS = 256, TP_K = 16;
 
-// Four consecutive residues from shared memory (one 16-byte load when VEC),
-// zero where the column is out of range.
-template <bool VEC>
-__device__ __forceinline__ void ld4(const uint32_t *p, const bool (&cv)[4], uint32_t (&v)[4]) {
-    if constexpr (VEC) {
-        const uint4 t = *reinterpret_cast<const uint4 *>(p);
-        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-    } else {
-#pragma unroll
-        for (int u = 0; u < 4; u++) v[u] = cv[u] ? p[u] : 0u;
+template <int NC>
+struct Toep {
+    static constexpr int BR = 4096 / NC;   // rows per block
+    static constexpr int TX = NC / 4;
+    static constexpr int AW = BR * TP_K / TP_THREADS, BW = NC * TP_K / TP_THREADS;  // words a thread loads
+};
+
+struct ToepArgs {
+    const uint32_t *M, *B;
+    uint32_t *C;
+    int64_t rows;       // rows of C (at most, see limit)
+    int64_t mrows, off; // rows of M, offset in units of me rows
+    int me, nf, q;
+    int64_t v0, vend, vper;  // block y: v in [v0 + y vper, v0 + (y + 1) vper) below vend
+    int64_t cstride;         // words between the partial sums of consecutive y
+    const int *vmax;         // window: vend is also at most *vmax + 1 (the basis degree)
+    const int *rmax;         // apply: rows at most (*rmax + 1) me (the new degree)
+    const int32_t *degl;     // apply: v at most the largest of the q local degrees
+};
+
+template <int NC, int FOLDK>
+__global__ void __launch_bounds__(TP_THREADS, 2) k_toeplitz(ToepArgs g, ModP mp) {
+    using T = Toep<NC>;
+    __shared__ __align__(16) uint32_t As[2][TP_K][T::BR + 4], Bs[2][TP_K][NC + 4];
+    const int tid = threadIdx.x;
+    int64_t rows = g.rows, vend = g.vend;
+    if (g.rmax) rows = min64(rows, ((int64_t)*g.rmax + 1) * g.me);
+    const int64_t R0 = (int64_t)blockIdx.x * T::BR;
+    if (R0 >= rows) return;
+    if (g.vmax) vend = min64(vend, (int64_t)*g.vmax + 1);
+    if (g.degl) {
+        int d = 0;
+        for (int c = tid & 31; c < g.q; c += 32) d = max(d, g.degl[c]);
+        d = __reduce_max_sync(0xffffffffu, d);
+        vend = min64(vend, (int64_t)d + 1);
     }
-}
-
-// Discrepancies of one chunk: E_i = sum_t S_{k0+i-t} P_t for orders
-// i < bb (m x q each), the coefficients t of P split over the blocks (each
-// writes its partial sums, reduced mod p, to Epart[block]).  A thread owns a
-// WIN_IB x WIN_CB tile (orders i0.. x columns c0..) of one row a.  For a fixed
-// r it walks the coefficients t of the tile: the S residues the tile needs at
-// step t+1 are those of step t shifted by one order, so they live in a
-// circular register window that takes one new shared-memory load per step
-// (slot indices are compile-time in an IB-fold unrolled loop), and the
-// WIN_CB residues of P are one 16-byte load (VEC: q a multiple of 4).
-template <int FOLDK, bool VEC, int IB>
-__global__ void __launch_bounds__(WIN_THREADS, 1)
-    k_window(const uint32_t *__restrict__ S, int64_t L, int m, int n, int q, const uint32_t *__restrict__ P,
-             int64_t k0, int bb, int TT, int64_t tper, const int *__restrict__ dmax_dev,
-             uint32_t *__restrict__ Epart, ModP mp) {
-    extern __shared__ uint32_t sm[];
-    const int mn = m * n, nq = n * q, mq = m * q;
-    static_assert(IB == 4 || IB == 8, "order tiles of 4 or 8");
-    const int nib = (bb + IB - 1) / IB, ncb = (q + WIN_CB - 1) / WIN_CB;
-    const int items = nib * m * ncb;
+    const int64_t va = g.v0 + (int64_t)blockIdx.y * g.vper, vb = min64(va + g.vper, vend);
+    const int nf = g.nf, q = g.q;
     const uint32_t fc = mp.r1;  // 2^32 mod p
-    uint32_t *out = Epart + (size_t)blockIdx.x * bb * mq;
-    const int64_t tmax = min64((int64_t)*dmax_dev, k0 + bb - 1);
-    const int64_t tb0 = (int64_t)blockIdx.x * tper;
-    const int64_t tb1 = min64(tb0 + tper, tmax + 1);
-    uint32_t *Ps = sm;                          // [TT][n][q]
-    uint32_t *Ss = sm + (size_t)TT * nq;        // [nib*IB + TT - 1][m][n]
-    for (int round = 0; round * WIN_THREADS < items; round++) {
-        const int it = round * WIN_THREADS + threadIdx.x;
-        const bool act = it < items;
-        const int cb = act ? it % ncb : 0;
-        const int a = act ? (it / ncb) % m : 0;
-        const int i0 = act ? (it / (ncb * m)) * IB : 0;
-        const int c0 = cb * WIN_CB;
-        bool cv[WIN_CB];
+    const int64_t ka = va * nf, kb = vb * nf;  // (v, f) pairs k = v nf + f
+    // this thread's loads of a chunk: pair kl of rows rl, rl + 16, ...; words of B
+    const int kl = tid % TP_K, rl = tid / TP_K;
+    uint32_t ra[T::AW], rb[T::BW];
+    // (v, f) of this thread's pair, advanced by TP_K a chunk
+    int64_t v = (ka + kl) / nf;
+    int f = (int)((ka + kl) - v * nf);
+    auto load = [&](int64_t k) {
+        const bool kv = k + kl < kb;
+        const int64_t row = R0 + rl + (g.off - v) * g.me;
+        const uint32_t *src = g.M + row * nf + f;
 #pragma unroll
-        for (int u = 0; u < WIN_CB; u++) cv[u] = c0 + u < q;
-        Acc2 acc[IB][WIN_CB];
+        for (int u = 0; u < T::AW; u++) {
+            const int64_t rr = row + u * (TP_THREADS / TP_K);
+            ra[u] = (kv && rr >= 0 && rr < g.mrows) ? __ldg(src + (int64_t)u * (TP_THREADS / TP_K) * nf) : 0u;
+        }
 #pragma unroll
-        for (int k = 0; k < IB; k++)
+        for (int u = 0; u < T::BW; u++) {
+            const int w = tid + u * TP_THREADS, c = w % NC;
+            const int64_t kk = k + w / NC;
+            rb[u] = (kk < kb && c < q) ? __ldg(g.B + kk * q + c) : 0u;
+        }
+        f += TP_K;
+        while (f >= nf) { f -= nf; v++; }
+    };
+    auto store = [&](int b) {
 #pragma unroll
-            for (int u = 0; u < WIN_CB; u++) acc[k][u] = Acc2{0u, 0u};
-        int cnt = 0;
-        for (int64_t t0 = tb0; t0 < tb1; t0 += TT) {
-            const int tt_n = (int)min64(TT, tb1 - t0);
-            const int64_t smin = k0 - (t0 + tt_n - 1);
-            const int srows = nib * IB + tt_n - 1;
-            __syncthreads();
-            for (int x = threadIdx.x; x < tt_n * nq; x += WIN_THREADS) Ps[x] = P[(size_t)t0 * nq + x];
-            for (int x = threadIdx.x; x < srows * mn; x += WIN_THREADS) {
-                const int64_t sidx = smin + x / mn;
-                Ss[x] = (sidx >= 0 && sidx < L) ? S[(size_t)sidx * mn + x % mn] : 0u;
-            }
-            __syncthreads();
-            if (!act) continue;
-            // order i0+k at coefficient t0+s reads S row smin + (i0 + k + tt_n - 1 - s) = row top - s + k
-            const int top = i0 + tt_n - 1;
-            for (int r = 0; r < n; r++) {
-                const uint32_t *scol = Ss + a * n + r;      // row u at scol[u * mn]
-                const uint32_t *pcol = Ps + r * q + c0;     // coefficient s at pcol[s * nq]
-                uint32_t sw[IB];                            // row top - s + k in slot (k - s) mod IB
+        for (int u = 0; u < T::AW; u++) As[b][kl][rl + u * (TP_THREADS / TP_K)] = ra[u];
 #pragma unroll
-                for (int k = 0; k < IB; k++) sw[k] = scol[(size_t)(top + k) * mn];
-                for (int s0 = 0; s0 < tt_n; s0 += IB) {
+        for (int u = 0; u < T::BW; u++) {
+            const int w = tid + u * TP_THREADS;
+            Bs[b][w / NC][w % NC] = rb[u];
+        }
+    };
+    unsigned long long acc[4][4];
 #pragma unroll
-                    for (int j = 0; j < IB; j++) {
-                        const int st = s0 + j;
-                        if (st < tt_n) {
-                            if (st > 0) sw[(IB - j) & (IB - 1)] = scol[(size_t)(top - st) * mn];
-                            uint32_t pv[WIN_CB];
-                            ld4<VEC>(pcol + (size_t)st * nq, cv, pv);
+    for (int i = 0; i < 4; i++)
 #pragma unroll
-                            for (int k = 0; k < IB; k++)
+        for (int j = 0; j < 4; j++) acc[i][j] = 0ull;
+    const int tx = tid % T::TX, ty = tid / T::TX;
+    if (ka < kb) {
+        load(ka);
+        store(0);
+        __syncthreads();
+        int b = 0;
+        for (int64_t k = ka; k < kb; k += TP_K, b ^= 1) {
+            const bool more = k + TP_K < kb;
+            if (more) load(k + TP_K);
 #pragma unroll
-                                for (int u = 0; u < WIN_CB; u++) mac2(acc[k][u], sw[(k - j) & (IB - 1)], pv[u]);
-                            if (++cnt == FOLDK) {
+            for (int kk = 0; kk < TP_K; kk++) {
+                const uint4 a4 = *reinterpret_cast<const uint4 *>(&As[b][kk][4 * ty]);
+                const uint4 b4 = *reinterpret_cast<const uint4 *>(&Bs[b][kk][4 * tx]);
+                const uint32_t av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
-                                for (int k = 0; k < IB; k++)
+                for (int i = 0; i < 4; i++)
 #pragma unroll
-                                    for (int u = 0; u < WIN_CB; u++) fold2w(acc[k][u], fc);
-                                cnt = 0;
-                            }
-                        }
-                    }
+                    for (int j = 0; j < 4; j++) acc[i][j] = madw(av[i], bv[j], acc[i][j]);
+                if ((kk + 1) % FOLDK == 0) {
+#pragma unroll
+                    for (int i = 0; i < 4; i++)
+#pragma unroll
+                        for (int j = 0; j < 4; j++) acc[i][j] = fold1(acc[i][j], fc);
                 }
             }
-        }
-        if (act) {
-#pragma unroll
-            for (int k = 0; k < IB; k++) {
-                const int i = i0 + k;
-#pragma unroll
-                for (int u = 0; u < WIN_CB; u++)
-                    if (i < bb && cv[u]) out[(size_t)(i * m + a) * q + c0 + u] = red64(acc2_u64(acc[k][u]), mp);
+            if (more) {
+                store(b ^ 1);
+                __syncthreads();
             }
+        }
+    }
+    uint32_t *out = g.C + (int64_t)blockIdx.y * g.cstride;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int64_t R = R0 + 4 * ty + i;
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int c = 4 * tx + j;
+            if (R < rows && c < q) out[R * q + c] = red64(acc[i][j], mp);
         }
     }
 }
@@ -221,60 +243,27 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// ---- local M-Basis over the window: one block, bb orders.
-//
-// The device keeps the basis in fraction-free form, M_g = M diag(S): the
-// elimination of a discrepancy whose columns are scaled by nonzero constants
-// picks the same pivots and yields the same reduced columns up to column
-// scales, so M_g stays a column-scaled copy of the order-by-order basis.  S
-// (per column, product of the scales of all orders) is divided out of P once
-// at the end.
-//
-// Warp 0 runs the critical path: per order it eliminates the discrepancy with
-// one column per lane (q <= 32; k_local_wide takes wider blocks), right-looking and fraction-free in
-// Montgomery form -- when the current column (in (degree, index) order) is
-// nonzero it becomes a pivot and every later column is reduced by it at once,
-// so each column is reduced by exactly the pivots created before it.  It
-// publishes the order's transform, new[j] = s_j old[j] + sum_t F[t][j]
-// old[pc[t]], and keeps the degree bookkeeping.  The other warps apply the
-// transform: first to window rows i and i+1 (the next discrepancy; warp 0
-// waits for these), then to rows i+2.., to Qtop (coefficient x^k of the last
-// m rows of M) and to the chunk transform Ml.  Named barriers hand the orders
-// over: T_i (transform i published; warp 0 arrives, the others wait) and RR_i
-// (rows i, i+1 done; the others arrive, warp 0 waits).  Phases alternate
-// between two ids per barrier, so a barrier is reused only after its previous
-// phase completed: the arrivals of phase k + 2 are ordered after a wait that
-// needs phase k complete.  There is no spin-wait.  Multiplying column c by x
-// moves no data: window column c is read at row i' - sh[c], and Ml column c
-// holds its coefficient s at row base[c] + s; the other warps use per-order
-// snapshots of sh and base.
-constexpr int LOCAL_THREADS = 1024;
-// threads of k_local: all 32 warps for m <= 8; 16 for m > 8; 8 with two
-// columns per lane (CPL = 2), so that the elimination warp keeps its columns
-// (about 200 residues) in registers
-__host__ __device__ constexpr int local_threads(int MM, int CPL) {
-    return CPL > 1 ? LOCAL_THREADS / 4 : (MM > 8 ? LOCAL_THREADS / 2 : LOCAL_THREADS);
+// Orders per chunk unless the context sets it (wr_set_sigma_chunk): the window and
+// product launches are spread over more orders by a longer chunk, the local kernel's
+// row work per order grows with it.  Measured: q = 16, 11,252 orders 58 / 53 ms
+// for 32 / 64; q = 32, 2,254 orders 20.0 / 19.6 / 23.1 ms for 16 / 32 / 64; q = 64,
+// 4,098 orders (256-order leaves) 126 / 122 / 135 ms for 8 / 16 / 32.
+inline int sigma_chunk_default(int q) {
+    return q <= 16 ? 64 : (q <= 32 ? 32 : 16);
 }
-// orders per chunk unless the context sets it (wr_set_sigma_chunk); for
-// q > 32 (k_local_wide, whose row work per order grows with the chunk) 4:
-// measured at q = 64, L = 8,192, 512-order leaves: 1,678 / 1,518 / 1,299 /
-// 1,496 / 1,415 ms for chunks of 2 / 3 / 4 / 5 / 7 orders
-constexpr int SIGMA_CHUNK_DEFAULT = 64;
-constexpr int SIGMA_CHUNK_WIDE = 4;
-// PM-Basis by default only for sequences longer than SIGMA_PM_MIN_L (q <=
-// 32), with leaves of SIGMA_LEAF_DEFAULT orders; measured on GB300 at
-// L = 45,002, q = 16 the blocked M-Basis alone is faster (744 ms against
-// 786-1058 ms for leaves of 16,384 down to 1,024 orders).  For q > 32 the
-// M-Basis chunks are a few orders long (shared memory) and the window and
-// apply passes over the basis grow with its degree, so PM-Basis with short
-// leaves takes over early: at q = 64, L = 8,192, 1,648 / 1,453 / 1,413 ms for
-// leaves of 2,048 / 512 / 256 orders, and at L = 118,752 21.5 s with 512
-// (46 s with 2,048).  wr_set_sigma_leaf chooses the leaf explicitly.
+// PM-Basis by default only for sequences longer than SIGMA_PM_MIN_L (q <= 32),
+// with leaves of SIGMA_LEAF_DEFAULT orders: the M-Basis trails a sequence chunk by
+// chunk, PM-Basis in segments.  For q > 32 the window and product passes over the
+// basis cost more per order, so PM-Basis with short leaves takes over early: at q =
+// 64, 4,098 orders, 125 / 122 / 132 ms for leaves of 128 / 256 / 512 orders, and
+// against the M-Basis alone 16.8 / 15.8 ms at 600 orders, 27.8 / 29.3 at 1,000,
+// 42.3 / 49.5 at 1,500, 58.5 / 75.5 at 2,040.  wr_set_sigma_leaf chooses the leaf
+// explicitly.
 constexpr int64_t SIGMA_LEAF_DEFAULT = 8192;
 constexpr int64_t SIGMA_PM_MIN_L = 131072;
-constexpr int64_t SIGMA_LEAF_WIDE = 512;
-constexpr int64_t SIGMA_PM_MIN_L_WIDE = 2048;
-constexpr int BAR_T0 = 1, BAR_RR0 = 3;  // ids BAR_T0 + (i & 1), BAR_RR0 + (i & 1)
+constexpr int64_t SIGMA_LEAF_WIDE = 256;
+constexpr int64_t SIGMA_PM_MIN_L_WIDE = 1024;
+constexpr int BAR_T0 = 1, BAR_E = 3;  // named barriers BAR_T0 + (i & 1), BAR_E
 
 __device__ __forceinline__ void named_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
@@ -284,805 +273,633 @@ __device__ __forceinline__ void named_arrive(int id, int nthreads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
-// The transform of one order held in registers by each lane: for its
-// column(s) j, the diagonal dg[j], the coefficients F[t][j] and where the
-// pivot columns of the same row live.  apply() computes new[j] = dg[j] old[j]
-// + sum_t F[t][j] old[pc[t]] for one row whose column j sits at p[0] (and
-// column j + 32 at p[1] when CPL = 2, that is q > 32, one row per warp).
-template <int MM, int CPL, int KLAZY>
-struct RowTransform {
-    uint32_t f[CPL][MM], d[CPL];
-    int src[MM];  // CPL = 1: lane holding pc[t]; CPL = 2: pc[t] itself
-    int np;
+// ---- local M-Basis over the window: one cluster of thread blocks, bb orders.
+//
+// The device keeps the basis in fraction-free form, M_g = M diag(S): the
+// elimination of a discrepancy whose columns are scaled by nonzero constants
+// picks the same pivots and yields the same reduced columns up to column
+// scales, so M_g stays a column-scaled copy of the order-by-order basis.  S
+// (per column, product of the scales of all orders) is divided out of P once
+// at the end.
+//
+// An order's transform is new[j] = s_j old[j] + sum_t F[t][j] old[pc[t]], then the
+// pivot columns times x.  It multiplies every row of the window (orders i ..), of
+// Qtop and of the chunk's transform Ml, each row for itself, so the rows are dealt
+// to the blocks of the cluster: block `rank` of CS holds the rows a = rank (mod CS)
+// of the window's orders and of Qtop, and the rows x = rank (mod CS) of Ml's
+// coefficients.  What the next order needs from everybody is its discrepancy,
+// m x q residues: every block writes its rows of it into the shared memory of all
+// the others, and after one cluster barrier each block runs the (same) elimination
+// for itself.
+//
+// Roles in a block: the first warps (EW of them) eliminate, the others multiply
+// rows.  Per order i
+//   elim    Gauss-Jordan by rows on the m x q discrepancy, columns in (degree,
+//           index) order, 4 column slots x MR rows over the EW warps, q / 4
+//           residues a lane.  A column is frozen (written to FR) at its turn; if it
+//           is nonzero outside the pivot rows so far it becomes pivot k, its first
+//           such row r_k the pivot row, and every other row of the later columns
+//           becomes d_k row - A[row][pc] row_k (fraction-free).  Row r_t then holds
+//           the coefficients of the pivot columns, times prod_{t <= i < k} d_i, so
+//           with pre_t = d_0 .. d_{t-1}: s_j = pre_k(j), F[t][j] = -pre_t FR[j][r_t]
+//           (t < k(j), the pivots before j) -- no inverse, and no transform
+//           carried beside the matrix.
+//   rows    first the block's rows of orders i and i + 1 (the next discrepancy:
+//           pivot columns take order i's value, the others order i + 1's), written
+//           to all blocks; then, beside the next elimination, the other rows.
+// Hand-overs: a named barrier T_i (transform i published; elim arrives, the row
+// warps wait) and the cluster barrier of order i (all threads arrive; it completes
+// when every block's rows of discrepancy i + 1 are everywhere).  The transform, its
+// snapshot of the offsets and the discrepancy are double-buffered; what is
+// overwritten two orders later was read before the barrier in between.
+// Multiplying column c by x moves no data: window column c is read at row
+// ip - sh[c], and Ml column c holds its coefficient s at row base[c] + s.
+//
+// Bound by the chain of one order: m pivot steps of a shared store, a barrier of EW
+// warps, a load, a ballot, two shuffles and one two-product Montgomery
+// reduction.  Measured per order (GB300): q = 16 9.6 -> 2.4 us, q = 32 70 -> 4.7 us,
+// q = 64 68 -> 17 us (one block, one elimination warp that also carried the
+// transform, or sixteen warps with all rows of the chunk on one SM, before).
+constexpr int LC_SNAP = 228;   // words of an order's snapshot
+constexpr int LC_INTS = 1392;  // words of the bookkeeping arrays
+__host__ __device__ constexpr int lc_threads(int MR) { return MR == 32 ? 512 : (MR == 16 ? 384 : 256); }
+// elimination warps: one for MR = 8 (4 column slots, handed round by shuffles), else 8 column slots
+__host__ __device__ constexpr int lc_ew(int MR) { return MR == 8 ? 1 : MR / 4; }
 
-    __device__ __forceinline__ void load(const uint32_t *F, const uint32_t *dg, const int *pcs, int np_, int q,
-                                         int W2, int grp, int col, int lane) {
-        np = np_;
-#pragma unroll
-        for (int k = 0; k < CPL; k++) {
-            const int j = CPL == 1 ? col : lane + 32 * k;
-            d[k] = j < q ? dg[j] : 0u;
-#pragma unroll
-            for (int t = 0; t < MM; t++) f[k][t] = (t < np && j < q) ? F[t * q + j] : 0u;
-        }
-#pragma unroll
-        for (int t = 0; t < MM; t++) {
-            const int c = t < np ? pcs[t] : 0;
-            src[t] = CPL == 1 ? grp * W2 + c : c;
-        }
-    }
-
-    __device__ __forceinline__ void apply(uint32_t *const (&ptr)[CPL], const ModP &mp) const {
-        uint32_t v[CPL];
-        unsigned long long a[CPL];
-#pragma unroll
-        for (int k = 0; k < CPL; k++) {
-            v[k] = ptr[k] ? *ptr[k] : 0u;
-            a[k] = (unsigned long long)d[k] * v[k];
-        }
-#pragma unroll
-        for (int t = 0; t < MM; t++) {
-            if (t < np) {
-                uint32_t oc;
-                if (CPL == 1) {
-                    oc = __shfl_sync(0xffffffffu, v[0], src[t]);
-                } else {
-                    const uint32_t x0 = __shfl_sync(0xffffffffu, v[0], src[t] & 31);
-                    const uint32_t x1 = __shfl_sync(0xffffffffu, v[CPL - 1], src[t] & 31);
-                    oc = src[t] >= 32 ? x1 : x0;
-                }
-#pragma unroll
-                for (int k = 0; k < CPL; k++) a[k] += (unsigned long long)f[k][t] * oc;
-                // at most KLAZY products (plus a reduced residue) between reductions
-                if (MM + 1 > KLAZY && (t + 2) % KLAZY == 0) {
-#pragma unroll
-                    for (int k = 0; k < CPL; k++) a[k] = red64(a[k], mp);
-                }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < CPL; k++)
-            if (ptr[k]) *ptr[k] = red64(a[k], mp);
-    }
-};
-
-// Warp 0 of k_local when q <= 16: two lanes per column.  Lane L holds
-// column j = L & 15 and half h = L >> 4 of it: discrepancy rows
-// h*MM/2 .. h*MM/2 + MM/2 - 1 and the same range of its transform row, so a
-// pivot step costs each lane half the Montgomery updates of the one-lane
-// layout.  The elimination, the published transform and the bookkeeping are
-// those of the one-lane path (same pivots, same fraction-free values).
-template <int MM>
-__device__ __forceinline__ void local_warp0_two_lane(int m, int q, int bb, const uint32_t *Es, uint32_t *Tb, int tw,
-                                                     int *snap, int snapw, int *deg, int *degl, int *sh, int *base,
-                                                     uint32_t *scale_g, int nth, const ModP &mp) {
-    constexpr int HM = MM / 2;
-    const int lane = threadIdx.x & 31;
-    const int j = lane & 15, h = lane >> 4;
-    const bool v = j < q;
-    const int mq = m * q;
-    uint32_t scum = mp.r1;  // cumulative column scale over the chunk (Montgomery form)
-    for (int i = 0; i < bb; i++) {
-        uint32_t *F = Tb + (i & 1) * tw;
-        uint32_t *dg = F + mq;
-        int *sn = snap + (i & 1) * snapw;
-        int *s_sh = sn, *s_base = sn + q, *s_isp = sn + 2 * q, *s_pc = sn + 3 * q;
-        uint32_t d[HM], tp[HM], sc = mp.r1;
-        int rk = 1 << 20;
-        if (v) {
-            int r0 = 0;
-            const int dj = deg[j];
-            for (int c2 = 0; c2 < q; c2++) {
-                const int dc2 = deg[c2];
-                r0 += (dc2 < dj || (dc2 == dj && c2 < j)) ? 1 : 0;
-            }
-            rk = r0;
-            if (h == 0) {
-                s_isp[j] = 0;
-                s_sh[j] = sh[j];
-                s_base[j] = base[j];
-            }
-        }
-        {
-            const uint32_t *er = Es + (size_t)(i - (v ? sh[j] : 0)) * mq + (v ? j : 0);
-#pragma unroll
-            for (int r = 0; r < HM; r++) {
-                const int a2 = h * HM + r;
-                d[r] = (v && a2 < m) ? to_mont(er[a2 * q], mp) : 0u;
-                tp[r] = 0u;
-            }
-        }
-        int np = 0;
-        for (int step = 0; step < q; step++) {
-            const bool mine = rk == step;
-            const unsigned who = __ballot_sync(0xffffffffu, mine);
-            const int src0 = __ffs(who) - 1;  // the h = 0 lane of the current column
-            int frl = -1;
-            if (mine) {
-#pragma unroll
-                for (int r = HM - 1; r >= 0; r--)
-                    if (d[r] != 0) frl = h * HM + r;
-            }
-            const int fr0 = __shfl_sync(0xffffffffu, frl, src0);
-            const int fr1 = __shfl_sync(0xffffffffu, frl, src0 + 16);
-            const int fr = fr0 >= 0 ? fr0 : fr1;
-            if (fr < 0) continue;
-            const int hp = fr / HM, rp = fr - hp * HM;
-            const uint32_t sc_cur = __shfl_sync(0xffffffffu, sc, src0);
-            uint32_t pv[HM], pt[HM];
-#pragma unroll
-            for (int r = 0; r < HM; r++) {
-                pv[r] = __shfl_sync(0xffffffffu, d[r], src0 + 16 * h);
-                pt[r] = __shfl_sync(0xffffffffu, tp[r], src0 + 16 * h);
-            }
-            uint32_t x = 0;  // this lane's residue at pivot row offset rp
-#pragma unroll
-            for (int r = 0; r < HM; r++)
-                if (r == rp) x = d[r];
-            const uint32_t dc = __shfl_sync(0xffffffffu, x, src0 + 16 * hp);
-            const uint32_t dj = __shfl_sync(0xffffffffu, x, j + 16 * hp);
-            if (rk > step && rk < (1 << 20) && dj != 0) {
-                // col <- dc col - dj pivot: one Montgomery reduction of
-                // dc*x + (p - dj)*y < 2 p^2 < p 2^32 per entry
-                const uint64_t ndj = mp.p - dj;
-#pragma unroll
-                for (int r = 0; r < HM; r++) d[r] = mont_redc((uint64_t)dc * d[r] + ndj * pv[r], mp);
-#pragma unroll
-                for (int r = 0; r < HM; r++) {
-                    const int t = h * HM + r;
-                    if (t < np) tp[r] = mont_redc((uint64_t)dc * tp[r] + ndj * pt[r], mp);
-                    else if (t == np) tp[r] = mont_redc(ndj * sc_cur, mp);
-                }
-                sc = mont_mul(sc, dc, mp);
-            }
-            if (lane == 0) {
-                s_pc[np] = src0;
-                s_isp[src0] = 1;
-            }
-            np++;
-        }
-        __syncwarp();
-        // publish the transform (normal form) and the local degree bounds
-        int dl = 0;
-        if (v) {
-            dl = degl[j];
-#pragma unroll
-            for (int r = 0; r < HM; r++) {
-                const int t = h * HM + r;
-                if (t < np) {
-                    const uint32_t val = from_mont(tp[r], mp);
-                    F[t * q + j] = val;
-                    if (val) dl = max(dl, degl[s_pc[t]]);
-                }
-            }
-            if (h == 0) dg[j] = from_mont(sc, mp);
-            scum = mont_mul(scum, sc, mp);
-        }
-        dl = max(dl, __shfl_xor_sync(0xffffffffu, dl, 16));  // both halves of the column
-        int dmx = dl;
-#pragma unroll
-        for (int off = 8; off > 0; off >>= 1) dmx = max(dmx, __shfl_xor_sync(0xffffffffu, dmx, off));
-        if (lane == 0) {
-            sn[3 * q + m] = np;
-            sn[3 * q + m + 1] = dmx;
-        }
-        __syncwarp();
-        named_arrive(BAR_T0 + (i & 1), nth);
-        // ---- bookkeeping of order i: local degrees, pivots times x
-        if (v && h == 0) degl[j] = dl;
-        __syncwarp();
-        for (int t = lane; t < np; t += 32) {
-            const int c = s_pc[t];
-            deg[c] += 1;
-            degl[c] += 1;
-            sh[c] += 1;
-            base[c] -= 1;
-        }
-        __syncwarp();
-        // ---- the next discrepancy (rows i, i+1) must be done
-        named_sync(BAR_RR0 + (i & 1), nth);
-    }
-    if (v && h == 0) scale_g[j] = mont_mul(scale_g[j], scum, mp);
+// Blocks per cluster for q columns (8 is the largest portable size): q = 16 84 / 82
+// ms for 4 / 8, q = 32 49 / 43, q = 64 413 / 400 (the whole sigma-basis with the
+// earlier window and product kernels); up to 8 columns 4 and 8 measure the same
+inline int local_cluster(int q) {
+    return q > 8 ? 8 : 4;
 }
 
-template <int MM, int CPL, int KLAZY>
-__global__ void __launch_bounds__(local_threads(MM, CPL))
-    k_local(int m, int n, int q, int bb, int nparts, const uint32_t *__restrict__ Epart,
-            uint32_t *__restrict__ qtop_g, int32_t *__restrict__ deg_g, uint32_t *__restrict__ Ml_g,
-            int32_t *__restrict__ degl_g, int *__restrict__ dmax_g, uint32_t *__restrict__ scale_g, int dbase,
-            ModP mp) {
-    extern __shared__ uint32_t sm[];
-    const int mq = m * q, qq = q * q;
-    const int mlrows = 2 * bb + 1;
-    const int tw = mq + q;                               // transform: F (m x q) then diagonal (q)
-    uint32_t *Es = sm;                                   // bb*m*q
-    uint32_t *Ml = Es + (size_t)bb * mq;                 // (2bb+1)*q*q
-    uint32_t *Tb = Ml + (size_t)mlrows * qq;             // 2 * tw (double buffer)
-    uint32_t *qt = Tb + 2 * tw;                          // m*q
-    int *deg = (int *)(qt + mq);                         // q
-    int *degl = deg + q;                                 // q
-    int *sh = degl + q;                                  // q
-    int *base = sh + q;                                  // q
-    int *snap = base + q;                                // 2 * snapw: sh, base, isp, pc, np, dl
-    const int snapw = 3 * q + m + 2;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const int lane = tid & 31, warp = tid >> 5, nwarps = nth >> 5;
-    const int E = bb * mq;
-    (void)n;
+struct LcLayout {  // word offsets of the dynamic shared memory (ints and residues are both words)
+    int ma, mx;    // most rows of a window order / of an Ml coefficient in a block
+    int Es, Ml, qt, disc, F, dg, FR, ints, total;
+};
+__host__ __device__ inline LcLayout lc_layout(int m, int q, int b, int CS, int MR) {
+    LcLayout l;
+    l.ma = (m + CS - 1) / CS;
+    l.mx = (q + CS - 1) / CS;
+    int o = 0;
+    l.Es = o; o += b * l.ma * q;
+    l.Ml = o; o += (2 * b + 1) * l.mx * q;
+    l.qt = o; o += l.ma * q;
+    l.disc = o; o += 2 * m * q;
+    l.F = o; o += 2 * m * q;
+    l.dg = o; o += 2 * 64;
+    l.FR = o; o += q * (MR + 1);
+    l.ints = o; o += LC_INTS;
+    l.total = o;
+    return l;
+}
 
-    for (int x = tid; x < mq; x += nth) qt[x] = qtop_g[x];
-    __syncthreads();
-    for (int x = tid; x < E; x += nth) {
-        unsigned long long v = 0;
-        int b = 0;
-        for (; b + 4 <= nparts; b += 4)
-            v += (unsigned long long)Epart[(size_t)b * E + x] + Epart[(size_t)(b + 1) * E + x] +
-                 Epart[(size_t)(b + 2) * E + x] + Epart[(size_t)(b + 3) * E + x];
-        for (; b < nparts; b++) v += Epart[(size_t)b * E + x];
-        uint32_t e = red64(v, mp);
-        if (x < mq) e = subm(e, qt[x], mp);
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// store to the same shared-memory address of block `rank` of the cluster
+__device__ __forceinline__ void st_cluster(uint32_t *p, uint32_t rank, uint32_t v) {
+    uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p)), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(r), "r"(v) : "memory");
+}
+
+// A row times the order's transform in registers (lane: column j and, CPL = 2,
+// column j + 32; f[k][t] = F[t][column k], d[k] its diagonal): x[k] the row's
+// residues of the lane's columns, g the row's residue at pivot column t = the
+// lane's index in its group of W2 lanes.  Two accumulators a column (even and odd
+// t), each folded after FOLDK of its own products.
+template <int TM, int CPL, int FOLDK>
+__device__ __forceinline__ void row_times(const uint32_t (&f)[CPL][TM], const uint32_t (&d)[CPL], int np, int W2,
+                                          const uint32_t (&x)[CPL], uint32_t g, uint32_t (&out)[CPL], uint32_t fc,
+                                          const ModP &mp) {
+    unsigned long long a0[CPL], a1[CPL];
+#pragma unroll
+    for (int k = 0; k < CPL; k++) {
+        a0[k] = (unsigned long long)d[k] * x[k];
+        a1[k] = 0ull;
+    }
+    // (f[k][t] = 0 from t = np on: whole groups of 8 without branches)
+#pragma unroll
+    for (int t0 = 0; t0 < TM; t0 += 8) {
+        if (TM == 8 || t0 < np) {
+            uint32_t v[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) v[u] = __shfl_sync(0xffffffffu, g, t0 + u, W2);
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                const int t = t0 + u;
+#pragma unroll
+                for (int k = 0; k < CPL; k++) {
+                    if ((t & 1) == 0) {
+                        a0[k] = madw(f[k][t], v[u], a0[k]);
+                        if ((t / 2 + 2) % FOLDK == 0) a0[k] = fold1(a0[k], fc);
+                    } else {
+                        a1[k] = madw(f[k][t], v[u], a1[k]);
+                        if (((t + 1) / 2) % FOLDK == 0) a1[k] = fold1(a1[k], fc);
+                    }
+                }
+            }
+        }
+    }
+    // folded, each is below p 2^32 + 2^32 <= 2^63: their sum fits
+#pragma unroll
+    for (int k = 0; k < CPL; k++) out[k] = red64(fold1(a0[k], fc) + fold1(a1[k], fc), mp);
+}
+
+// The update of a pivot step on the lane's residues from k0 on: A[k] <- d A[k] -
+// v y with y the pivot row's residue of the same column (nv = p - v; the pivot
+// row itself stays).  One block without branches: independent chains.
+template <int KR>
+__device__ __forceinline__ void pivot_step(uint32_t (&A)[KR], const uint32_t (&y)[KR], int k0, uint32_t d, uint32_t nv,
+                                           bool other, uint32_t p, uint32_t pneg) {
+#pragma unroll
+    for (int k = 0; k < KR; k++) {
+        if (k < k0) continue;  // (a constant after unrolling)
+        // d x + (p - v) y < 2 p^2 < p 2^32
+        const unsigned long long t = madw(nv, y[k], (unsigned long long)d * A[k]);
+        const uint32_t u = (uint32_t)(madw((uint32_t)t * pneg, p, t) >> 32);
+        A[k] = other ? min(u, u - p) : A[k];
+    }
+}
+
+template <int MR, int CPL, int QC, int FOLDK>
+__global__ void __launch_bounds__(lc_threads(MR), 1)
+    k_local(int m, int q, int bb, const uint32_t *__restrict__ E, uint32_t *__restrict__ qtop_g,
+            int32_t *__restrict__ deg_g, uint32_t *__restrict__ Ml_g, int32_t *__restrict__ degl_g,
+            int *__restrict__ dmax_g, uint32_t *__restrict__ scale_g, int dbase, ModP mp) {
+    constexpr int NT = lc_threads(MR), EW = lc_ew(MR), NE = 32 * EW, NWK = NT / 32 - EW;
+    constexpr int CL = EW * 32 / MR;        // column slots of the elimination
+    constexpr int KR = QC / CL;             // residues a lane of the elimination (q <= QC)
+    constexpr int TM = MR;                  // most pivots of an order
+    constexpr unsigned FULL = 0xffffffffu;
+    extern __shared__ uint32_t sm[];
+    const int CS = (int)cluster_size(), rank = (int)cluster_rank();
+    const LcLayout l = lc_layout(m, q, bb, CS, MR);
+    uint32_t *Es = sm + l.Es;      // [bb][ma][q]
+    uint32_t *Ml = sm + l.Ml;      // [2 bb + 1][mx][q]
+    uint32_t *qt = sm + l.qt;      // [ma][q]
+    uint32_t *disc = sm + l.disc;  // [2][m][q], written by every block
+    uint32_t *Fs = sm + l.F;       // [2][m][q]
+    uint32_t *dgs = sm + l.dg;     // [2][64]
+    uint32_t *FR = sm + l.FR;      // [q][MR + 1] frozen columns by position
+    int *deg = (int *)(sm + l.ints);  // [64] degrees, local degrees (before and after the transform), offsets
+    int *degl = deg + 64, *dln = degl + 64, *sh = dln + 64, *base = sh + 64;
+    int *posc = base + 64;         // [64] column of each position
+    int *rk = posc + 64;           // [64] position of each column
+    int *kj = rk + 64;             // [64] pivots before the position's turn
+    uint32_t *scum = (uint32_t *)(kj + 64);  // [64] column scales of the chunk (Montgomery form)
+    uint32_t *preN = scum + 64;    // [33] pre_t in normal form
+    uint32_t *preM = preN + 36;    // [33] pre_t in Montgomery form
+    int *pr = (int *)(preM + 36);  // [32] pivot rows
+    int *snap = pr + 32;           // [2][LC_SNAP]: sh, base, isp [64 each], pc [32], np, D
+    int *dmx = snap + 2 * LC_SNAP; // [8]
+    int *pdl = dmx + 8;            // [32] the pivots' local degrees before the order
+    int *ppos = pdl + 32;          // [32] the pivots' positions
+    int *pmax = ppos + 32;         // [33]
+    int *degl_n = pmax + 36;       // [64]
+    uint32_t *sck = (uint32_t *)(degl_n + 64);  // [64] the order's column scales (Montgomery form)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int mq = m * q;
+    const uint32_t fc = mp.r1;  // 2^32 mod p
+    const int ma = (m - rank + CS - 1) / CS, mx = (q - rank + CS - 1) / CS;  // rows of this block (may be 0)
+
+    for (int x = tid; x < bb * l.ma * q; x += NT) {
+        const int c = x % q, al = x / q % l.ma, i = x / (q * l.ma), a = rank + CS * al;
+        uint32_t e = 0;
+        if (a < m) {
+            e = E[((size_t)i * m + a) * q + c];
+            if (i == 0) e = subm(e, qtop_g[a * q + c], mp);
+        }
         Es[x] = e;
     }
-    for (int x = tid; x < mlrows * qq; x += nth) {
-        const int s2 = x / qq, rem = x - s2 * qq;
-        Ml[x] = (s2 == bb && rem / q == rem % q) ? 1u : 0u;  // logical coefficient 0 at row base = bb
+    for (int x = tid; x < mq; x += NT) disc[x] = subm(E[x], qtop_g[x], mp);
+    for (int x = tid; x < l.ma * q; x += NT) {
+        const int a = rank + CS * (x / q);
+        qt[x] = a < m ? qtop_g[a * q + x % q] : 0u;
     }
-    for (int c = tid; c < q; c += nth) {
-        deg[c] = deg_g[c];
+    for (int x = tid; x < (2 * bb + 1) * l.mx * q; x += NT) {
+        const int c = x % q, xl = x / q % l.mx, s = x / (q * l.mx);
+        Ml[x] = (s == bb && rank + CS * xl == c) ? 1u : 0u;  // coefficient 0 at row base = bb
+    }
+    for (int c = tid; c < 64; c += NT) {
+        snap[c] = 0;
+        snap[64 + c] = bb;
+        deg[c] = c < q ? deg_g[c] : 0;
         degl[c] = 0;
         sh[c] = 0;
         base[c] = bb;
+        scum[c] = mp.r1;
     }
     __syncthreads();
-    int W2 = 1;
-    while (W2 < q && W2 < 32) W2 <<= 1;
-    const int rpw = 32 / W2;
-    const int grp = lane / W2, col = lane % W2;
+    cluster_arrive();  // (every block has read qtop_g and set up before anybody writes)
+    cluster_wait();
 
-    if (warp == 0 && CPL == 1 && q <= 16) {
-        local_warp0_two_lane<MM>(m, q, bb, Es, Tb, tw, snap, snapw, deg, degl, sh, base, scale_g, nth, mp);
-    } else if (warp == 0) {
-        uint32_t scum[CPL];  // cumulative column scales over the chunk (Montgomery form)
-#pragma unroll
-        for (int k = 0; k < CPL; k++) scum[k] = mp.r1;
-        for (int i = 0; i < bb; i++) {
-            uint32_t *F = Tb + (i & 1) * tw;
-            uint32_t *dg = F + mq;
-            int *sn = snap + (i & 1) * snapw;
-            int *s_sh = sn, *s_base = sn + q, *s_isp = sn + 2 * q, *s_pc = sn + 3 * q;
-            // ---- elimination of order i
-            uint32_t d[CPL][MM], tp[CPL][MM], sc[CPL];
-            int rk[CPL];
-#pragma unroll
-            for (int k = 0; k < CPL; k++) {
-                const int j = lane + 32 * k;
-                const bool v = j < q;
-                sc[k] = mp.r1;
-                rk[k] = 1 << 20;
-                if (v) {
-                    int r0 = 0;
-                    for (int c2 = 0; c2 < q; c2++)
-                        r0 += (deg[c2] < deg[j] || (deg[c2] == deg[j] && c2 < j)) ? 1 : 0;
-                    rk[k] = r0;
-                    s_isp[j] = 0;
-                    s_sh[j] = sh[j];
-                    s_base[j] = base[j];
+    if (warp < EW) {
+        const int a = lane % MR, slot = warp * (32 / MR) + lane / MR;
+        auto esync = [&]() {
+            if constexpr (EW == 1) __syncwarp();
+            else named_sync(BAR_E, NE);
+        };
+        int D = 0;  // largest local degree
+        int QP = 1;
+        while (QP < q) QP <<= 1;
+        const int parts = QP < NE ? NE / QP : 1, part = tid % parts;  // threads a column
+        // positions by (degree, index)
+        auto ranks = [&]() {
+            for (int c0 = 0; c0 < q; c0 += NE / parts) {
+                const int c = c0 + tid / parts, dc = deg[c & 63];
+                int r = 0;
+#pragma unroll 4
+                for (int c2 = part; c2 < q; c2 += parts) {
+                    const int d2 = deg[c2];
+                    r += (d2 < dc || (d2 == dc && c2 < c)) ? 1 : 0;
                 }
-                const uint32_t *er = Es + (size_t)(i - (v ? sh[j] : 0)) * mq + (v ? j : 0);
-#pragma unroll
-                for (int a2 = 0; a2 < MM; a2++) {
-                    d[k][a2] = (v && a2 < m) ? to_mont(er[a2 * q], mp) : 0u;
-                    tp[k][a2] = 0u;
+                for (int off = 1; off < parts; off <<= 1) r += __shfl_xor_sync(FULL, r, off);
+                if (c < q && part == 0) {
+                    rk[c] = r;
+                    posc[r] = c;
                 }
             }
-            int np = 0;
-            for (int step = 0; step < q; step++) {
-                int mine = -1;
+        };
+        ranks();
+        esync();
+        const int nk = (q + CL - 1) / CL, am = a < m ? a : 0;
+        // The order's elimination with pivots wherever they are: columns that are zero
+        // outside the pivot rows, pivot rows in any order.  Writes what the straight
+        // path below writes, through FR; returns the number of pivots.
+        auto slow = [&](int i) -> int {
+            const uint32_t *dc = disc + (i & 1) * mq;
+            uint32_t *F = Fs + (i & 1) * mq, *dg = dgs + (i & 1) * 64;
+            int *sn = snap + (i & 1) * LC_SNAP;
+            uint32_t A[KR], y[KR];
 #pragma unroll
-                for (int k = 0; k < CPL; k++)
-                    if (rk[k] == step) mine = k;
-                const unsigned who = __ballot_sync(0xffffffffu, mine >= 0);
-                const int src = __ffs(who) - 1;
-                int fr = -1;
-                uint32_t sc_cur = 0;
-                if (mine >= 0) {
+            for (int k = 0; k < KR; k++) {
+                const int pos = CL * k + slot;
+                A[k] = to_mont(dc[am * q + posc[min(pos, q - 1)]], mp);
+                if (pos >= q || a >= m) A[k] = 0u;
+            }
+            for (int c = tid; c < 64; c += NE) {
+                sn[128 + c] = 0;
+                dln[c] = degl[c];
+            }
+            esync();
+            uint32_t pre = mp.r1, rmask = m == 32 ? FULL : (1u << m) - 1u;  // rows without a pivot
+            int np = 0, pos = 0;
+            for (int g4 = 0; g4 < nk; g4++) {
+                for (int s = 0; s < CL && pos < q && np < m; s++, pos++) {
+                    // the pivot row is nearly always the first row without a pivot: its
+                    // residues are fetched before the column is known to have it
+                    int fr = __ffs(rmask) - 1;
 #pragma unroll
-                    for (int k = 0; k < CPL; k++)
-                        if (k == mine) {
-                            sc_cur = sc[k];
+                    for (int k = 0; k < KR; k++) y[k] = __shfl_sync(FULL, A[k], fr, MR);
+                    if (slot == s) FR[pos * (MR + 1) + a] = A[0];
+                    uint32_t v, d;
+                    if constexpr (EW == 1) {
+                        v = __shfl_sync(FULL, A[0], s * MR + a);
+                        d = __shfl_sync(FULL, A[0], s * MR + fr);
+                    } else {
+                        esync();
+                        v = FR[pos * (MR + 1) + a];
+                        d = FR[pos * (MR + 1) + fr];
+                    }
+                    if (tid == 0) kj[pos] = np;
+                    if (d == 0u) {  // another row, or a column that is zero there
+                        const uint32_t nz = __ballot_sync(FULL, v != 0u) & rmask;
+                        if (nz == 0u) continue;
+                        fr = __ffs(nz) - 1;
+                        d = __shfl_sync(FULL, v, fr);
 #pragma unroll
-                            for (int a2 = MM - 1; a2 >= 0; a2--)
-                                if (d[k][a2] != 0) fr = a2;
+                        for (int k = 0; k < KR; k++) y[k] = __shfl_sync(FULL, A[k], fr, MR);
+                    }
+                    if (tid == 0) {
+                        pr[np] = fr;
+                        ppos[np] = pos;
+                        preM[np] = pre;
+                    }
+                    const uint32_t nv = v != 0u ? mp.p - v : 0u;
+                    pivot_step(A, y, 0, d, nv, a != fr, mp.p, mp.pneg);
+                    pre = mont_mul(pre, d, mp);
+                    rmask &= ~(1u << fr);
+                    np++;
+                }
+                if (np == m || pos >= q) {
+                    // the columns not yet frozen, at their final values
+#pragma unroll
+                    for (int k = 0; k < KR; k++) {
+                        const int pk = CL * (g4 + k) + slot;
+                        if (pk >= pos && pk < q) {
+                            FR[pk * (MR + 1) + a] = A[k];
+                            if (a == 0) kj[pk] = np;
                         }
+                    }
+                    break;
                 }
-                fr = __shfl_sync(0xffffffffu, fr, src);
-                if (fr < 0) continue;
-                const int jcur = __shfl_sync(0xffffffffu, lane + 32 * (mine >= 0 ? mine : 0), src);
-                sc_cur = __shfl_sync(0xffffffffu, sc_cur, src);
-                uint32_t pv[MM], pt[MM];
 #pragma unroll
-                for (int a2 = 0; a2 < MM; a2++) {
-                    uint32_t x0 = 0, x1 = 0;
-#pragma unroll
-                    for (int k = 0; k < CPL; k++)
-                        if (k == mine) { x0 = d[k][a2]; x1 = tp[k][a2]; }
-                    pv[a2] = __shfl_sync(0xffffffffu, x0, src);
-                    pt[a2] = __shfl_sync(0xffffffffu, x1, src);
+                for (int k = 0; k + 1 < KR; k++) A[k] = A[k + 1];
+            }
+            if (tid == 0) {
+                preM[np] = pre;
+                sn[224] = np;
+                sn[225] = D;
+            }
+            esync();
+            // the pivots' columns, local degrees and scales
+            for (int t = tid; t <= np; t += NE) {
+                preN[t] = from_mont(preM[t], mp);
+                if (t < np) {
+                    const int c = posc[ppos[t]];
+                    sn[192 + t] = c;
+                    pdl[t] = degl[c];
+                    sn[128 + c] = 1;
                 }
-                uint32_t dc = 0;
+            }
+            esync();
+            // publish the transform (normal form) and the local degree bounds
+            for (int c0 = 0; c0 < q; c0 += NE / parts) {
+                const int j = c0 + tid / parts;
+                if (j < q) {
+                    const int pj = rk[j], kk = kj[pj];
+                    const uint32_t *fj = FR + pj * (MR + 1);
+                    int dl = 0;
+#pragma unroll 4
+                    for (int t = part; t < np; t += parts) {
+                        const uint32_t x = mont_mul(fj[pr[t]], preN[t], mp);
+                        const uint32_t v = t < kk ? x : 0u;
+                        F[t * q + j] = v != 0u ? mp.p - v : 0u;
+                        dl = max(dl, v != 0u ? pdl[t] : 0);
+                    }
+                    if (dl > 0) atomicMax(&dln[j], dl);
+                    if (part == 0) {
+                        dg[j] = preN[kk];
+                        sck[j] = preM[kk];
+                    }
+                }
+            }
+            return np;
+        };
+        for (int i = 0; i < bb; i++) {
+            const uint32_t *dc = disc + (i & 1) * mq;
+            uint32_t *F = Fs + (i & 1) * mq, *dg = dgs + (i & 1) * 64;
+            int *sn = snap + (i & 1) * LC_SNAP;
+            uint32_t A[KR], y[KR];
+            int col[KR];  // the lane's columns
 #pragma unroll
-                for (int a2 = 0; a2 < MM; a2++)
-                    if (a2 == fr) dc = pv[a2];
-                // col <- dc col - dj pivot: one Montgomery reduction of
-                // dc*x + (p - dj)*y < 2 p^2 < p 2^32 per entry
+            for (int k = 0; k < KR; k++) {
+                col[k] = posc[min(CL * k + slot, q - 1)];
+                A[k] = to_mont(dc[am * q + col[k]], mp);
+                if (CL * k + slot >= q || a >= m) A[k] = 0u;
+            }
+            int np = m;
+            // Straight through: position t becomes pivot t with row t its pivot row, as it
+            // does unless residues vanish.  Registers keep a column's values from its turn
+            // on, so a lane holds row a of every column it has: F and the scales come from
+            // registers, with pre_a kept as the lane's own.
+            uint32_t pre = mp.r1, pre_a = mp.r1;
+            bool bad = m > q;
 #pragma unroll
-                for (int k = 0; k < CPL; k++) {
-                    if (rk[k] > step && rk[k] < (1 << 20)) {
-                        uint32_t dj = 0;
+            for (int g = 0; g < MR / CL; g++) {
 #pragma unroll
-                        for (int a2 = 0; a2 < MM; a2++)
-                            if (a2 == fr) dj = d[k][a2];
-                        if (dj != 0) {
-                            const uint64_t ndj = mp.p - dj;
+                for (int s = 0; s < CL; s++) {
+                    const int t = CL * g + s;
+                    if (t < m) {  // (the same for all)
+                        uint32_t v, d;
 #pragma unroll
-                            for (int a2 = 0; a2 < MM; a2++)
-                                d[k][a2] = mont_redc((uint64_t)dc * d[k][a2] + ndj * pv[a2], mp);
+                        for (int k = g; k < KR; k++) y[k] = __shfl_sync(FULL, A[k], t, MR);
+                        if constexpr (EW == 1) {
+                            v = __shfl_sync(FULL, A[g], s * MR + a);
+                            d = __shfl_sync(FULL, A[g], s * MR + t);
+                        } else {
+                            uint32_t *fr = FR + (t & 1) * MR;  // (two slots: a barrier apart)
+                            if (slot == s) fr[a] = A[g];
+                            esync();
+                            v = fr[a];
+                            d = fr[t];
+                        }
+                        bad |= d == 0u;
+                        const uint32_t nv = v != 0u ? mp.p - v : 0u;
+                        const uint32_t keep = A[g];
+                        pivot_step(A, y, g, d, nv, a != t, mp.p, mp.pneg);
+                        if (slot <= s) A[g] = keep;
+                        pre_a = a == t ? pre : pre_a;
+                        pre = mont_mul(pre, d, mp);
+                    }
+                }
+            }
+            if (!bad) {
+                const uint32_t pa = from_mont(pre_a, mp), pm = from_mont(pre, mp);
 #pragma unroll
-                            for (int t = 0; t < MM; t++) {
-                                if (t < np) tp[k][t] = mont_redc((uint64_t)dc * tp[k][t] + ndj * pt[t], mp);
-                                else if (t == np) tp[k][t] = mont_redc(ndj * sc_cur, mp);
-                            }
-                            sc[k] = mont_mul(sc[k], dc, mp);
+                for (int k = 0; k < KR; k++) {
+                    const int pos = CL * k + slot, kk = min(pos, m);
+                    if (pos < q && a < m) {
+                        const uint32_t v = mont_mul(A[k], pa, mp);
+                        F[a * q + col[k]] = a < kk && v != 0u ? mp.p - v : 0u;
+                        if (a == (pos < m ? pos : 0)) {
+                            dg[col[k]] = pos < m ? pa : pm;
+                            sck[col[k]] = pos < m ? pre_a : pre;
                         }
                     }
                 }
-                if (lane == 0) {
-                    s_pc[np] = jcur;
-                    s_isp[jcur] = 1;
+                for (int c = tid; c < q; c += NE) sn[128 + c] = rk[c] < m ? 1 : 0;
+                if (tid < m) sn[192 + tid] = posc[tid];
+                if (tid == 0) {
+                    sn[224] = m;
+                    sn[225] = D;
                 }
-                np++;
+            } else {
+                np = slow(i);
             }
-            __syncwarp();
-            // publish the transform (normal form) and the local degree bounds
-            int dln[CPL];
+            if constexpr (EW == 1) __syncwarp();
+            named_arrive(BAR_T0 + (i & 1), NE + 32 * NWK);
+            // bookkeeping, beside the rows
+            if (!bad && warp == 0) {  // pmax[k]: largest local degree of the first k pivots
+                int v = lane < m ? degl[posc[lane]] : 0;
 #pragma unroll
-            for (int k = 0; k < CPL; k++) {
-                const int j = lane + 32 * k;
-                dln[k] = 0;
-                if (j < q) {
-                    int dl = degl[j];
-#pragma unroll
-                    for (int t = 0; t < MM; t++)
-                        if (t < np) {
-                            const uint32_t v = from_mont(tp[k][t], mp);
-                            F[t * q + j] = v;
-                            if (v) dl = max(dl, degl[s_pc[t]]);
-                        }
-                    dg[j] = from_mont(sc[k], mp);
-                    scum[k] = mont_mul(scum[k], sc[k], mp);
-                    dln[k] = dl;
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int u = __shfl_up_sync(FULL, v, off);
+                    if (lane >= off) v = max(v, u);
                 }
+                pmax[lane + 1] = v;
+                if (lane == 0) pmax[0] = 0;
             }
-            int dmx = 0;
-#pragma unroll
-            for (int k = 0; k < CPL; k++) dmx = max(dmx, dln[k]);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) dmx = max(dmx, __shfl_xor_sync(0xffffffffu, dmx, off));
-            if (lane == 0) {
-                sn[3 * q + m] = np;
-                sn[3 * q + m + 1] = dmx;
+            esync();
+            int *sx = snap + ((i + 1) & 1) * LC_SNAP;  // the next order's snapshot
+            int Dn = 0;
+            for (int c = tid; c < q; c += NE) {
+                const int ip = sn[128 + c];
+                // local degrees after the transform: exact from the slow path, else the
+                // largest of the column's and of the pivots before it (pmax)
+                const int pos = rk[c], dl = (bad ? dln[c] : max(degl[c], pmax[min(pos, m)])) + ip;
+                deg[c] += ip;
+                degl_n[c] = dl;
+                sx[c] = sh[c] += ip;
+                sx[64 + c] = base[c] -= ip;
+                scum[c] = mont_mul(scum[c], sck[c], mp);
+                Dn = max(Dn, dl);
             }
-            __syncwarp();
-            named_arrive(BAR_T0 + (i & 1), nth);
-            // ---- bookkeeping of order i: local degrees, pivots times x
+            Dn = __reduce_max_sync(FULL, Dn);
+            if (lane == 0) dmx[warp] = Dn;
+            esync();
 #pragma unroll
-            for (int k = 0; k < CPL; k++)
-                if (lane + 32 * k < q) degl[lane + 32 * k] = dln[k];
-            __syncwarp();
-            for (int t = lane; t < np; t += 32) {
-                const int c = s_pc[t];
-                deg[c] += 1;
-                degl[c] += 1;
-                sh[c] += 1;
-                base[c] -= 1;
-            }
-            __syncwarp();
-            // ---- the next discrepancy (rows i, i+1) must be done
-            named_sync(BAR_RR0 + (i & 1), nth);
-        }
-        // cumulative scales of this chunk into the running product
-#pragma unroll
-        for (int k = 0; k < CPL; k++) {
-            const int j = lane + 32 * k;
-            if (j < q) scale_g[j] = mont_mul(scale_g[j], scum[k], mp);
+            for (int w = 0; w < EW; w++) D = max(D, dmx[w]);
+            for (int c = tid; c < q; c += NE) degl[c] = degl_n[c];
+            ranks();
+            esync();
+            cluster_arrive();
+            cluster_wait();
         }
     } else {
-        // warps on warp 0's SM sub-partition (w % 4 == 0) take no rows, so
-        // the elimination keeps its issue slots
-        const bool worker = (warp & 3) != 0;
-        const int ow = warp - 1 - (warp >> 2), nw = nwarps - nwarps / 4;
-        const int NG = nw * rpw;        // row groups over all worker warps
-        const int gg = ow * rpw + grp;  // this lane group's first row
-        int jc[CPL];
+        const int ow = warp - EW;
+        int W2 = 1;
+        while (W2 < q && W2 < 32) W2 <<= 1;
+        const int rpw = 32 / W2, grp = lane / W2, col = lane % W2;
+        const int NG = NWK * rpw, gg = ow * rpw + grp;  // row groups, this group's first row
         bool cok[CPL];
 #pragma unroll
-        for (int k = 0; k < CPL; k++) {
-            jc[k] = CPL == 1 ? col : lane + 32 * k;
-            cok[k] = jc[k] < q;
-        }
-        RowTransform<MM, CPL, KLAZY> tr;
+        for (int k = 0; k < CPL; k++) cok[k] = col + 32 * k < q;
         for (int i = 0; i < bb; i++) {
-            named_sync(BAR_T0 + (i & 1), nth);
-            const uint32_t *F = Tb + (i & 1) * tw;
-            const uint32_t *dg = F + mq;
-            const int *sn = snap + (i & 1) * snapw;
-            const int *s_sh = sn, *s_base = sn + q, *s_isp = sn + 2 * q, *s_pc = sn + 3 * q;
-            const int np = sn[3 * q + m], dl = sn[3 * q + m + 1];
-            if (worker) tr.load(F, dg, s_pc, np, q, W2, grp, col, lane);
+            named_sync(BAR_T0 + (i & 1), NE + 32 * NWK);
+            const uint32_t *F = Fs + (i & 1) * mq, *dg = dgs + (i & 1) * 64;
+            const int *sn = snap + (i & 1) * LC_SNAP;
+            const int np = sn[224], D = sn[225];
+            uint32_t f[CPL][TM], d[CPL];
             int shc[CPL], bsc[CPL];
+            bool isp[CPL];
 #pragma unroll
             for (int k = 0; k < CPL; k++) {
-                shc[k] = cok[k] ? s_sh[jc[k]] : 0;
-                bsc[k] = cok[k] ? s_base[jc[k]] : 0;
-            }
-            // window row (ip, a2) of column j sits at Es[((ip - sh[j]) m + a2) q + j]
-            auto es = [&](bool ok, int ip, int a2, uint32_t *(&ptr)[CPL]) {
+                const int j = col + 32 * k;
+                d[k] = cok[k] ? dg[j] : 0u;
+                shc[k] = cok[k] ? sn[j] : 0;
+                bsc[k] = cok[k] ? sn[64 + j] : 0;
+                isp[k] = cok[k] && sn[128 + j] != 0;
 #pragma unroll
-                for (int k = 0; k < CPL; k++)
-                    ptr[k] = (ok && cok[k]) ? Es + ((size_t)(ip - shc[k]) * m + a2) * q + jc[k] : nullptr;
+                for (int t = 0; t < TM; t++) f[k][t] = (t < np && cok[k]) ? F[t * q + j] : 0u;
+            }
+            // lane t of a group fetches the row's residue at pivot column t
+            const bool pok = col < np;
+            const int pc = pok ? sn[192 + col] : 0;
+            const int shp = pok ? sn[pc] : 0, bsp = pok ? sn[64 + pc] : 0;
+            // one row: rp[k] the lane's columns, gp its pivot column (when ok); x[k] the new residues
+            auto row = [&](bool ok, uint32_t *const (&rp)[CPL], const uint32_t *gp, uint32_t (&x)[CPL]) {
+                uint32_t v[CPL];
+#pragma unroll
+                for (int k = 0; k < CPL; k++) v[k] = ok && cok[k] ? *rp[k] : 0u;
+                const uint32_t g = ok && pok ? *gp : 0u;
+                row_times<TM, CPL, FOLDK>(f, d, np, W2, v, g, x, fc, mp);
+                __syncwarp();
             };
-            // rows i and i+1 first (the next discrepancy)
-            if (worker) {
-                const int r1 = (i + 1 < bb ? 2 : 1) * m;
-                for (int row0 = ow * rpw; row0 < r1; row0 += NG) {
-                    const int row = row0 + grp;
-                    uint32_t *ptr[CPL];
-                    es(row < r1, i + (row >= m ? 1 : 0), row - (row >= m ? m : 0), ptr);
-                    tr.apply(ptr, mp);
-                }
-            }
-            named_arrive(BAR_RR0 + (i & 1), nth);
-            if (worker && np > 0) {
-                // window orders i+2 .. bb-1: rows gg, gg + NG, ... walked incrementally
-                const int wr = (bb - i - 2) > 0 ? (bb - i - 2) * m : 0;
-                {
-                    const int stepi = NG / m, stepa = NG - (NG / m) * m;
-                    int ip = i + 2 + gg / m, a2 = gg - (gg / m) * m;
-                    for (int row0 = ow * rpw; row0 < wr; row0 += NG) {
-                        uint32_t *ptr[CPL];
-                        es(row0 + grp < wr, ip, a2, ptr);
-                        tr.apply(ptr, mp);
-                        ip += stepi;
-                        a2 += stepa;
-                        if (a2 >= m) { a2 -= m; ip++; }
-                    }
-                }
-                // Qtop rows; the next Qtop keeps the pivot columns of Qtop T
-                for (int row0 = ow * rpw; row0 < m; row0 += NG) {
-                    const int a2 = row0 + grp;
-                    uint32_t *ptr[CPL];
+            auto es_at = [&](int ip, int al, int s, int c) { return Es + ((size_t)(ip - s) * l.ma + al) * q + c; };
+            // the next discrepancy: rows i and i + 1, to every block
+            if (i + 1 < bb) {
+                uint32_t *dn = disc + ((i + 1) & 1) * mq;
+                for (int r0 = ow * rpw; r0 < 2 * ma; r0 += NG) {
+                    // row i of a (its pivot columns) or row i + 1 (the others)
+                    const int al = (r0 + grp) >> 1, h = (r0 + grp) & 1;
+                    const bool ok = al < ma;
+                    uint32_t *rp[CPL], x[CPL];
 #pragma unroll
-                    for (int k = 0; k < CPL; k++) ptr[k] = (a2 < m && cok[k]) ? qt + a2 * q + jc[k] : nullptr;
-                    tr.apply(ptr, mp);
+                    for (int k = 0; k < CPL; k++) rp[k] = es_at(i + h, al, shc[k], col + 32 * k);
+                    row(ok, rp, es_at(i + h, al, shp, pc), x);
 #pragma unroll
-                    for (int k = 0; k < CPL; k++)
-                        if (ptr[k] && !s_isp[jc[k]]) *ptr[k] = 0;
-                }
-                // Ml coefficients 0..dl: rows (s2, x) walked incrementally
-                {
-                    const int mrows = (dl + 1) * q;
-                    const int steps2 = NG / q, stepx = NG - (NG / q) * q;
-                    int s2 = gg / q, x = gg - (gg / q) * q;
-                    for (int row0 = ow * rpw; row0 < mrows; row0 += NG) {
-                        const bool ok = row0 + grp < mrows;
-                        uint32_t *ptr[CPL];
-#pragma unroll
-                        for (int k = 0; k < CPL; k++)
-                            ptr[k] = (ok && cok[k]) ? Ml + ((size_t)(bsc[k] + s2) * q + x) * q + jc[k] : nullptr;
-                        tr.apply(ptr, mp);
-                        s2 += steps2;
-                        x += stepx;
-                        if (x >= q) { x -= q; s2++; }
-                    }
-                }
-            }
-            if (np == 0)  // no pivot: the next Qtop is zero
-                for (int x = tid - 32; x < mq; x += nth - 32) qt[x] = 0;
-        }
-    }
-    __syncthreads();
-    for (int x = tid; x < (bb + 1) * qq; x += nth) {
-        const int s2 = x / qq, c = x % q, y = (x / q) % q;
-        Ml_g[x] = Ml[((size_t)(base[c] + s2) * q + y) * q + c];
-    }
-    for (int x = tid; x < mq; x += nth) qtop_g[x] = qt[x];
-    for (int c = tid; c < q; c += nth) {
-        deg_g[c] = deg[c];
-        degl_g[c] = degl[c];
-    }
-    if (tid == 0) {
-        // bound on the polynomial degree of the basis: column c's degree
-        // minus the smallest starting degree (the row shifts)
-        int dmx = 0;
-        for (int c = 0; c < q; c++) dmx = max(dmx, deg[c] - dbase);
-        *dmax_g = dmx;
-    }
-}
-
-// ---- local M-Basis for wide blocks (q = m + n > 32; m <= 32, q <= 64): one
-// block of LW_THREADS threads, every warp taking part in every phase of an
-// order, with barriers between the phases.
-//
-//   ranks : the (degree, index) order of the columns, and the discrepancy
-//           column registers: warp w holds columns w, w + 16, w + 32, w + 48,
-//           lane a row a of each (and coefficient a of its transform);
-//   elim  : one step per column in that order, ended once m pivots are found
-//           (then every remaining column is zero on all m rows).  The owner
-//           warp of the step's column finds its first nonzero row and, if
-//           there is one, publishes the pivot column through a double-buffered
-//           shared slot; after a barrier every warp reduces its later columns
-//           by it, fraction-free as in k_local;
-//   publish: the transform (normal form) and the local degree bounds;
-//   rows  : every row of the window (orders i ..), of Qtop and of the chunk
-//           transform Ml (coefficients 0 .. dl) times the transform, one row
-//           per warp, the pivot residues read as shared-memory broadcasts;
-//   shift : the pivot columns times x, moved in place: window orders i+1 ..
-//           and Ml coefficients 1 .. dl+1 take the column's values one order /
-//           one coefficient down, so that rows stay plain (no per-column
-//           offsets).
-// The pivots, the transforms, P and the degrees are those of k_local.
-constexpr int LW_THREADS = 512;
-constexpr int LW_WARPS = LW_THREADS / 32;
-constexpr int LW_CPW = 64 / LW_WARPS;  // columns per warp in the elimination
-constexpr int LW_SLOT = 68;            // pivot slot: 32 residues, 32 transform coefficients, fr, dc, scale
-
-// dynamic shared memory of k_local_wide for chunks of b orders; the rows of
-// the window and of the transform are padded to q + 1 words, so that a
-// column (one residue per lane, rows apart) falls on distinct banks
-__host__ __device__ constexpr size_t local_wide_bytes(int b, int m, int q) {
-    return sizeof(uint32_t) * ((size_t)b * m * (q + 1) + (size_t)(b + 1) * q * q + (size_t)m * (q + 1) + (size_t)m * q +
-                               64 + 2 * LW_SLOT) +
-           sizeof(int) * (5 * 64 + 32 + 8);
-}
-
-template <int FOLDK>
-__global__ void __launch_bounds__(LW_THREADS, 1)
-    k_local_wide(int m, int n, int q, int bb, int nparts, const uint32_t *__restrict__ Epart,
-                 uint32_t *__restrict__ qtop_g, int32_t *__restrict__ deg_g, uint32_t *__restrict__ Ml_g,
-                 int32_t *__restrict__ degl_g, int *__restrict__ dmax_g, uint32_t *__restrict__ scale_g, int dbase,
-                 ModP mp) {
-    extern __shared__ uint32_t sm[];
-    const int mq = m * q, qq = q * q, qs = q + 1;
-    uint32_t *Es = sm;                            // [bb][m][qs]
-    uint32_t *Ml = Es + (size_t)bb * m * qs;      // [bb+1][q][q]
-    uint32_t *F = Ml + (size_t)(bb + 1) * qq;     // [m][qs] transform of the order
-    uint32_t *qt = F + (size_t)m * qs;            // [m][q]
-    uint32_t *dg = qt + mq;                       // [64]
-    uint32_t *slot = dg + 64;                     // [2][LW_SLOT]
-    int *deg = (int *)(slot + 2 * LW_SLOT);       // [64]
-    int *degl = deg + 64;                         // [64] local degrees
-    int *dln = degl + 64;                         // [64] local degrees after the transform
-    int *colof = dln + 64;                        // [64] column of each rank
-    int *isp = colof + 64;                        // [64] pivot flags of the order
-    int *pcs = isp + 64;                          // [32] pivot columns in order
-    int *misc = pcs + 32;                         // [0]: max local degree after the transform
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned FULL = 0xffffffffu;
-    const uint32_t fc = mp.r1;  // 2^32 mod p
-    (void)n;
-
-    for (int x = tid; x < mq; x += LW_THREADS) qt[x] = qtop_g[x];
-    __syncthreads();
-    const int E = bb * mq;
-    for (int x = tid; x < E; x += LW_THREADS) {
-        unsigned long long v = 0;
-        for (int b = 0; b < nparts; b++) v += Epart[(size_t)b * E + x];
-        uint32_t e = red64(v, mp);
-        if (x < mq) e = subm(e, qt[x], mp);
-        Es[(x / q) * qs + x % q] = e;
-    }
-    for (int x = tid; x < (bb + 1) * qq; x += LW_THREADS) Ml[x] = (x < qq && x / q == x % q) ? 1u : 0u;
-    for (int c = tid; c < 64; c += LW_THREADS) {
-        deg[c] = c < q ? deg_g[c] : 0;
-        degl[c] = 0;
-    }
-    uint32_t scum[LW_CPW];  // cumulative column scales over the chunk (Montgomery form)
-#pragma unroll
-    for (int k = 0; k < LW_CPW; k++) scum[k] = mp.r1;
-    __syncthreads();
-
-    for (int i = 0; i < bb; i++) {
-        // ---- ranks and the discrepancy registers
-        uint32_t d[LW_CPW], tp[LW_CPW], sc[LW_CPW];
-        int rk[LW_CPW];
-        {
-            const int la = lane, lb = lane + 32;
-            const int da = la < q ? deg[la] : 0, db = lb < q ? deg[lb] : 0;
-#pragma unroll
-            for (int k = 0; k < LW_CPW; k++) {
-                const int c = warp + LW_WARPS * k;
-                const bool cv = c < q;
-                const int dc = cv ? deg[c] : 0;
-                const bool xa = cv && la < q && (da < dc || (da == dc && la < c));
-                const bool xb = cv && lb < q && (db < dc || (db == dc && lb < c));
-                const int r = __popc(__ballot_sync(FULL, xa)) + __popc(__ballot_sync(FULL, xb));
-                rk[k] = cv ? r : (1 << 20);
-                d[k] = (cv && lane < m) ? to_mont(Es[((size_t)i * m + lane) * qs + c], mp) : 0u;
-                tp[k] = 0u;
-                sc[k] = mp.r1;
-                if (cv && lane == 0) {
-                    colof[r] = c;
-                    isp[c] = 0;
-                }
-            }
-        }
-        if (tid == 0) misc[0] = 0;
-        __syncthreads();
-        // ---- elimination
-        int np = 0;
-        for (int step = 0; step < q && np < m; step++) {
-            const int c = colof[step];
-            uint32_t *sl = slot + (step & 1) * LW_SLOT;
-            if ((c & (LW_WARPS - 1)) == warp) {
-                const int kk = c / LW_WARPS;
-                uint32_t v = 0, t = 0, s = 0;
-#pragma unroll
-                for (int k = 0; k < LW_CPW; k++)
-                    if (k == kk) {
-                        v = d[k];
-                        t = tp[k];
-                        s = sc[k];
-                    }
-                const int fr = __ffs(__ballot_sync(FULL, v != 0u)) - 1;
-                if (fr >= 0) {
-                    const uint32_t dcv = __shfl_sync(FULL, v, fr);
-                    sl[lane] = v;
-                    sl[32 + lane] = t;
-                    if (lane == 0) {
-                        sl[64] = (uint32_t)fr;
-                        sl[65] = dcv;
-                        sl[66] = s;
-                        pcs[np] = c;
-                        isp[c] = 1;
-                    }
-                } else if (lane == 0) {
-                    sl[64] = 0xffffffffu;
-                }
-            }
-            __syncthreads();
-            const int fr = (int)sl[64];
-            if (fr < 0) continue;
-            const uint32_t pv = sl[lane], pt = sl[32 + lane], dcv = sl[65], scc = sl[66];
-#pragma unroll
-            for (int k = 0; k < LW_CPW; k++) {
-                if (rk[k] > step && rk[k] < (1 << 20)) {
-                    const uint32_t dj = __shfl_sync(FULL, d[k], fr);
-                    if (dj != 0u) {
-                        // col <- dc col - dj pivot: dc x + (p - dj) y < 2 p^2 < p 2^32
-                        const uint32_t ndj = mp.p - dj;
-                        d[k] = mont_redc(madw(ndj, pv, (unsigned long long)dcv * d[k]), mp);
-                        if (lane < np) tp[k] = mont_redc(madw(ndj, pt, (unsigned long long)dcv * tp[k]), mp);
-                        else if (lane == np) tp[k] = mont_redc((unsigned long long)ndj * scc, mp);
-                        sc[k] = mont_mul(sc[k], dcv, mp);
-                    }
-                }
-            }
-            np++;
-        }
-        // ---- publish the transform (normal form) and the local degree bounds
-#pragma unroll
-        for (int k = 0; k < LW_CPW; k++) {
-            const int c = warp + LW_WARPS * k;
-            if (c < q) {
-                const uint32_t fv = lane < np ? from_mont(tp[k], mp) : 0u;
-                if (lane < np) F[lane * qs + c] = fv;
-                const int v = __reduce_max_sync(FULL, fv != 0u ? degl[pcs[lane]] : 0);
-                const int dl = max(degl[c], v);
-                if (lane == 0) {
-                    dg[c] = from_mont(sc[k], mp);
-                    dln[c] = dl;
-                    atomicMax(misc, dl);
-                }
-                scum[k] = mont_mul(scum[k], sc[k], mp);
-            }
-        }
-        __syncthreads();
-        const int dl = misc[0];
-        // ---- rows times the transform
-        if (np > 0) {
-            const int ja = lane, jb = lane + 32;
-            const bool vb = jb < q;
-            uint32_t fa[32], fb[32];
-#pragma unroll
-            for (int t = 0; t < 32; t++) {
-                fa[t] = t < np ? F[t * qs + ja] : 0u;
-                fb[t] = (t < np && vb) ? F[t * qs + jb] : 0u;
-            }
-            const uint32_t ga = dg[ja], gb = vb ? dg[jb] : 0u;
-            const int pcl = lane < np ? pcs[lane] : 0;  // lane t fetches the row's residue at pivot column t
-            const int nwin = (bb - i) * m;
-            const int nrows = nwin + m + (dl + 1) * q;
-            for (int row = warp; row < nrows; row += LW_WARPS) {
-                uint32_t *rp = row < nwin ? Es + ((size_t)i * m + row) * qs
-                                          : (row < nwin + m ? qt + (row - nwin) * q : Ml + (size_t)(row - nwin - m) * q);
-                const uint32_t xa = rp[ja], xb = vb ? rp[jb] : 0u, g = rp[pcl];
-                // two accumulators per column (even and odd t), each folded
-                // after FOLDK of its own products
-                unsigned long long a0 = (unsigned long long)ga * xa, b0 = (unsigned long long)gb * xb;
-                unsigned long long a1 = 0ull, b1 = 0ull;
-#pragma unroll
-                for (int t = 0; t < 32; t++) {
-                    if (t < np) {
-                        const uint32_t v = __shfl_sync(FULL, g, t);
-                        if ((t & 1) == 0) {
-                            a0 = madw(fa[t], v, a0);
-                            b0 = madw(fb[t], v, b0);
-                            if ((t / 2 + 2) % FOLDK == 0) {
-                                a0 = fold2(a0, fc);
-                                b0 = fold2(b0, fc);
-                            }
-                        } else {
-                            a1 = madw(fa[t], v, a1);
-                            b1 = madw(fb[t], v, b1);
-                            if (((t + 1) / 2) % FOLDK == 0) {
-                                a1 = fold2(a1, fc);
-                                b1 = fold2(b1, fc);
+                    for (int k = 0; k < CPL; k++) {
+                        if (ok && cok[k]) {
+                            *rp[k] = x[k];
+                            if (isp[k] == (h == 0)) {
+                                uint32_t *dst = dn + (rank + CS * al) * q + col + 32 * k;
+                                for (int b = 0; b < CS; b++) st_cluster(dst, (uint32_t)b, x[k]);
                             }
                         }
                     }
                 }
-                // folded, each is below 2^62 + 2^32: their sum fits
-                uint32_t ra = red64(fold2(a0, fc) + fold2(a1, fc), mp), rb = red64(fold2(b0, fc) + fold2(b1, fc), mp);
-                if (row >= nwin && row < nwin + m) {  // the next Qtop keeps the pivot columns of Qtop T
-                    if (!isp[ja]) ra = 0u;
-                    if (vb && !isp[jb]) rb = 0u;
-                }
-                __syncwarp();
-                rp[ja] = ra;
-                if (vb) rp[jb] = rb;
-                __syncwarp();
             }
-        } else {
-            for (int x = tid; x < mq; x += LW_THREADS) qt[x] = 0u;  // no pivot: the next Qtop is zero
-        }
-        __syncthreads();
-        // ---- pivot columns times x (consecutive threads: the pivots of one
-        // row, distinct columns)
-        for (int w = tid; w < np * m; w += LW_THREADS) {
-            const int a = w / np, c = pcs[w - a * np];
-            for (int ip = bb - 1; ip > i; ip--)
-                Es[((size_t)ip * m + a) * qs + c] = Es[((size_t)(ip - 1) * m + a) * qs + c];
-        }
-        for (int w = tid; w < np * q; w += LW_THREADS) {
-            const int y = w / np, c = pcs[w - y * np];
-            for (int s = dl + 1; s > 0; s--) Ml[((size_t)s * q + y) * q + c] = Ml[((size_t)(s - 1) * q + y) * q + c];
-            Ml[(size_t)y * q + c] = 0u;
-        }
-        for (int c = tid; c < q; c += LW_THREADS) {
-            degl[c] = dln[c] + isp[c];
-            deg[c] += isp[c];
-        }
-        __syncthreads();
-    }
-    for (int x = tid; x < (bb + 1) * qq; x += LW_THREADS) Ml_g[x] = Ml[x];
-    for (int x = tid; x < mq; x += LW_THREADS) qtop_g[x] = qt[x];
-    for (int c = tid; c < q; c += LW_THREADS) {
-        deg_g[c] = deg[c];
-        degl_g[c] = degl[c];
-    }
-    if (lane == 0) {
+            __syncwarp();
+            cluster_arrive();
+            // window orders i + 2 .. bb - 1
+            if (np > 0 && ma > 0) {
+                const int rows = (bb - i - 2) * ma;
+                const int stepi = NG / ma, stepa = NG - stepi * ma;
+                int ip = i + 2 + gg / ma, al = gg % ma;
+                for (int r0 = ow * rpw; r0 < rows; r0 += NG) {
+                    const bool ok = r0 + grp < rows;
+                    uint32_t *rp[CPL], x[CPL];
 #pragma unroll
-        for (int k = 0; k < LW_CPW; k++) {
-            const int c = warp + LW_WARPS * k;
-            if (c < q) scale_g[c] = mont_mul(scale_g[c], scum[k], mp);
+                    for (int k = 0; k < CPL; k++) rp[k] = es_at(ip, al, shc[k], col + 32 * k);
+                    row(ok, rp, es_at(ip, al, shp, pc), x);
+#pragma unroll
+                    for (int k = 0; k < CPL; k++)
+                        if (ok && cok[k]) *rp[k] = x[k];
+                    ip += stepi;
+                    al += stepa;
+                    if (al >= ma) { al -= ma; ip++; }
+                }
+            }
+            // Qtop; the next one keeps the pivot columns of Qtop T
+            for (int r0 = ow * rpw; r0 < ma; r0 += NG) {
+                const int al = r0 + grp;
+                const bool ok = al < ma;
+                uint32_t *rp[CPL], x[CPL];
+#pragma unroll
+                for (int k = 0; k < CPL; k++) rp[k] = qt + al * q + col + 32 * k;
+                row(ok, rp, qt + al * q + pc, x);
+#pragma unroll
+                for (int k = 0; k < CPL; k++)
+                    if (ok && cok[k]) *rp[k] = isp[k] ? x[k] : 0u;
+            }
+            // Ml coefficients 0 .. D
+            if (np > 0 && mx > 0) {
+                const int rows = (D + 1) * mx;
+                const int steps = NG / mx, stepx = NG - steps * mx;
+                int s = gg / mx, xl = gg % mx;
+                for (int r0 = ow * rpw; r0 < rows; r0 += NG) {
+                    const bool ok = r0 + grp < rows;
+                    uint32_t *rp[CPL], x[CPL];
+#pragma unroll
+                    for (int k = 0; k < CPL; k++) rp[k] = Ml + ((size_t)(bsc[k] + s) * l.mx + xl) * q + col + 32 * k;
+                    row(ok, rp, Ml + ((size_t)(bsp + s) * l.mx + xl) * q + pc, x);
+#pragma unroll
+                    for (int k = 0; k < CPL; k++)
+                        if (ok && cok[k]) *rp[k] = x[k];
+                    s += steps;
+                    xl += stepx;
+                    if (xl >= mx) { xl -= mx; s++; }
+                }
+            }
+            __syncwarp();
+            cluster_wait();
         }
     }
-    if (tid == 0) {
-        // bound on the polynomial degree of the basis: column c's degree
-        // minus the smallest starting degree (the row shifts)
-        int dmx = 0;
-        for (int c = 0; c < q; c++) dmx = max(dmx, deg[c] - dbase);
-        *dmax_g = dmx;
+    __syncthreads();
+    const int qq = q * q;
+    for (int y = tid; y < (bb + 1) * l.mx * q; y += NT) {
+        const int c = y % q, xl = y / q % l.mx, s = y / (q * l.mx), x = rank + CS * xl;
+        if (x < q) Ml_g[(size_t)s * qq + x * q + c] = Ml[((size_t)(base[c] + s) * l.mx + xl) * q + c];
+    }
+    for (int x = tid; x < l.ma * q; x += NT) {
+        const int a = rank + CS * (x / q);
+        if (a < m) qtop_g[a * q + x % q] = qt[x];
+    }
+    if (rank == 0) {
+        for (int c = tid; c < q; c += NT) {
+            deg_g[c] = deg[c];
+            degl_g[c] = degl[c];
+            scale_g[c] = mont_mul(scale_g[c], scum[c], mp);
+        }
+        if (tid == 0) {
+            // bound on the polynomial degree of the basis: column c's degree
+            // minus the smallest starting degree (the row shifts)
+            int d = 0;
+            for (int c = 0; c < q; c++) d = max(d, deg[c] - dbase);
+            *dmax_g = d;
+        }
     }
 }
 
@@ -1095,207 +912,6 @@ __global__ void k_unscale(uint32_t *__restrict__ P, int n, int q, int64_t D, con
     const int64_t nq = (int64_t)n * q;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < (D + 1) * nq; x += (int64_t)gridDim.x * blockDim.x)
         P[x] = mulm(P[x], inv[x % q], mp);
-}
-
-// ---- apply: P_new[t][r][c] = sum_{s <= degl[c]} sum_x P[t-s][r][x] Ml[s][x][c]
-constexpr int APP_THREADS = 256;
-constexpr int APP_TB = 8;  // coefficients per thread
-constexpr int APP_CB = 4;  // columns per thread
-static_assert(APP_TB == 8 && APP_CB == 4, "the register window and 16-byte loads assume an 8 x 4 tile");
-
-// P' = P Ml (the chunk transform, logical layout: coefficient s of column c
-// at Ml[s][.][c], zero above degl[c]), coefficients t0 .. t0 + TA - 1 of P' per
-// block.  Coefficients above the new maximal column degree (*dmax_dev) are
-// zero in P' and already zero in the target buffer (it held an older basis of
-// no larger degree), so blocks beyond it return at once.  A thread owns a
-// APP_TB x APP_CB tile (coefficients x columns) of one row r of P'.  For a
-// fixed x it walks s: the P residues of step s+1 are those of step s shifted
-// by one coefficient (circular register window, one new load per step), and
-// the APP_CB residues of Ml are one 16-byte load (VEC).
-template <int FOLDK, bool VEC>
-__global__ void __launch_bounds__(APP_THREADS)
-    k_apply(const uint32_t *__restrict__ P, uint32_t *__restrict__ Pn, int n, int q,
-            const uint32_t *__restrict__ Ml_g, const int32_t *__restrict__ degl_g, int bb, int64_t Dbound,
-            int TA, const int *__restrict__ dmax_dev, ModP mp) {
-    extern __shared__ uint32_t sm[];
-    uint32_t *Mls = sm;                               // (bb+1)*q*q
-    uint32_t *Pss = Mls + (size_t)(bb + 1) * q * q;   // (TA + bb) * n * q
-    __shared__ int degl[64];
-    const int64_t dlim = min64(Dbound, (int64_t)*dmax_dev);
-    const int64_t t0 = (int64_t)blockIdx.x * TA;
-    if (t0 > dlim) return;
-    const int ta = (int)min64(TA, dlim + 1 - t0);
-    const int nq = n * q;
-    const uint32_t fc = mp.r1;  // 2^32 mod p
-    for (int x = threadIdx.x; x < (bb + 1) * q * q; x += APP_THREADS) Mls[x] = Ml_g[x];
-    for (int x = threadIdx.x; x < q; x += APP_THREADS) degl[x] = degl_g[x];
-    const int64_t pbase = t0 - bb;  // Pss[u] holds P[pbase + u]
-    for (int x = threadIdx.x; x < (ta + bb) * nq; x += APP_THREADS) {
-        const int64_t t = pbase + x / nq;
-        Pss[x] = t >= 0 ? P[(size_t)t * nq + x % nq] : 0u;
-    }
-    __syncthreads();
-    const int ntb = (ta + APP_TB - 1) / APP_TB, ncb = (q + APP_CB - 1) / APP_CB;
-    for (int it = threadIdx.x; it < ntb * n * ncb; it += APP_THREADS) {
-        const int cb = it % ncb, r = (it / ncb) % n, tb = it / (ncb * n);
-        const int c0 = cb * APP_CB, tl0 = tb * APP_TB;
-        bool cv[APP_CB];
-        int smax = 0;
-#pragma unroll
-        for (int u = 0; u < APP_CB; u++) {
-            cv[u] = c0 + u < q;
-            if (cv[u]) smax = max(smax, degl[c0 + u]);
-        }
-        Acc2 acc[APP_TB][APP_CB];
-#pragma unroll
-        for (int k = 0; k < APP_TB; k++)
-#pragma unroll
-            for (int u = 0; u < APP_CB; u++) acc[k][u] = Acc2{0u, 0u};
-        int cnt = 0;
-        // coefficient t0 + tl0 + k - s of P is Pss row top - s + k
-        const int top = tl0 + bb;
-        for (int x = 0; x < q; x++) {
-            const uint32_t *pc = Pss + r * q + x;          // row u at pc[u * nq]
-            const uint32_t *mc = Mls + (size_t)x * q + c0;  // coefficient s at mc[s * q * q]
-            uint32_t pw[APP_TB];                            // row top - s + k in slot (k - s) & 7
-#pragma unroll
-            for (int k = 0; k < APP_TB; k++) pw[k] = pc[(size_t)(top + k) * nq];
-            for (int s0 = 0; s0 <= smax; s0 += 8) {
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    const int st = s0 + j;
-                    if (st <= smax) {
-                        if (st > 0) pw[(8 - j) & 7] = pc[(size_t)(top - st) * nq];
-                        uint32_t mv[APP_CB];
-                        ld4<VEC>(mc + (size_t)st * q * q, cv, mv);
-#pragma unroll
-                        for (int k = 0; k < APP_TB; k++)
-#pragma unroll
-                            for (int u = 0; u < APP_CB; u++) mac2(acc[k][u], pw[(k - j) & 7], mv[u]);
-                        if (++cnt == FOLDK) {
-#pragma unroll
-                            for (int k = 0; k < APP_TB; k++)
-#pragma unroll
-                                for (int u = 0; u < APP_CB; u++) fold2w(acc[k][u], fc);
-                            cnt = 0;
-                        }
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < APP_TB; k++) {
-            const int tl = tl0 + k;
-#pragma unroll
-            for (int u = 0; u < APP_CB; u++)
-                if (tl < ta && cv[u]) Pn[(size_t)(t0 + tl) * nq + r * q + c0 + u] = red64(acc2_u64(acc[k][u]), mp);
-        }
-    }
-}
-
-// Four consecutive residues through the read-only data cache (one 16-byte
-// load when VEC), zero where the column is out of range.
-template <bool VEC>
-__device__ __forceinline__ void ldg4(const uint32_t *p, const bool (&cv)[4], uint32_t (&v)[4]) {
-    if constexpr (VEC) {
-        const uint4 t = __ldg(reinterpret_cast<const uint4 *>(p));
-        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-    } else {
-#pragma unroll
-        for (int u = 0; u < 4; u++) v[u] = cv[u] ? __ldg(p + u) : 0u;
-    }
-}
-
-// P' = P Ml for wide blocks (q > 32), where Ml and whole coefficients of P
-// do not fit in shared memory together: block (coefficient tile of APW_TA,
-// group of APW_RB rows of P); the tile's rows of P (with the bb coefficients
-// below it) in shared memory, Ml through the read-only cache (it is shared by
-// all blocks).  The thread tiles and the register window are those of k_apply.
-constexpr int APW_RB = 4, APW_TA = 32;
-
-__host__ __device__ constexpr size_t apply_wide_bytes(int b, int q) {
-    return sizeof(uint32_t) * (size_t)(APW_TA + b) * APW_RB * q;
-}
-
-template <int FOLDK, bool VEC>
-__global__ void __launch_bounds__(APP_THREADS, 2)
-    k_apply_wide(const uint32_t *__restrict__ P, uint32_t *__restrict__ Pn, int n, int q,
-                 const uint32_t *__restrict__ Ml_g, const int32_t *__restrict__ degl_g, int bb, int64_t Dbound,
-                 const int *__restrict__ dmax_dev, ModP mp) {
-    extern __shared__ uint32_t sm[];
-    __shared__ int degl[64];
-    const int64_t dlim = min64(Dbound, (int64_t)*dmax_dev);
-    const int64_t t0 = (int64_t)blockIdx.x * APW_TA;
-    if (t0 > dlim) return;
-    const int ta = (int)min64(APW_TA, dlim + 1 - t0);
-    const int r0 = blockIdx.y * APW_RB, rn = min(APW_RB, n - r0);
-    const int nq = n * q, rq = APW_RB * q, qq = q * q;
-    const uint32_t fc = mp.r1;  // 2^32 mod p
-    for (int x = threadIdx.x; x < q; x += APP_THREADS) degl[x] = degl_g[x];
-    const int64_t pbase = t0 - bb;  // sm[u rq + rl q + x] holds P[pbase + u][r0 + rl][x]
-    for (int x = threadIdx.x; x < (ta + bb) * rq; x += APP_THREADS) {
-        const int u = x / rq, rem = x - u * rq, rl = rem / q;
-        const int64_t t = pbase + u;
-        sm[x] = (t >= 0 && rl < rn) ? P[(size_t)t * nq + (size_t)(r0 + rl) * q + (rem - rl * q)] : 0u;
-    }
-    __syncthreads();
-    const int ntb = (ta + APP_TB - 1) / APP_TB, ncb = (q + APP_CB - 1) / APP_CB;
-    for (int it = threadIdx.x; it < ntb * APW_RB * ncb; it += APP_THREADS) {
-        const int cb = it % ncb, rl = (it / ncb) % APW_RB, tb = it / (ncb * APW_RB);
-        if (rl >= rn) continue;
-        const int c0 = cb * APP_CB, tl0 = tb * APP_TB;
-        bool cv[APP_CB];
-        int smax = 0;
-#pragma unroll
-        for (int u = 0; u < APP_CB; u++) {
-            cv[u] = c0 + u < q;
-            if (cv[u]) smax = max(smax, degl[c0 + u]);
-        }
-        Acc2 acc[APP_TB][APP_CB];
-#pragma unroll
-        for (int k = 0; k < APP_TB; k++)
-#pragma unroll
-            for (int u = 0; u < APP_CB; u++) acc[k][u] = Acc2{0u, 0u};
-        int cnt = 0;
-        const int top = tl0 + bb;  // coefficient t0 + tl0 + k - s of P is slab row top - s + k
-        for (int x = 0; x < q; x++) {
-            const uint32_t *pc = sm + rl * q + x;       // slab row u at pc[u * rq]
-            const uint32_t *mc = Ml_g + (size_t)x * q + c0;  // coefficient s at mc[s * qq]
-            uint32_t pw[APP_TB];                        // slab row top - s + k in slot (k - s) & 7
-#pragma unroll
-            for (int k = 0; k < APP_TB; k++) pw[k] = pc[(size_t)(top + k) * rq];
-            for (int s0 = 0; s0 <= smax; s0 += 8) {
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    const int st = s0 + j;
-                    if (st <= smax) {
-                        if (st > 0) pw[(8 - j) & 7] = pc[(size_t)(top - st) * rq];
-                        uint32_t mv[APP_CB];
-                        ldg4<VEC>(mc + (size_t)st * qq, cv, mv);
-#pragma unroll
-                        for (int k = 0; k < APP_TB; k++)
-#pragma unroll
-                            for (int u = 0; u < APP_CB; u++) mac2(acc[k][u], pw[(k - j) & 7], mv[u]);
-                        if (++cnt == FOLDK) {
-#pragma unroll
-                            for (int k = 0; k < APP_TB; k++)
-#pragma unroll
-                                for (int u = 0; u < APP_CB; u++) fold2w(acc[k][u], fc);
-                            cnt = 0;
-                        }
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < APP_TB; k++) {
-            const int tl = tl0 + k;
-#pragma unroll
-            for (int u = 0; u < APP_CB; u++)
-                if (tl < ta && cv[u])
-                    Pn[(size_t)(t0 + tl) * nq + (size_t)(r0 + rl) * q + c0 + u] = red64(acc2_u64(acc[k][u]), mp);
-        }
-    }
 }
 
 // ---------------------------------------------------------------- readout
@@ -1444,33 +1060,15 @@ static wr_status mbasis_run(wr_ctx *ctx, const uint32_t *d_S, int64_t L, int m, 
 
     // chunk size b and tiles: every kernel's shared memory must fit
     const size_t budget = std::min<size_t>(ctx->smem_optin, 227 * 1024) - 1024;
-    auto local_bytes = [&](int b) {
-        return sizeof(uint32_t) * ((size_t)b * m * q + (size_t)(2 * b + 1) * q * q + 3 * (size_t)m * q + 2 * q) +
-               sizeof(int) * (4 * q + 2 * (3 * q + m + 2));
-    };
-    auto window_bytes = [&](int TT, int b) {
-        const int nib = (b + WIN_IB - 1) / WIN_IB;
-        return sizeof(uint32_t) * ((size_t)TT * nq + (size_t)(nib * WIN_IB + TT - 1) * m * nr);
-    };
-    auto apply_bytes = [&](int ta, int b) { return sizeof(uint32_t) * ((size_t)(b + 1) * q * q + (size_t)(ta + b) * nq); };
-    // wide blocks (q > 32): k_local_wide and k_apply_wide, and chunks one
-    // order shorter at a time (their shared memory grows in steps of a few KB)
-    const bool wide = q > 32;
-    auto local_need = [&](int b) { return wide ? local_wide_bytes(b, m, q) : local_bytes(b); };
-    auto apply_need = [&](int ta, int b) { return wide ? apply_wide_bytes(b, q) : apply_bytes(ta, b); };
-    int bmax = ctx->sigma_chunk > 0 ? std::min(ctx->sigma_chunk, 64) : (wide ? SIGMA_CHUNK_WIDE : SIGMA_CHUNK_DEFAULT),
-        TT = 32, TA = 64;
-    for (;;) {
-        while (TT > 4 && window_bytes(TT, bmax) > budget) TT /= 2;
-        while (TA > APP_TB && apply_need(TA, bmax) > budget) TA /= 2;
-        if (local_need(bmax) <= budget && window_bytes(TT, bmax) <= budget && apply_need(TA, bmax) <= budget) break;
-        if (bmax == 1) return fail(WR_EINVAL, "block sizes too large for shared memory");
-        bmax = wide ? bmax - 1 : bmax / 2;
-        TT = 32;
-        TA = 64;
-    }
-    if (wide) TA = APW_TA;
-    const int nparts_max = std::max(1, 2 * ctx->num_sms);
+    const int MR = m <= 8 ? 8 : (m <= 16 ? 16 : 32), CS = local_cluster(q);
+    auto local_need = [&](int b) { return sizeof(uint32_t) * (size_t)lc_layout(m, q, b, CS, MR).total; };
+    int bmax = ctx->sigma_chunk > 0 ? std::min(ctx->sigma_chunk, 64) : sigma_chunk_default(q);
+    while (bmax > 1 && local_need(bmax) > budget) bmax--;
+    if (local_need(bmax) > budget) return fail(WR_EINVAL, "block sizes too large for shared memory");
+    // the window's coefficients split so that about three blocks an SM run
+    const int NC = q <= 16 ? 16 : (q <= 32 ? 32 : 64), BR = 4096 / NC;
+    const int wtiles = (bmax * m + BR - 1) / BR;
+    const int nparts_max = std::max(1, 3 * ctx->num_sms / wtiles);
     WR_TRY(dev_alloc(ctx, Epart, sizeof(uint32_t) * (size_t)nparts_max * bmax * m * q));
     WR_TRY(dev_alloc(ctx, Ml, sizeof(uint32_t) * (size_t)(bmax + 1) * q * q));
     WR_TRY(dev_alloc(ctx, degl, sizeof(int32_t) * q));
@@ -1480,45 +1078,21 @@ static wr_status mbasis_run(wr_ctx *ctx, const uint32_t *d_S, int64_t L, int m, 
         WR_CUDA(cudaMemcpyAsync(scale.ptr, one.data(), sizeof(uint32_t) * q, cudaMemcpyHostToDevice, s));
         WR_CUDA(cudaStreamSynchronize(s));
     }
-    const bool lazy16 = mp.lazy >= 16;
-    const bool vec = q % 4 == 0;
-    // fold interval of the lazily reduced sums: 14 (p < 2^30), 3 (2^32 mod p
-    // small, as for p = 2^31 - 19), else 2
-    const int fk = fold_products(p), fold = fk >= 14 ? 14 : (fk >= 3 ? 3 : 2);
-    // order tiles of 4 for chunks of at most 4 orders (8 would idle half the tile)
-    auto win_for = [&](int b) {
-        if (b <= 4)
-            return fold == 14 ? (vec ? k_window<14, true, 4> : k_window<14, false, 4>)
-                   : fold == 3 ? (vec ? k_window<3, true, 4> : k_window<3, false, 4>)
-                               : (vec ? k_window<2, true, 4> : k_window<2, false, 4>);
-        return fold == 14 ? (vec ? k_window<14, true, 8> : k_window<14, false, 8>)
-               : fold == 3 ? (vec ? k_window<3, true, 8> : k_window<3, false, 8>)
-                           : (vec ? k_window<2, true, 8> : k_window<2, false, 8>);
-    };
-    auto *kwin = win_for(bmax);
-    auto *kwin_tail = win_for(std::min<int64_t>(bmax, L % bmax ? L % bmax : bmax));
-    auto *kapp = fold == 14 ? (vec ? k_apply<14, true> : k_apply<14, false>)
-                 : fold == 3 ? (vec ? k_apply<3, true> : k_apply<3, false>)
-                             : (vec ? k_apply<2, true> : k_apply<2, false>);
-    auto *kapp_w = fold == 14 ? (vec ? k_apply_wide<14, true> : k_apply_wide<14, false>)
-                   : fold == 3 ? (vec ? k_apply_wide<3, true> : k_apply_wide<3, false>)
-                               : (vec ? k_apply_wide<2, true> : k_apply_wide<2, false>);
+    const bool big = p > (1u << 30);  // fold1_products: 4 products, else 12
+    auto *ktoep = NC == 16 ? (big ? k_toeplitz<16, 4> : k_toeplitz<16, 8>)
+                  : NC == 32 ? (big ? k_toeplitz<32, 4> : k_toeplitz<32, 8>)
+                             : (big ? k_toeplitz<64, 4> : k_toeplitz<64, 8>);
     DevBuf Esum;
     WR_TRY(dev_alloc(ctx, Esum, sizeof(uint32_t) * (size_t)bmax * m * q));
-    using LocalFn = void (*)(int, int, int, int, int, const uint32_t *, uint32_t *, int32_t *, uint32_t *, int32_t *,
-                             int *, uint32_t *, int, ModP);
-    LocalFn kloc;
-    if (wide)
-        kloc = fold == 14 ? k_local_wide<14> : (fold == 3 ? k_local_wide<3> : k_local_wide<2>);
-    else if (m <= 8)
-        kloc = lazy16 ? k_local<8, 1, 16> : k_local<8, 1, 4>;
-    else
-        kloc = lazy16 ? k_local<32, 1, 16> : k_local<32, 1, 4>;
-    WR_CUDA(cudaFuncSetAttribute(kwin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
-    WR_CUDA(cudaFuncSetAttribute(kwin_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
+    using LocalFn = void (*)(int, int, int, const uint32_t *, uint32_t *, int32_t *, uint32_t *, int32_t *, int *,
+                             uint32_t *, int, ModP);
+    LocalFn kloc = nullptr;
+#define WR_LOCAL(MRV, CPLV, QCV) kloc = big ? k_local<MRV, CPLV, QCV, 4> : k_local<MRV, CPLV, QCV, 12>
+    if (MR == 8) { if (q <= 16) WR_LOCAL(8, 1, 16); else if (q <= 32) WR_LOCAL(8, 1, 32); else WR_LOCAL(8, 2, 40); }
+    else if (MR == 16) { if (q <= 32) WR_LOCAL(16, 1, 32); else WR_LOCAL(16, 2, 48); }
+    else { if (q <= 32) WR_LOCAL(32, 1, 32); else WR_LOCAL(32, 2, 64); }
+#undef WR_LOCAL
     WR_CUDA(cudaFuncSetAttribute(kloc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
-    WR_CUDA(cudaFuncSetAttribute(kapp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
-    WR_CUDA(cudaFuncSetAttribute(kapp_w, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
 
     uint32_t *Pcur = d_P, *Pnext = P2.as<uint32_t>();
     int64_t Dbound = 1;
@@ -1569,15 +1143,18 @@ static wr_status mbasis_run(wr_ctx *ctx, const uint32_t *d_S, int64_t L, int m, 
             }
         }
         // a sequence still in flight: the window reads S rows below k0 + bb
-        // rounded up to its order tile
-        if (feed) WR_TRY(feed_wait(ctx, feed, std::min<int64_t>(L, k0 + (bb + WIN_IB - 1) / WIN_IB * WIN_IB)));
+        if (feed) WR_TRY(feed_wait(ctx, feed, std::min<int64_t>(L, k0 + bb)));
         if (prof) WR_CUDA(cudaEventRecord(pe[0], s));
-        // window: split coefficients [0, min(Dbound, k0 + bb - 1)] over the blocks
+        // window: coefficients [0, min(Dbound, k0 + bb - 1)] split over the parts
         const int64_t tspan = std::min<int64_t>(Dbound, k0 + bb - 1) + 1;
-        const int nparts = (int)std::min<int64_t>(nparts_max, std::max<int64_t>(1, (tspan + TT - 1) / TT));
-        const int64_t tper = (tspan + nparts - 1) / nparts;
-        (bb == bmax ? kwin : kwin_tail)<<<nparts, WIN_THREADS, window_bytes(TT, bb), s>>>(d_S, L, m, nr, q, Pcur, k0, bb, TT, tper,
-                                                                dmax.as<int>(), Epart.as<uint32_t>(), mp);
+        const int64_t rows = (int64_t)bb * m;
+        const int64_t tper = std::max<int64_t>((tspan + nparts_max - 1) / nparts_max, (TP_K + nr - 1) / nr);
+        const int nparts = (int)((tspan + tper - 1) / tper);
+        {
+            const ToepArgs g{d_S, Pcur, Epart.as<uint32_t>(), rows, L * m, k0, m, nr, q, 0, tspan, tper, rows * q,
+                             dmax.as<int>(), nullptr, nullptr};
+            ktoep<<<dim3((unsigned)((rows + BR - 1) / BR), (unsigned)nparts), TP_THREADS, 0, s>>>(g, mp);
+        }
         WR_LAUNCHED(ctx);
         const uint32_t *Ewin = Epart.as<uint32_t>();
         if (nparts > 1) {
@@ -1593,20 +1170,31 @@ static wr_status mbasis_run(wr_ctx *ctx, const uint32_t *d_S, int64_t L, int m, 
             WR_LAUNCHED(ctx);
         }
         if (prof) WR_CUDA(cudaEventRecord(pe[1], s));
-        kloc<<<1, wide ? LW_THREADS : local_threads(m <= 8 ? 8 : 32, 1), local_need(bb), s>>>(
-            m, n, q, bb, 1, Ewin, qtop.as<uint32_t>(), d_deg, Ml.as<uint32_t>(),
-            degl.as<int32_t>(), dmax.as<int>(), scale.as<uint32_t>(), dbase, mp);
+        {
+            cudaLaunchConfig_t lc{};
+            cudaLaunchAttribute at{};
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = (unsigned)CS;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            lc.gridDim = dim3((unsigned)CS);
+            lc.blockDim = dim3((unsigned)lc_threads(MR));
+            lc.dynamicSmemBytes = local_need(bb);
+            lc.stream = s;
+            lc.attrs = &at;
+            lc.numAttrs = 1;
+            WR_CUDA(cudaLaunchKernelEx(&lc, kloc, m, q, bb, Ewin, qtop.as<uint32_t>(), d_deg, Ml.as<uint32_t>(),
+                                       degl.as<int32_t>(), dmax.as<int>(), scale.as<uint32_t>(), dbase, mp));
+        }
         WR_LAUNCHED(ctx);
         if (prof) WR_CUDA(cudaEventRecord(pe[2], s));
         if (Dbound + bb > Dcap + 1) return fail(WR_EINVAL, "sigma-basis degree cap too small");
         const int64_t Dnew = std::min<int64_t>(Dbound + bb, Dcap);
-        if (wide)
-            kapp_w<<<dim3((unsigned)((Dnew + TA) / TA), (unsigned)((nr + APW_RB - 1) / APW_RB)), APP_THREADS,
-                     apply_need(TA, bb), s>>>(Pcur, Pnext, nr, q, Ml.as<uint32_t>(), degl.as<int32_t>(), bb, Dnew,
-                                              dmax.as<int>(), mp);
-        else
-            kapp<<<(unsigned)((Dnew + TA) / TA), APP_THREADS, apply_bytes(TA, bb), s>>>(
-                Pcur, Pnext, nr, q, Ml.as<uint32_t>(), degl.as<int32_t>(), bb, Dnew, TA, dmax.as<int>(), mp);
+        {
+            const int64_t prow = (Dnew + 1) * nr;
+            const ToepArgs g{Pcur, Ml.as<uint32_t>(), Pnext, prow, prow, 0, nr, q, q, 0, bb + 1, bb + 1, 0,
+                             nullptr, dmax.as<int>(), degl.as<int32_t>()};
+            ktoep<<<dim3((unsigned)((prow + BR - 1) / BR)), TP_THREADS, 0, s>>>(g, mp);
+        }
         WR_LAUNCHED(ctx);
         if (prof) {
             WR_CUDA(cudaEventRecord(pe[3], s));
