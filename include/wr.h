@@ -135,8 +135,8 @@ wr_status wr_set_sigma_chunk(wr_ctx *ctx, int32_t orders);
  * of the halves' bases done as polynomial matrix products by number-theoretic
  * transforms over three FFT primes and the CRT.  The result is the same basis
  * bit for bit; a leaf as large as the sequence turns PM-Basis off.  0
- * (default) = automatic: PM-Basis with 8,192-order leaves for sequences longer
- * than 131,072 orders when m + n <= 32, with 256-order leaves for sequences
+ * (default) = automatic: PM-Basis with 4,096-order leaves for sequences longer
+ * than 16,384 orders when m + n <= 32, with 256-order leaves for sequences
  * longer than 1,024 orders when m + n > 32, the blocked M-Basis otherwise.
  * With the pipeline (wr_set_pipeline) PM-Basis trails the sequence in
  * segments, each about half of the orders still to come but at most a
@@ -152,9 +152,9 @@ wr_status wr_set_sigma_leaf(wr_ctx *ctx, int64_t orders);
  * entries and the output rows are loaded and stored evict-first, so that L2
  * keeps rows of the gathered block).
  * With autotuning on (default), the first sequence or black-box application
- * on a matrix with at least 2^20 stored entries times each candidate (every
- * lane width, with and without the hints) on that matrix's two layouts (a few
- * launches each, CUDA events) and keeps the
+ * on a matrix with at least 2^20 stored entries times the candidates (2, 4 and 8
+ * residues, the fastest of them with the hints) on that matrix's two layouts (a
+ * few launches each, CUDA events) and keeps the
  * fastest, per matrix, layout and block width; smaller matrices and autotune
  * off use the default (2 residues for n <= 4, 4 above).  wr_set_lane_width
  * forces one (0 = tuned or default).  Results never depend on it. */

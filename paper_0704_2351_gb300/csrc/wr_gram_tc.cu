@@ -129,16 +129,17 @@ __device__ __forceinline__ void put_digits(unsigned char *tile, const uint32_t (
 // polls, and the issuer then lets the copies and MMAs in flight finish.
 template <int NB, int RB>
 __global__ void __launch_bounds__(GT_THREADS, 2)
-    k_gram_tc(int64_t N, int m, int n, const uint32_t *__restrict__ w, const uint32_t *__restrict__ t, int yoff,
-              unsigned long long *__restrict__ s_raw, const int *__restrict__ term_counter, int tmul, int toff,
-              int64_t L, ModP mp, int *__restrict__ err) {
+    k_gram_tc(const __grid_constant__ GramItems items, int m, int n, int yoff, const int *__restrict__ term_counter,
+              int tmul, int64_t L, int *__restrict__ err) {
     using S = GramShape<NB, RB>;
+    const GramItem &it = items.item[blockIdx.y];
+    const int64_t N = it.rows;
+    const uint32_t *__restrict__ w = it.w, *__restrict__ t = it.t;
+    const ModP mp = it.mp;
+    pdl_launch();
     constexpr int RW = RB / 4;      // residues per raw row
     constexpr int HB = NB / 2;      // right-factor columns a draining thread holds
     constexpr uint32_t IDESC = tc::idesc_f16_f32(128, S::TN);
-    const int64_t k_term = term_counter ? (int64_t)tmul * *term_counter + toff : (int64_t)toff;
-    if (k_term < 0 || k_term >= L) return;  // the same for every block
-
     extern __shared__ unsigned char gsm[];
     unsigned char *base = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(gsm) + 1023) & ~uintptr_t(1023));
     unsigned char *raw = base + 2 * S::OPB;
@@ -156,6 +157,7 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
     const int64_t t_begin = tiles * blockIdx.x / gridDim.x;
     const int64_t ntile = tiles * (blockIdx.x + 1) / gridDim.x - t_begin;
 
+    // (everything up to pdl_wait overlaps the pass before)
     // both operand stages start at zero: digit rows of absent columns stay zero
     for (uint32_t i = (uint32_t)tid * 16u; i < 2u * S::OPB; i += GT_THREADS * 16u)
         *reinterpret_cast<uint4 *>(base + i) = make_uint4(0u, 0u, 0u, 0u);
@@ -178,6 +180,12 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_wait();
+    const int64_t k_term = term_counter ? (int64_t)tmul * *term_counter + it.toff : (int64_t)it.toff;
+    if (k_term < 0 || k_term >= L) {  // the same for every block of the item
+        if (warp == 0) tc::tmem_dealloc(tmem, S::TMEM_COLS);
+        return;
+    }
 
     int64_t issued = 0, committed = 0;  // (issuer) raw tiles requested, MMA commits
     auto issue = [&](int64_t tl) {
@@ -341,7 +349,7 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
             for (int b = 0; b < HB; b++) red[(i * 32 + lane) * NB + hf * HB + b] = mulm(red_s64(acc[b], mp), sc, mp);
         }
         __syncthreads();
-        unsigned long long *dst = s_raw + (size_t)k_term * m * n;
+        unsigned long long *dst = it.s_raw + (size_t)k_term * m * n;
         for (int e = tid; e < m * n; e += GT_THREADS) {
             const int a = e / n, b = e % n;
             unsigned long long v = 0;
@@ -360,9 +368,8 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
 }
 
 template <int NB, int RB>
-wr_status launch_gram_tc_t(wr_ctx *ctx, int64_t N, int m, int n, const uint32_t *w, const uint32_t *t, int yoff,
-                           unsigned long long *s_raw, const int *term_counter, int tmul, int toff, int64_t L,
-                           const ModP &mp, int *err) {
+wr_status launch_gram_tc_t(wr_ctx *ctx, const GramItems &items, int count, int m, int n, int yoff,
+                           const int *term_counter, int tmul, int64_t L, int *err) {
     using S = GramShape<NB, RB>;
     static std::once_flag once[8];
     static cudaError_t attr_err[8];
@@ -372,11 +379,14 @@ wr_status launch_gram_tc_t(wr_ctx *ctx, int64_t N, int m, int n, const uint32_t 
                                              (int)S::SMEM);
     });
     WR_CUDA(attr_err[dev]);
-    const int64_t tiles = (N + GT_KT - 1) / GT_KT;
-    const unsigned grid = (unsigned)std::min<int64_t>(tiles, 2 * (int64_t)ctx->num_sms);  // two blocks a SM
+    int64_t rows = 0;
+    for (int i = 0; i < count; i++) rows = max64(rows, items.item[i].rows);
+    const int64_t tiles = (rows + GT_KT - 1) / GT_KT;
+    // two blocks a SM over all items, all resident at once
+    const unsigned grid = (unsigned)std::min<int64_t>(tiles, std::max(1, 2 * ctx->num_sms / count));
     if (grid == 0) return WR_OK;
-    k_gram_tc<NB, RB><<<grid, GT_THREADS, S::SMEM, ctx->stream>>>(N, m, n, w, t, yoff, s_raw, term_counter, tmul,
-                                                                  toff, L, mp, err);
+    launch_dep(ctx, k_gram_tc<NB, RB>, dim3(grid, (unsigned)count), dim3(GT_THREADS), S::SMEM, items, m, n, yoff,
+               term_counter, tmul, L, err);
     WR_LAUNCHED(ctx);
     return WR_OK;
 }
@@ -466,16 +476,14 @@ bool gram_tc_supported(int m, int n, int tstride, int yoff) {
     return true;
 }
 
-wr_status launch_gram_tc(wr_ctx *ctx, int64_t N, int m, int n, const uint32_t *w, const uint32_t *t, int tstride,
-                         int yoff, unsigned long long *s_raw, const int *term_counter, int tmul, int toff, int64_t L,
-                         const ModP &mp, int *err) {
+wr_status launch_gram_tc(wr_ctx *ctx, const GramItems &items, int count, int m, int n, int tstride, int yoff,
+                         const int *term_counter, int tmul, int64_t L, int *err) {
     if (!gram_tc_supported(m, n, tstride, yoff)) return fail(WR_EINVAL, "tensor-core Gram: unsupported shape");
-    if (N <= 0) return WR_OK;
     const int rb = 4 * tstride;
     const int nb = n <= 8 ? 8 : (n <= 16 ? 16 : 32);
-#define WR_GT(NBV, RBV)                                                                                        \
-    if (nb == NBV && rb == RBV)                                                                                \
-        return launch_gram_tc_t<NBV, RBV>(ctx, N, m, n, w, t, yoff, s_raw, term_counter, tmul, toff, L, mp, err);
+#define WR_GT(NBV, RBV)          \
+    if (nb == NBV && rb == RBV) \
+        return launch_gram_tc_t<NBV, RBV>(ctx, items, count, m, n, yoff, term_counter, tmul, L, err);
     WR_GT(8, 32)
     WR_GT(8, 64)
     WR_GT(16, 64)

@@ -107,6 +107,14 @@ __host__ __device__ __forceinline__ uint32_t red64(uint64_t x, const ModP &m) {
 }
 
 #ifdef __CUDACC__
+// Programmatic dependent launch (launch_dep): a kernel lets the next one of its
+// stream start as soon as all its blocks run (pdl_launch), and touches what earlier
+// kernels read or write only after pdl_wait (which returns once the kernel before
+// has completed and its writes are visible; at once in a plain launch).  Before it,
+// kernels read the matrix layouts only.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // d = a b + c in one 32x32 -> 64-bit multiply-add
 __device__ __forceinline__ unsigned long long madw(uint32_t a, uint32_t b, unsigned long long c) {
     unsigned long long d;
@@ -410,6 +418,7 @@ struct wr_ctx {
     int pipeline = 1;       // wr_rank: the sigma-basis trails the sequence on a second stream
                             // (0 off, 1 automatic priority, 2 the sigma-basis's stream first,
                             // 3 the sequence's first)
+    bool dep_launch = false;    // launch_dep: programmatic dependent launches (set by DepScope)
     bool high_priority = false; // this context's own stream has the greatest priority
     bool seq_high = false;      // seq_stream has the greatest priority
     int64_t early_term = 0; // quiet orders that end the sequence early (0: the full L terms)
@@ -466,6 +475,35 @@ struct wr_result {
 namespace wr {
 
 wr_status dev_alloc(wr_ctx *ctx, DevBuf &b, size_t bytes);
+
+// Within a scope the kernels launched by launch_dep may start while the one before
+// them on the context's stream drains; every such kernel calls pdl_wait before it
+// touches data.
+struct DepScope {
+    wr_ctx *ctx;
+    bool keep;
+    DepScope(wr_ctx *c, bool on) : ctx(c), keep(c->dep_launch) { c->dep_launch = on; }
+    ~DepScope() { ctx->dep_launch = keep; }
+    DepScope(const DepScope &) = delete;
+    DepScope &operator=(const DepScope &) = delete;
+};
+
+#ifdef __CUDACC__
+template <class... K, class... A>
+inline void launch_dep(wr_ctx *ctx, void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, A... args) {
+    cudaLaunchConfig_t lc{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    lc.gridDim = grid;
+    lc.blockDim = block;
+    lc.dynamicSmemBytes = smem;
+    lc.stream = ctx->stream;
+    lc.attrs = &at;
+    lc.numAttrs = ctx->dep_launch ? 1 : 0;
+    cudaLaunchKernelEx(&lc, kernel, K(args)...);  // (WR_LAUNCHED checks cudaGetLastError)
+}
+#endif
 
 // chain reduction (wr_reduce.cu): the reduced CSR, its rows' and columns'
 // indices in the input, and the number of unit pivots taken
@@ -538,12 +576,24 @@ bool sigma_uses_pm(const wr_ctx *ctx, int64_t L, int m, int n, bool early = fals
 void copy_settings(const wr_ctx *parent, wr_ctx *child);
 wr_status blackbox_apply(wr_ctx *ctx, const wr_matrix *mat, const wr_params &prm,
                          const uint32_t *d_in, uint32_t *d_out, int64_t width);
-// tensor-core Gram products (wr_gram_tc.cu): S_raw[k] += sum_r w_r t[r][0..m)^T
-// t[r][yoff..yoff+n) mod p, w in Montgomery form, k = tmul * counter + toff
+// Gram products of one launch: item y adds sum_r w_r t[r][0..m)^T t[r][yoff..yoff+n)
+// mod p over its rows (w in Montgomery form) to s_raw[k], k = tmul * counter + toff
+// (skipped unless 0 <= k < L).
+constexpr int GRAM_MAX_ITEMS = 2 * 4;  // both sides of an application for up to MULTI_MAX_JOBS jobs
+struct GramItem {
+    int64_t rows;
+    const uint32_t *w, *t;
+    unsigned long long *s_raw;
+    int toff;
+    ModP mp;
+};
+struct GramItems {
+    GramItem item[GRAM_MAX_ITEMS];
+};
+// on the tensor cores (wr_gram_tc.cu)
 bool gram_tc_supported(int m, int n, int tstride, int yoff);
-wr_status launch_gram_tc(wr_ctx *ctx, int64_t N, int m, int n, const uint32_t *w, const uint32_t *t, int tstride,
-                         int yoff, unsigned long long *s_raw, const int *term_counter, int tmul, int toff, int64_t L,
-                         const ModP &mp, int *err);
+wr_status launch_gram_tc(wr_ctx *ctx, const GramItems &items, int count, int m, int n, int tstride, int yoff,
+                         const int *term_counter, int tmul, int64_t L, int *err);
 wr_status probe_mma(wr_ctx *ctx, int64_t iters, int blocks, float *d_out, double *ms);
 wr_status gram_device(wr_ctx *ctx, uint32_t p, int64_t N, int m, int n, const uint32_t *t, int tstride, int yoff,
                       const uint32_t *w, uint32_t *G);

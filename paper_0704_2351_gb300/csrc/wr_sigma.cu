@@ -251,16 +251,20 @@ __global__ void __launch_bounds__(256)
 inline int sigma_chunk_default(int q) {
     return q <= 16 ? 64 : (q <= 32 ? 32 : 16);
 }
-// PM-Basis by default only for sequences longer than SIGMA_PM_MIN_L (q <= 32),
-// with leaves of SIGMA_LEAF_DEFAULT orders: the M-Basis trails a sequence chunk by
-// chunk, PM-Basis in segments.  For q > 32 the window and product passes over the
-// basis cost more per order, so PM-Basis with short leaves takes over early: at q =
+// PM-Basis by default for sequences longer than SIGMA_PM_MIN_L (q <= 32), with
+// leaves of SIGMA_LEAF_DEFAULT orders: the M-Basis's window and product passes grow
+// with the square of the length (11,252 orders at q = 16: 53 ms, 57 with 2,048-order
+// leaves; 45,002 orders: 387 ms, 198 / 201 / 221 with leaves of 2,048 / 4,096 /
+// 8,192), and trailing a sequence they take its SMs (the rank of the 200,000 x
+// 180,000 matrix: 1,777 ms with the M-Basis chunk by chunk, 1,622 / 1,607 in
+// PM-Basis segments with 2,048- / 4,096-order leaves).  For q > 32 those passes
+// cost more per order, so PM-Basis with short leaves takes over early: at q =
 // 64, 4,098 orders, 125 / 122 / 132 ms for leaves of 128 / 256 / 512 orders, and
 // against the M-Basis alone 16.8 / 15.8 ms at 600 orders, 27.8 / 29.3 at 1,000,
 // 42.3 / 49.5 at 1,500, 58.5 / 75.5 at 2,040.  wr_set_sigma_leaf chooses the leaf
 // explicitly.
-constexpr int64_t SIGMA_LEAF_DEFAULT = 8192;
-constexpr int64_t SIGMA_PM_MIN_L = 131072;
+constexpr int64_t SIGMA_LEAF_DEFAULT = 4096;
+constexpr int64_t SIGMA_PM_MIN_L = 16384;
 constexpr int64_t SIGMA_LEAF_WIDE = 256;
 constexpr int64_t SIGMA_PM_MIN_L_WIDE = 1024;
 constexpr int BAR_T0 = 1, BAR_E = 3;  // named barriers BAR_T0 + (i & 1), BAR_E

@@ -37,12 +37,23 @@ namespace {
 // the paired block [D1 X | D1 Y]).
 constexpr int PROJ_THREADS = 256;
 
+// One launch does the products of several items (blockIdx.y): both sides of an
+// application, of all jobs of a fused batch.  For small matrices the products of a
+// launch cost mostly its latency: eight of 4.7 us each (5,000 rows, four jobs)
+// took 37 of 49 us an application before; the batch of four primes on 6,000 x 5,000
+// 32.4 -> 16.5 ms.
 template <int NV, int FOLDK, bool GRAM>
 __global__ void __launch_bounds__(PROJ_THREADS)
-    k_project(int64_t N, int m, int n, const uint32_t *__restrict__ xh, const uint32_t *__restrict__ t,
-              unsigned long long *__restrict__ s_raw, const int *__restrict__ term_counter, int tmul, int toff,
-              int64_t L, int tstride, int yoff, ModP mp) {
-    const int64_t k_term = (int64_t)tmul * *term_counter + toff;
+    k_project(const __grid_constant__ GramItems items, int m, int n, const int *__restrict__ term_counter, int tmul,
+              int64_t L, int tstride, int yoff) {
+    const GramItem &it = items.item[blockIdx.y];
+    const int64_t N = it.rows;
+    const uint32_t *__restrict__ xh = it.w, *__restrict__ t = it.t;
+    unsigned long long *__restrict__ s_raw = it.s_raw;
+    const ModP mp = it.mp;
+    pdl_launch();
+    pdl_wait();
+    const int64_t k_term = (int64_t)tmul * *term_counter + it.toff;
     if (k_term < 0 || k_term >= L) return;  // the same for every thread
     // red32[w][a][b]: per-warp sums reduced mod p (m divides 32); red: one
     // shared row of atomically added sums (other m)
@@ -148,6 +159,8 @@ __global__ void k_reduce_seq(int64_t count, const unsigned long long *__restrict
 // permutation of A~'s rows and columns, X and Y)
 __global__ void k_derive_diag(uint64_t seed, uint64_t tag, int64_t len, uint32_t p,
                               uint32_t *__restrict__ out, const uint32_t *__restrict__ map) {
+    pdl_launch();
+    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < len) {
         const uint64_t gi = map ? (uint64_t)map[i] : (uint64_t)i;
@@ -163,6 +176,8 @@ __global__ void k_prepare(int64_t N, int m, int n, int nv, uint64_t seed, uint64
                           int ycol0, int gram, int paired, const uint32_t *__restrict__ d1, uint32_t *__restrict__ t0,
                           uint32_t *__restrict__ xh, uint32_t *__restrict__ d1sq, const uint32_t *__restrict__ nmap,
                           ModP mp, int trow) {
+    pdl_launch();
+    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const uint64_t gi = nmap ? (uint64_t)nmap[i] : (uint64_t)i;  // index of the draws
@@ -198,8 +213,43 @@ __global__ void k_prepare(int64_t N, int m, int n, int nv, uint64_t seed, uint64
 // out = d^{-1} R mod p, elementwise (the Gram weights D2^{-1} of the odd terms of
 // the symmetric projection: S_2k+1 = W^T D2^{-1} W with W = D2 A D1 V_k)
 __global__ void k_inv_diag(int64_t len, const uint32_t *__restrict__ d, uint32_t *__restrict__ out, ModP mp) {
+    pdl_launch();
+    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < len) out[i] = to_mont(invm(d[i], mp), mp);  // Montgomery form for the Gram projection
+}
+
+// One black-box application's set-up in one launch: D1, D2 drawn, out (N x nv,
+// padded) = D1 in (N x width).  Blocks [0, nblocks) take AS_ROWS rows of N each (a
+// row's draw once, through shared memory), the others AS_ROWS of M.  (in: as in
+// k_scale_pad)
+constexpr int AS_ROWS = 64, AS_THREADS = 256;
+__global__ void __launch_bounds__(AS_THREADS)
+    k_apply_setup(uint64_t seed, int64_t N, int64_t M, unsigned nblocks, int width, int nv,
+                  const uint32_t *__restrict__ in, uint32_t *__restrict__ d1, uint32_t *__restrict__ d2,
+                  uint32_t *__restrict__ out, const uint32_t *__restrict__ nmap, const uint32_t *__restrict__ mmap,
+                  ModP mp) {
+    __shared__ uint32_t ds[AS_ROWS];
+    pdl_launch();
+    pdl_wait();
+    const bool nside = blockIdx.x < nblocks;
+    const int64_t r0 = (int64_t)(nside ? blockIdx.x : blockIdx.x - nblocks) * AS_ROWS;
+    const int rows = (int)min64(AS_ROWS, (nside ? N : M) - r0);
+    const uint32_t *map = nside ? nmap : mmap;
+    if (threadIdx.x < rows) {
+        const int64_t r = r0 + threadIdx.x;
+        const uint64_t g = map ? (uint64_t)map[r] : (uint64_t)r;
+        const uint32_t d = (uint32_t)(1 + stream_hash(seed, nside ? TAG_D1 : TAG_D2, g) % (uint64_t)(mp.p - 1));
+        (nside ? d1 : d2)[r] = d;
+        ds[threadIdx.x] = d;
+    }
+    if (!nside) return;
+    __syncthreads();
+    for (int x = threadIdx.x; x < rows * nv; x += AS_THREADS) {
+        const int rl = x / nv, b = x % nv;
+        const int64_t r = r0 + rl, g = nmap ? (int64_t)nmap[r] : r;
+        out[r * nv + b] = b < width ? mulm(ds[rl], in[g * width + b], mp) : 0;
+    }
 }
 
 // out (N x nv, padded) = D1 in (N x width)
@@ -208,6 +258,8 @@ __global__ void k_inv_diag(int64_t len, const uint32_t *__restrict__ d, uint32_t
 __global__ void k_scale_pad(int64_t N, int width, int nv, const uint32_t *__restrict__ in,
                             const uint32_t *__restrict__ d1, uint32_t *__restrict__ out,
                             const uint32_t *__restrict__ nmap, ModP mp) {
+    pdl_launch();
+    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N * nv) return;
     int64_t r = i / nv;
@@ -218,6 +270,8 @@ __global__ void k_scale_pad(int64_t N, int width, int nv, const uint32_t *__rest
 
 __global__ void k_unpad(int64_t N, int width, int nv, const uint32_t *__restrict__ in,
                         uint32_t *__restrict__ out, const uint32_t *__restrict__ nmap) {
+    pdl_launch();
+    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N * width) return;
     int64_t r = i / width;
@@ -261,8 +315,8 @@ void launch_spmm_kernel(wr_ctx *ctx, const SellView &A, const uint32_t *x, uint3
     if (blocks <= 0) return;
     const MultiEpi one{};
 #define WR_SPMM_LAUNCH(WIDEV, CSV, MULTIV)                                                                     \
-    k_spmm<NV, WL, WIDEV, CSV, MULTIV><<<(unsigned)blocks, 32 * SPMM_WARPS, 0, ctx->stream>>>(                 \
-        A, x, y, scale, acc64, mp, term_counter, vblocks, pieces, me ? *me : one, part)
+    launch_dep(ctx, k_spmm<NV, WL, WIDEV, CSV, MULTIV>, dim3((unsigned)blocks), dim3(32 * SPMM_WARPS), 0, A, x, y, scale, \
+               acc64, mp, term_counter, vblocks, pieces, me ? *me : one, part)
     if constexpr (NV >= 16) {
         if (me && me->jobs > 1) {
             if (A.wvals) {
@@ -305,11 +359,11 @@ wr_status launch_spmm_t(wr_ctx *ctx, const SellView &A, const uint32_t *x, uint3
     if (finalize && A.nsplit > 0) {
         int64_t cnt = A.nsplit * NV;
         if (me && me->jobs > 1)
-            k_finalize_split_multi<<<blocks_for(cnt, 256), 256, 0, ctx->stream>>>(A.nsplit, NV, A.split_row, acc64,
-                                                                                 y, *me);
+            launch_dep(ctx, k_finalize_split_multi, dim3(blocks_for(cnt, 256)), dim3(256), 0, A.nsplit, NV, A.split_row,
+                       acc64, y, *me);
         else
-            k_finalize_split<<<blocks_for(cnt, 256), 256, 0, ctx->stream>>>(A.nsplit, NV, A.split_row, acc64,
-                                                                           y, scale, mp, part);
+            launch_dep(ctx, k_finalize_split, dim3(blocks_for(cnt, 256)), dim3(256), 0, A.nsplit, NV, A.split_row, acc64,
+                       y, scale, mp, part);
         WR_LAUNCHED(ctx);
     }
     return WR_OK;
@@ -339,8 +393,7 @@ wr_status launch_spmm(wr_ctx *ctx, int nv, const SellView &A, const uint32_t *x,
     }
 }
 
-// Lane-width tuner: times the candidate residues-per-lane (1, 2, 4, 8; at
-// most 32 lanes per gathered row) of one SpMM layout on the matrix itself (zero block: the gather addresses, which
+// Lane-width tuner: times the candidate residues-per-lane of one SpMM layout on the matrix itself (zero block: the gather addresses, which
 // set the time, do not depend on the values) and keeps the fastest.  The
 // result never depends on the choice.
 int nv_index(int nv) {
@@ -366,29 +419,33 @@ static wr_status tune_lane_width(wr_ctx *ctx, const Sell &S, int nv, int *out) {
     cudaEvent_t e0, e1;
     WR_CUDA(cudaEventCreate(&e0));
     WR_CUDA(cudaEventCreate(&e1));
+    // one warm-up and three timed launches a candidate: 2, 4 and 8 residues a lane,
+    // then the streaming hints with the best of them.  (1 residue a lane was slowest
+    // on every matrix measured, by a third and more.)
     float best = 0.0f;
-    for (int cs : {0, SPMM_CS})
-        for (int wl : {1, 2, 4, 8}) {
-            if (wl > nv || nv % wl != 0 || nv / wl > 32) continue;
-            for (int w = 0; w < 2; w++)
-                WR_TRY(launch_spmm(ctx, nv, v, x.as<uint32_t>(), y.as<uint32_t>(), scale.as<uint32_t>(),
-                                   acc.as<unsigned long long>(), mp, nullptr, wl | cs, false));
-            WR_CUDA(cudaEventRecord(e0, s));
-            for (int r = 0; r < 5; r++)
-                WR_TRY(launch_spmm(ctx, nv, v, x.as<uint32_t>(), y.as<uint32_t>(), scale.as<uint32_t>(),
-                                   acc.as<unsigned long long>(), mp, nullptr, wl | cs, false));
-            WR_CUDA(cudaEventRecord(e1, s));
-            WR_CUDA(cudaEventSynchronize(e1));
-            float ms = 0.0f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (best == 0.0f || ms < best) {
-                best = ms;
-                *out = wl | cs;
-            }
+    auto time_one = [&](int variant) -> wr_status {
+        for (int k = 0; k < 4; k++) {
+            if (k == 1) WR_CUDA(cudaEventRecord(e0, s));
+            WR_TRY(launch_spmm(ctx, nv, v, x.as<uint32_t>(), y.as<uint32_t>(), scale.as<uint32_t>(),
+                               acc.as<unsigned long long>(), mp, nullptr, variant, false));
         }
+        WR_CUDA(cudaEventRecord(e1, s));
+        WR_CUDA(cudaEventSynchronize(e1));
+        float ms = 0.0f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (best == 0.0f || ms < best) {
+            best = ms;
+            *out = variant;
+        }
+        return WR_OK;
+    };
+    wr_status tst = WR_OK;
+    for (int wl : {1, 2, 4, 8})
+        if (tst == WR_OK && wl <= nv && (wl > 1 || nv == 1)) tst = time_one(wl);
+    if (tst == WR_OK) tst = time_one(*out | SPMM_CS);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    return WR_OK;
+    return tst;
 }
 
 // the lane width for a layout: forced by the context, else tuned once per
@@ -430,33 +487,28 @@ wr_status spmm_variant_for(wr_ctx *ctx, const wr_matrix *mat, const Sell &S, int
 namespace {
 
 template <int NV, bool GRAM>
-void launch_project_t(wr_ctx *ctx, unsigned grid, int64_t N, int m, int n, const uint32_t *xh,
-                      const uint32_t *t, unsigned long long *s_raw, const int *term_counter, int tmul, int toff,
-                      int64_t L, int tstride, int yoff, const ModP &mp) {
+void launch_project_t(wr_ctx *ctx, dim3 grid, const GramItems &items, int count, int m, int n, const int *term_counter,
+                      int tmul, int64_t L, int tstride, int yoff) {
     if (tstride <= 0) tstride = NV;
-    if (mp.lazy >= 16)  // p < 2^30
-        k_project<NV, 14, GRAM><<<grid, PROJ_THREADS, 0, ctx->stream>>>(N, m, n, xh, t, s_raw, term_counter, tmul,
-                                                                         toff, L, tstride, yoff, mp);
-    else
-        k_project<NV, 2, GRAM><<<grid, PROJ_THREADS, 0, ctx->stream>>>(N, m, n, xh, t, s_raw, term_counter, tmul,
-                                                                        toff, L, tstride, yoff, mp);
+    bool small = true;  // p < 2^30 for every item: sums folded every 14 products, else every 2
+    for (int i = 0; i < count; i++) small = small && items.item[i].mp.lazy >= 16;
+    launch_dep(ctx, small ? k_project<NV, 14, GRAM> : k_project<NV, 2, GRAM>, grid, dim3(PROJ_THREADS), 0, items, m, n,
+               term_counter, tmul, L, tstride, yoff);
 }
 
-// gram = false: S_raw[k] += xh^T t (xh: N x m).  gram = true: S_raw[k] +=
-// sum_r xh[r] t[r]^T t[r] (xh: N weights, m = n).  k = tmul * counter + toff.
-wr_status launch_project(wr_ctx *ctx, int64_t N, int m, int n, int nv, const uint32_t *xh,
-                         const uint32_t *t, unsigned long long *s_raw, const int *term_counter,
-                         const ModP &mp, bool gram = false, int tmul = 1, int toff = 0,
-                         int64_t L = INT64_MAX, int tstride = 0, int yoff = 0) {
+// Per item, gram = false: S_raw[k] += w^T t (w: rows x m).  gram = true: S_raw[k] +=
+// sum_r w[r] t[r]^T t[r] (w: one weight a row).  k = tmul * counter + toff.
+wr_status launch_project(wr_ctx *ctx, const GramItems &items, int count, int m, int n, int nv, const int *term_counter,
+                         bool gram, int tmul, int64_t L, int tstride, int yoff) {
     const int per = PROJ_THREADS / m;
-    const int64_t need = std::max<int64_t>((N + per - 1) / per, 1);
-    const unsigned grid = (unsigned)std::min<int64_t>(need, (int64_t)ctx->num_sms * 2);
-#define WR_PROJ_CASE(NVV)                                                                                    \
-    case NVV:                                                                                                \
-        if (gram)                                                                                            \
-            launch_project_t<NVV, true>(ctx, grid, N, m, n, xh, t, s_raw, term_counter, tmul, toff, L, tstride, yoff, mp); \
-        else                                                                                                 \
-            launch_project_t<NVV, false>(ctx, grid, N, m, n, xh, t, s_raw, term_counter, tmul, toff, L, tstride, yoff, mp); \
+    int64_t rows = 0;
+    for (int i = 0; i < count; i++) rows = std::max<int64_t>(rows, items.item[i].rows);
+    const int64_t need = std::max<int64_t>((rows + per - 1) / per, 1);
+    const dim3 grid((unsigned)std::min<int64_t>(need, std::max(1, 4 * ctx->num_sms / count)), (unsigned)count);
+#define WR_PROJ_CASE(NVV)                                                                                     \
+    case NVV:                                                                                                 \
+        if (gram) launch_project_t<NVV, true>(ctx, grid, items, count, m, n, term_counter, tmul, L, tstride, yoff); \
+        else launch_project_t<NVV, false>(ctx, grid, items, count, m, n, term_counter, tmul, L, tstride, yoff);     \
         break;
     switch (nv) {
         WR_PROJ_CASE(1)
@@ -582,22 +634,30 @@ static bool use_tc_gram(const wr_ctx *ctx, int m, int n, int tstride, int yoff) 
     return ctx->tensor_proj == 1 || (m >= 16 && n >= 16);
 }
 
-static wr_status launch_gram_to(wr_ctx *ctx, const Resolved &r, const ModP &mp, int64_t rows, const uint32_t *w,
-                                const uint32_t *t, int tmul, int toff, int tstride, int yoff,
-                                unsigned long long *s_raw, const int *counter, int *err) {
+static wr_status launch_grams(wr_ctx *ctx, const Resolved &r, const GramItems &items, int count, int tmul, int tstride,
+                              int yoff, const int *counter, int *err) {
     if (use_tc_gram(ctx, r.m, r.n, tstride, yoff))
-        return launch_gram_tc(ctx, rows, r.m, r.n, w, t, tstride, yoff, s_raw, counter, tmul, toff, r.L, mp, err);
-    return launch_project(ctx, rows, r.m, r.n, r.nv, w, t, s_raw, counter, mp, true, tmul, toff, r.L, tstride, yoff);
+        return launch_gram_tc(ctx, items, count, r.m, r.n, tstride, yoff, counter, tmul, r.L, err);
+    return launch_project(ctx, items, count, r.m, r.n, r.nv, counter, true, tmul, r.L, tstride, yoff);
 }
 
+// one Gram projection of a sequence's state
 static wr_status launch_gram(wr_ctx *ctx, SeqState &st, int64_t rows, const uint32_t *w, const uint32_t *t,
                              int tmul, int toff, int tstride, int yoff, const int *counter = nullptr) {
-    return launch_gram_to(ctx, st.r, st.mp, rows, w, t, tmul, toff, tstride, yoff, st.s_raw.as<unsigned long long>(),
-                          counter ? counter : st.counter.as<int>(), st.err.as<int>());
+    if (rows <= 0) return WR_OK;
+    GramItems g{};
+    g.item[0] = GramItem{rows, w, t, st.s_raw.as<unsigned long long>(), toff, st.mp};
+    return launch_grams(ctx, st.r, g, 1, tmul, tstride, yoff, counter ? counter : st.counter.as<int>(), st.err.as<int>());
 }
 
-static wr_status seq_setup(wr_ctx *ctx, const wr_matrix *mat, const Resolved &r, SeqState &st,
-                           bool want_projection) {
+// S_raw[counter + 0] += Xh^T T (the generic projection, one term per application)
+static wr_status launch_generic(wr_ctx *ctx, SeqState &st, int64_t L) {
+    GramItems g{};
+    g.item[0] = GramItem{st.r.N, st.xh.as<uint32_t>(), st.T.as<uint32_t>(), st.s_raw.as<unsigned long long>(), 0, st.mp};
+    return launch_project(ctx, g, 1, st.r.m, st.r.n, st.r.nv, st.counter.as<int>(), false, 1, L, st.r.nvs, 0);
+}
+
+static wr_status seq_setup(wr_ctx *ctx, const wr_matrix *mat, const Resolved &r, SeqState &st) {
     st.r = r;
     st.mp = make_modp(r.p);
     st.first = r.side == 0 ? &mat->a : &mat->at;
@@ -624,7 +684,7 @@ static wr_status seq_setup(wr_ctx *ctx, const wr_matrix *mat, const Resolved &r,
     WR_CUDA(cudaMemsetAsync(st.acc1.ptr, 0, st.acc1.bytes, s));
     WR_CUDA(cudaMemsetAsync(st.acc2.ptr, 0, st.acc2.bytes, s));
     WR_CUDA(cudaMemsetAsync(st.counter.ptr, 0, sizeof(int), s));
-    if (want_projection && ctx->proj_overlap && (r.gram || r.paired)) {
+    if (ctx->proj_overlap && (r.gram || r.paired)) {
         int prio = 0;
         WR_CUDA(cudaStreamGetPriority(s, &prio));
         WR_CUDA(cudaStreamCreateWithPriority(&st.side, cudaStreamNonBlocking, prio));
@@ -636,21 +696,23 @@ static wr_status seq_setup(wr_ctx *ctx, const wr_matrix *mat, const Resolved &r,
         WR_LAUNCHED(ctx);
     }
     if (r.N > 0) {
-        k_derive_diag<<<blocks_for(r.N, 256), 256, 0, s>>>(r.seed, TAG_D1, r.N, r.p, st.D1.as<uint32_t>(), r.nmap);
+        launch_dep(ctx, k_derive_diag, dim3(blocks_for(r.N, 256)), dim3(256), 0, r.seed, TAG_D1, r.N, r.p,
+                   st.D1.as<uint32_t>(), r.nmap);
         WR_LAUNCHED(ctx);
     }
     if (r.M > 0) {
-        k_derive_diag<<<blocks_for(r.M, 256), 256, 0, s>>>(r.seed, TAG_D2, r.M, r.p, st.D2.as<uint32_t>(), r.mmap);
+        launch_dep(ctx, k_derive_diag, dim3(blocks_for(r.M, 256)), dim3(256), 0, r.seed, TAG_D2, r.M, r.p,
+                   st.D2.as<uint32_t>(), r.mmap);
         WR_LAUNCHED(ctx);
     }
-    if (want_projection && r.N > 0) {
+    if (r.N > 0) {
         k_prepare<<<blocks_for(r.N, 128), 128, 0, s>>>(r.N, r.m, r.n, r.nv, r.seed, r.xtag, r.xwidth, r.ystride,
                                                       r.ycol0, r.gram ? 1 : 0, r.paired ? 1 : 0, st.D1.as<uint32_t>(),
                                                       st.T.as<uint32_t>(), st.xh.as<uint32_t>(),
                                                       st.d1sq.as<uint32_t>(), r.nmap, st.mp, 0);
         WR_LAUNCHED(ctx);
     }
-    if (want_projection && (r.gram || r.paired) && r.M > 0) {
+    if ((r.gram || r.paired) && r.M > 0) {
         WR_TRY(dev_alloc(ctx, st.w2, sizeof(uint32_t) * r.M));
         k_inv_diag<<<blocks_for(r.M, 256), 256, 0, s>>>(r.M, st.D2.as<uint32_t>(), st.w2.as<uint32_t>(), st.mp);
         WR_LAUNCHED(ctx);
@@ -715,13 +777,13 @@ static wr_status seq_iteration(wr_ctx *ctx, SeqState &st, cudaEvent_t *ev) {
                        st.d1sq.as<uint32_t>(), st.acc2.as<unsigned long long>(), st.mp, nullptr, st.wl2));
     if (ev) WR_CUDA(cudaEventRecord(ev[2], ctx->stream));
     if (st.r.gram || st.r.paired) {
-        const int ts = nv, yo = st.r.paired ? st.r.nv : 0;
-        WR_TRY(launch_gram(ctx, st, st.r.M, st.w2.as<uint32_t>(), st.Wb.as<uint32_t>(), 2, -1, ts, yo));
-        WR_TRY(launch_gram(ctx, st, st.r.N, st.xh.as<uint32_t>(), st.T.as<uint32_t>(), 2, 0, ts, yo));
+        // both Gram products of the application in one launch
+        GramItems g{};
+        g.item[0] = GramItem{st.r.M, st.w2.as<uint32_t>(), st.Wb.as<uint32_t>(), st.s_raw.as<unsigned long long>(), -1, st.mp};
+        g.item[1] = GramItem{st.r.N, st.xh.as<uint32_t>(), st.T.as<uint32_t>(), st.s_raw.as<unsigned long long>(), 0, st.mp};
+        WR_TRY(launch_grams(ctx, st.r, g, 2, 2, nv, st.r.paired ? st.r.nv : 0, st.counter.as<int>(), st.err.as<int>()));
     } else {
-        WR_TRY(launch_project(ctx, st.r.N, st.r.m, st.r.n, nv, st.xh.as<uint32_t>(), st.T.as<uint32_t>(),
-                              st.s_raw.as<unsigned long long>(), st.counter.as<int>(), st.mp, false, 1, 0,
-                              st.r.L));
+        WR_TRY(launch_generic(ctx, st, st.r.L));
     }
     return WR_OK;
 }
@@ -805,7 +867,7 @@ wr_status run_sequence_resolved(wr_ctx *ctx, const wr_matrix *mat, Resolved r, i
     WR_CUDA(cudaEventCreateWithFlags(&e2, cudaEventBlockingSync));  // waited on below, asleep
     WR_CUDA(cudaEventRecord(e0, s));
     SeqState st;
-    WR_TRY(seq_setup(ctx, mat, r, st, true));
+    WR_TRY(seq_setup(ctx, mat, r, st));
     const int64_t E = (int64_t)r.m * r.n;
     WR_TRY(dev_alloc(ctx, st.s_raw, sizeof(unsigned long long) * std::max<int64_t>(L * E, 1)));
     WR_CUDA(cudaMemsetAsync(st.s_raw.ptr, 0, st.s_raw.bytes, s));
@@ -814,9 +876,7 @@ wr_status run_sequence_resolved(wr_ctx *ctx, const wr_matrix *mat, Resolved r, i
             WR_TRY(launch_gram(ctx, st, r.N, st.xh.as<uint32_t>(), st.T.as<uint32_t>(), 2, 0, r.nvs,
                                r.paired ? r.nv : 0));
         else
-            WR_TRY(launch_project(ctx, r.N, r.m, r.n, r.nv, st.xh.as<uint32_t>(), st.T.as<uint32_t>(),
-                                  st.s_raw.as<unsigned long long>(), st.counter.as<int>(), st.mp, false, 1, 0, L,
-                                  r.nvs, 0));
+            WR_TRY(launch_generic(ctx, st, L));
     }
     if (out && out->snap_at == 0) WR_TRY(export_state(ctx, st, out->d_snap));
     int64_t published = 0;
@@ -987,6 +1047,11 @@ wr_status gram_device(wr_ctx *ctx, uint32_t p, int64_t N, int m, int n, const ui
     return WR_OK;
 }
 
+static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
+
+// One application with its temporaries in one allocation.  The kernels start while
+// the one before them drains (DepScope): a 2,000 x 1,800 matrix 47 -> 21 us a
+// call with the launches, allocations and the set-up joined.
 wr_status blackbox_apply(wr_ctx *ctx, const wr_matrix *mat, const wr_params &prm, const uint32_t *d_in,
                          uint32_t *d_out, int64_t width) {
     if (width < 1 || width > 32) return fail(WR_EINVAL, "width must be in 1..32");
@@ -995,23 +1060,43 @@ wr_status blackbox_apply(wr_ctx *ctx, const wr_matrix *mat, const wr_params &prm
     p2.m = 1;
     Resolved r;
     WR_TRY(resolve(mat, &p2, r));
-    SeqState st;
-    WR_TRY(seq_setup(ctx, mat, r, st, false));
+    const Sell &first = r.side == 0 ? mat->a : mat->at, &second = r.side == 0 ? mat->at : mat->a;
+    const int nv = r.nv;
+    const ModP mp = make_modp(r.p);
     cudaStream_t s = ctx->stream;
-    if (r.N > 0) {
-        k_scale_pad<<<blocks_for(r.N * r.nv, 256), 256, 0, s>>>(r.N, (int)width, r.nv, d_in,
-                                                               st.D1.as<uint32_t>(), st.T.as<uint32_t>(), r.nmap,
-                                                               st.mp);
+    int w1 = 0, w2 = 0;
+    const std::vector<Sell> *slabs1 = nullptr, *slabs2 = nullptr;
+    WR_TRY(lane_width_for(ctx, mat, first, nv, &w1));
+    WR_TRY(lane_width_for(ctx, mat, second, nv, &w2));
+    WR_TRY(slabs_for(ctx, mat, first, nv, &slabs1));
+    WR_TRY(slabs_for(ctx, mat, second, nv, &slabs2));
+    // the second pass writes the caller's block itself when its rows are the layout's
+    const bool direct = width == nv && !r.nmap && reinterpret_cast<uintptr_t>(d_out) % 16 == 0;
+    const size_t nT = align256(sizeof(uint32_t) * (size_t)r.N * nv), nW = align256(sizeof(uint32_t) * (size_t)r.M * nv);
+    const size_t nD1 = align256(sizeof(uint32_t) * (size_t)r.N), nD2 = align256(sizeof(uint32_t) * (size_t)r.M);
+    const size_t nA1 = align256(sizeof(unsigned long long) * (size_t)max_split(first, slabs1) * nv);
+    const size_t nA2 = align256(sizeof(unsigned long long) * (size_t)max_split(second, slabs2) * nv);
+    DevBuf ws;
+    WR_TRY(dev_alloc(ctx, ws, nT + nW + nD1 + nD2 + nA1 + nA2 + 256));
+    // (the caller's allocator may align to less)
+    unsigned char *b = reinterpret_cast<unsigned char *>(align256(reinterpret_cast<uintptr_t>(ws.ptr)));
+    uint32_t *T = reinterpret_cast<uint32_t *>(b), *Wb = reinterpret_cast<uint32_t *>(b + nT);
+    uint32_t *D1 = reinterpret_cast<uint32_t *>(b + nT + nW), *D2 = reinterpret_cast<uint32_t *>(b + nT + nW + nD1);
+    unsigned char *acc = b + nT + nW + nD1 + nD2;
+    if (nA1 + nA2) WR_CUDA(cudaMemsetAsync(acc, 0, nA1 + nA2, s));
+    const DepScope dep(ctx, true);
+    const unsigned nb = blocks_for(r.N, AS_ROWS), mb = blocks_for(r.M, AS_ROWS);
+    if (nb + mb > 0) {
+        launch_dep(ctx, k_apply_setup, dim3(nb + mb), dim3(AS_THREADS), 0, r.seed, r.N, r.M, nb, (int)width, nv, d_in, D1,
+                   D2, T, r.nmap, r.mmap, mp);
         WR_LAUNCHED(ctx);
     }
-    WR_TRY(launch_pass(ctx, r.nv, *st.first, st.slabs1, st.T.as<uint32_t>(), st.Wb.as<uint32_t>(),
-                       st.D2.as<uint32_t>(), st.acc1.as<unsigned long long>(), st.mp, nullptr, st.wl1));
+    WR_TRY(launch_pass(ctx, nv, first, slabs1, T, Wb, D2, reinterpret_cast<unsigned long long *>(acc), mp, nullptr, w1));
     // second pass scaled by D1 (not D1^2): out = D1 A^T D2 A D1 in
-    WR_TRY(launch_pass(ctx, r.nv, *st.second, st.slabs2, st.Wb.as<uint32_t>(), st.T.as<uint32_t>(),
-                       st.D1.as<uint32_t>(), st.acc2.as<unsigned long long>(), st.mp, nullptr, st.wl2));
-    if (r.N > 0) {
-        k_unpad<<<blocks_for(r.N * width, 256), 256, 0, s>>>(r.N, (int)width, r.nv, st.T.as<uint32_t>(), d_out,
-                                                             r.nmap);
+    WR_TRY(launch_pass(ctx, nv, second, slabs2, Wb, direct ? d_out : T, D1,
+                       reinterpret_cast<unsigned long long *>(acc + nA1), mp, nullptr, w2));
+    if (r.N > 0 && !direct) {
+        launch_dep(ctx, k_unpad, dim3(blocks_for(r.N * width, 256)), dim3(256), 0, r.N, (int)width, nv, T, d_out, r.nmap);
         WR_LAUNCHED(ctx);
     }
     WR_CUDA(cudaStreamSynchronize(s));
@@ -1122,19 +1207,19 @@ wr_status run_sequence_multi(wr_ctx *ctx, const wr_matrix *mat, const std::vecto
         me1.scale[g] = j.D2.as<uint32_t>();
         me2.scale[g] = j.d1sq.as<uint32_t>();
     }
-    auto grams = [&](bool w_side, int tmul, int toff) -> wr_status {
+    // the Gram products of all jobs, of T alone or of W and T, in one launch
+    auto grams = [&](bool w_side) -> wr_status {
+        GramItems it{};
+        int k = 0;
         for (int g = 0; g < G; g++) {
             Job &j = jobs[g];
-            if (w_side)
-                WR_TRY(launch_gram_to(ctx, rs[g], j.mp, M, j.w2.as<uint32_t>(), Wb.as<uint32_t>() + g * jw, tmul, toff,
-                                      W, r0.nv, j.s_raw.as<unsigned long long>(), counter.as<int>(), err.as<int>()));
-            else
-                WR_TRY(launch_gram_to(ctx, rs[g], j.mp, N, j.xh.as<uint32_t>(), T.as<uint32_t>() + g * jw, tmul, toff,
-                                      W, r0.nv, j.s_raw.as<unsigned long long>(), counter.as<int>(), err.as<int>()));
+            unsigned long long *sr = j.s_raw.as<unsigned long long>();
+            if (w_side && M > 0) it.item[k++] = GramItem{M, j.w2.as<uint32_t>(), Wb.as<uint32_t>() + g * jw, sr, -1, j.mp};
+            if (N > 0) it.item[k++] = GramItem{N, j.xh.as<uint32_t>(), T.as<uint32_t>() + g * jw, sr, 0, j.mp};
         }
-        return WR_OK;
+        return k > 0 ? launch_grams(ctx, rs[0], it, k, 2, W, r0.nv, counter.as<int>(), err.as<int>()) : WR_OK;
     };
-    if (L > 0) WR_TRY(grams(false, 2, 0));  // S_0
+    if (L > 0) WR_TRY(grams(false));  // S_0
     // fed mode: after every group the terms it finished are reduced into
     // each job's sequence and an event published to that job's sigma-basis
     int64_t published = 0;
@@ -1169,8 +1254,7 @@ wr_status run_sequence_multi(wr_ctx *ctx, const wr_matrix *mat, const std::vecto
                                  counter.as<int>(), v1));
         WR_TRY(launch_spmm_multi(ctx, W, sc, Wb.as<uint32_t>(), T.as<uint32_t>(), acc2.as<unsigned long long>(), me2,
                                  nullptr, v2));
-        WR_TRY(grams(true, 2, -1));
-        return grams(false, 2, 0);
+        return grams(true);
     };
     const int64_t terms = std::max<int64_t>(L - 1, 0), iters = (terms + 1) / 2;
     const int64_t Gk = 64;
@@ -1298,8 +1382,6 @@ static wr_status noalloc_scratch_address(int device, void **out) {
     *out = g_noalloc_addr[device];
     return WR_OK;
 }
-
-static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 wr_status blackbox_apply_noalloc(wr_ctx *ctx, const wr_matrix *mat, const wr_params &prm,
                                  const uint32_t *d_in, uint32_t *d_out, int64_t width) {

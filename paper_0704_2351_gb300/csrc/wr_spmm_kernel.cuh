@@ -299,16 +299,22 @@ __global__ void __launch_bounds__(32 * SPMM_WARPS, WIDE && Tile<NV, WL>::LG == 1
     using Ln = Lanes<NV, WL>;
     using Tl = Tile<NV, WL>;
     constexpr int W = Ln::W, G = Ln::G, RPW = Ln::RPW, TE = Tl::TE, E = Tl::E, U = Tl::U;
-    if (term_counter && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(term_counter, 1);
+    pdl_launch();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int sub = lane / G, lanepart = lane % G;
+    // the pass before this one (its output is x) is done from here on; the first
+    // entries are loaded before
+    auto begin = [&]() {
+        pdl_wait();
+        if (term_counter && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(term_counter, 1);
+    };
     const uint32_t xpart = lanepart * W * 4;
     int64_t acc[W];
 #pragma unroll
     for (int w = 0; w < W; w++) acc[w] = 0;
     if ((int64_t)blockIdx.x < vblocks) {
         const int64_t seg = (int64_t)blockIdx.x * SPMM_WARPS + warp;
-        if (seg >= A.nseg) return;
+        if (seg >= A.nseg) return;  // (thread 0 of block 0 has a segment)
         const uint32_t *e = A.ventries + A.seg_start[seg];
         const int16_t *ev = WIDE ? A.vwvals + A.seg_start[seg] : nullptr;
         const int len = A.seg_len[seg];
@@ -327,6 +333,7 @@ __global__ void __launch_bounds__(32 * SPMM_WARPS, WIDE && Tile<NV, WL>::LG == 1
             cur[h] = jh < len ? lde<CS>(e + jh) : 0u;
             cwv[h] = WIDE && jh < len ? (int32_t)__ldg(ev + jh) : 0;
         }
+        begin();
         for (int j = 0; j < len; j += 32 * NR) {
             uint32_t nxt[NR];
             int32_t nwv[NR];
@@ -372,7 +379,10 @@ __global__ void __launch_bounds__(32 * SPMM_WARPS, WIDE && Tile<NV, WL>::LG == 1
     // (fewer than 2^31 rows: chunk * G + q fits 32 bits)
     const uint32_t nlw = (uint32_t)A.nchunks * G;
     uint32_t lw = (blockIdx.x - (uint32_t)vblocks) * pieces * SPMM_WARPS + warp;
-    if (lw >= nlw) return;
+    if (lw >= nlw) {
+        if (blockIdx.x == 0) begin();  // (a launch for the counter alone)
+        return;
+    }
     uint32_t ee[TE];
     int32_t wv[TE];
     // entries [j0, j0 + E) of this lane's row in a chunk of `len` slots at word `at`
@@ -388,6 +398,7 @@ __global__ void __launch_bounds__(32 * SPMM_WARPS, WIDE && Tile<NV, WL>::LG == 1
     int len = __ldg(A.chunk_len + lw / G);
     int64_t at = __ldg(A.chunk_off + lw / G) + (lw % G) * RPW + sub;
     load_tile(at, 0, len, ee, wv);
+    begin();
     for (int k = pieces;;) {
         const uint32_t vr = __ldg(A.vrow + lw * RPW + sub);  // chunk * 32 + q * RPW + sub
         lw += SPMM_WARPS;
@@ -433,6 +444,8 @@ __global__ void __launch_bounds__(32 * SPMM_WARPS, WIDE && Tile<NV, WL>::LG == 1
 __global__ void k_finalize_split(int64_t nsplit, int nv, const int32_t *__restrict__ split_row,
                                  unsigned long long *__restrict__ acc64, uint32_t *__restrict__ y,
                                  const uint32_t *__restrict__ scale, ModP mp, int part) {
+    pdl_launch();
+    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nsplit * nv) return;
     int64_t sid = i / nv;
@@ -450,6 +463,8 @@ __global__ void k_finalize_split(int64_t nsplit, int nv, const int32_t *__restri
 // the same for a multi-job block: column b is reduced with its job's modulus and scale
 __global__ void k_finalize_split_multi(int64_t nsplit, int nv, const int32_t *__restrict__ split_row,
                                        unsigned long long *__restrict__ acc64, uint32_t *__restrict__ y, MultiEpi me) {
+    pdl_launch();
+    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nsplit * nv) return;
     int64_t sid = i / nv;
