@@ -8,20 +8,21 @@
 //
 // over the N rows of a block t (the symmetric projection: L = R; X beside Y:
 // the X and Y halves of the paired block).  They are computed exactly from
-// half-precision products of 8-bit digits.  A residue x < 2^31 is written in
-// balanced digits x = sum_i d_i 2^{8i}: with y = x + 0x808080, d_i = byte_i(y) -
-// 128 for i < 3 and d_3 = byte_3(y) in [0, 128].  Every digit is an integer of
-// magnitude <= 128 (exact in fp16), a digit product is at most 2^14, so the
-// fp32 sums of GT_DRAIN * 64 = 512 rows stay below 2^23 and are exact.
+// half-precision products of 8-bit digits.  A residue x < 2^31 is its four bytes,
+// x = sum_i d_i 2^{8i}, and a byte zero-extended to 16 bits is the fp16 subnormal
+// d 2^-24, exactly; so a digit costs half a byte permutation and no arithmetic
+// (balanced digits took an addition, two permutations and a subtraction a pair).
+// A digit product is below 2^16 (times 2^-48), so the fp32 sums of GT_DRAIN * 64 =
+// 256 rows stay below 2^24 units and are exact.
 //
 // Per tile of 64 rows (the MMA's K), one tcgen05 MMA chain computes
 //   D[i*32 + a][j*NB + b] = sum_r d_i(w_r L_r[a]) d_j(R_r[b])
 // (kind::f16 with fp16 operands, M = 128 = 4 digits x 32 left columns, N = 4
-// digits x NB right columns, fp32 in tensor memory); every 512 rows the eight
+// digits x NB right columns, fp32 in tensor memory); every 256 rows the eight
 // converter warps drain the accumulator (TMEM lane: digit i = warp % 4, column
-// a = lane; half warp / 4 of the right columns) into exact int64 sums
-// acc[b] += sum_j 2^{8j} D[i*32 + a][j*NB + b], and at the end
-//   G[a][b] = sum_i 2^{8i} acc_i[a][b]  mod p.
+// a = lane; half warp / 4 of the right columns) into int32 sums acc[j][b] +=
+// D[i*32 + a][j*NB + b] (a block takes at most GT_MAX_DRAINS of them), and at the end
+//   G[a][b] = sum_i sum_j 2^{8(i+j)} acc_i[j][a][b]  mod p.
 // The rows of t and their weights reach shared memory by 1-D bulk copies
 // (up to five tiles in flight per block, two blocks per SM), eight warps
 // rewrite them as digit tiles in the MMA's swizzled layout, and a ninth warp
@@ -45,7 +46,8 @@ namespace {
 constexpr int GT_CONV = 256;              // converter threads (warps 0-7)
 constexpr int GT_THREADS = GT_CONV + 32;  // and the issuer warp
 constexpr int GT_KT = 64;     // rows per tile
-constexpr int GT_DRAIN = 8;   // tiles per drain of the accumulator (512 rows)
+constexpr int GT_DRAIN = 4;   // tiles per drain of the accumulator (256 rows: sums below 2^24)
+constexpr int GT_MAX_DRAINS = 127;  // sums of a block below 2^31
 constexpr uint64_t GT_WAIT_NS = 2000000000ull;
 constexpr int GT_ERR_TIMEOUT = 1;
 
@@ -69,17 +71,13 @@ struct GramShape {
     static_assert(2 * (SMEM + 1024) <= 228 * 1024, "two blocks a SM");
 };
 
-// Digit I of two consecutive values (y = x + 0x808080 each) as an fp16 pair:
-// the two bytes are placed under 0x64 (fp16 bits 0x64ee = 1024 + e, exact for
-// e < 1024) and 1024 + 128 (digits 0..2) or 1024 (digit 3) is subtracted in
-// one packed half-precision subtraction; every result is an integer of
-// magnitude <= 128, exact.  The lower K index goes to the lower half.
+// Byte I of two consecutive residues as fp16 subnormals, the lower K index in the
+// lower half.  The zero bytes are the sign of byte 3 (permutation mode bit 3), which
+// is 0: residues are below 2^31.
 template <int I>
-__device__ __forceinline__ uint32_t digit_h2(uint32_t y0, uint32_t y1) {
-    const uint32_t t = __byte_perm(y0, y1, I | ((I + 4) << 4));  // [b_I(y0), b_I(y1), ., .]
-    const uint32_t h = __byte_perm(t, 0x64646464u, 0x4140);      // [b_I(y0), 0x64, b_I(y1), 0x64]
+__device__ __forceinline__ uint32_t digit_h2(uint32_t x0, uint32_t x1) {
     uint32_t r;
-    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(I < 3 ? 0x64806480u : 0x64006400u));
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(x0), "r"(x1), "n"(I | 0xB0 | ((I + 4) << 8) | 0xB000));
     return r;
 }
 
@@ -92,16 +90,13 @@ __device__ __forceinline__ void digit_offsets(int row0, int stride, int c, uint3
 
 // the 4 digit rows of 8 consecutive K values into their chunks (off)
 __device__ __forceinline__ void put_digits(unsigned char *tile, const uint32_t (&off)[4], const uint32_t (&x)[8]) {
-    uint32_t y[8];
-#pragma unroll
-    for (int u = 0; u < 8; u++) y[u] = x[u] + 0x808080u;
 #define WR_DIGIT_ROW(I)                                                                              \
     {                                                                                                \
         uint4 q;                                                                                     \
-        q.x = digit_h2<I>(y[0], y[1]);                                                               \
-        q.y = digit_h2<I>(y[2], y[3]);                                                               \
-        q.z = digit_h2<I>(y[4], y[5]);                                                               \
-        q.w = digit_h2<I>(y[6], y[7]);                                                               \
+        q.x = digit_h2<I>(x[0], x[1]);                                                               \
+        q.y = digit_h2<I>(x[2], x[3]);                                                               \
+        q.z = digit_h2<I>(x[4], x[5]);                                                               \
+        q.w = digit_h2<I>(x[6], x[7]);                                                               \
         *reinterpret_cast<uint4 *>(tile + off[I]) = q;                                               \
     }
     WR_DIGIT_ROW(0)
@@ -198,9 +193,11 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
         if (wrows) tc::bulk_g2s(wts + s * GT_KT, w + r0, wrows * 4u, &bar_raw[s]);
     };
 
-    long long acc[HB];
+    int acc[4][HB];
 #pragma unroll
-    for (int b = 0; b < HB; b++) acc[b] = 0;
+    for (int j = 0; j < 4; j++)
+#pragma unroll
+        for (int b = 0; b < HB; b++) acc[j][b] = 0;
 
     if (issuer) {
         if (lane == 0) {
@@ -314,7 +311,7 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
                     tc::tmem_ldn<HB>(tmem + lanes + (uint32_t)(j * NB + hf * HB), v);
                     tc::tmem_ld_wait();
 #pragma unroll
-                    for (int b = 0; b < HB; b++) acc[b] += (long long)__float2int_rn(__uint_as_float(v[b])) << (8 * j);
+                    for (int b = 0; b < HB; b++) acc[j][b] += __float2int_rn(__uint_as_float(v[b]) * 0x1p48f);
                 }
                 tc::tc_fence_before();
                 __syncwarp();
@@ -346,7 +343,11 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
             const int i = warp & 3, hf = warp >> 2;
             const uint32_t sc = powm(256u % mp.p, (uint32_t)i, mp);  // 2^{8 i} mod p
 #pragma unroll
-            for (int b = 0; b < HB; b++) red[(i * 32 + lane) * NB + hf * HB + b] = mulm(red_s64(acc[b], mp), sc, mp);
+            for (int b = 0; b < HB; b++) {
+                const uint64_t v = (uint64_t)(uint32_t)acc[0][b] + ((uint64_t)(uint32_t)acc[1][b] << 8) +
+                                   ((uint64_t)(uint32_t)acc[2][b] << 16) + ((uint64_t)(uint32_t)acc[3][b] << 24);
+                red[(i * 32 + lane) * NB + hf * HB + b] = mulm(red64(v, mp), sc, mp);
+            }
         }
         __syncthreads();
         unsigned long long *dst = it.s_raw + (size_t)k_term * m * n;
@@ -382,8 +383,11 @@ wr_status launch_gram_tc_t(wr_ctx *ctx, const GramItems &items, int count, int m
     int64_t rows = 0;
     for (int i = 0; i < count; i++) rows = max64(rows, items.item[i].rows);
     const int64_t tiles = (rows + GT_KT - 1) / GT_KT;
-    // two blocks a SM over all items, all resident at once
-    const unsigned grid = (unsigned)std::min<int64_t>(tiles, std::max(1, 2 * ctx->num_sms / count));
+    // two blocks a SM over all items, all resident at once; more where a block would
+    // take more tiles than its sums hold
+    const int64_t most = (int64_t)GT_DRAIN * GT_MAX_DRAINS;
+    const unsigned grid =
+        (unsigned)std::min<int64_t>(tiles, std::max<int64_t>(std::max(1, 2 * ctx->num_sms / count), (tiles + most - 2) / (most - 1)));
     if (grid == 0) return WR_OK;
     launch_dep(ctx, k_gram_tc<NB, RB>, dim3(grid, (unsigned)count), dim3(GT_THREADS), S::SMEM, items, m, n, yoff,
                term_counter, tmul, L, err);

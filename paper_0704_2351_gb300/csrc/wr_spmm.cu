@@ -1002,9 +1002,11 @@ wr_status run_sequence_resolved(wr_ctx *ctx, const wr_matrix *mat, Resolved r, i
     return WR_OK;
 }
 
-__global__ void k_to_mont_vec(int64_t len, const uint32_t *__restrict__ in, uint32_t *__restrict__ out, ModP mp) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < len) out[i] = to_mont(in[i], mp);
+// S = factor * s_raw mod p
+__global__ void k_reduce_scaled(int count, const unsigned long long *__restrict__ s_raw, uint32_t *__restrict__ S,
+                                uint32_t factor, ModP mp) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < count) S[i] = mulm(red64(s_raw[i], mp), factor, mp);
 }
 
 // G (m x n) = sum_r w_r t[r][0..m)^T t[r][yoff..yoff+n) mod p, through the
@@ -1017,31 +1019,39 @@ wr_status gram_device(wr_ctx *ctx, uint32_t p, int64_t N, int m, int n, const ui
         return fail(WR_EINVAL, "rows of t: tstride residues, a multiple of the padded width nv >= m and >= yoff + nv, "
                                "yoff a multiple of nv");
     if (reinterpret_cast<uintptr_t>(t) % 16 != 0) return fail(WR_EINVAL, "t must be 16-byte aligned");
-    SeqState st;
-    st.mp = make_modp(p);
-    st.r.m = m;
-    st.r.n = n;
-    st.r.nv = nv;
-    st.r.L = 1;
     cudaStream_t s = ctx->stream;
-    DevBuf wm;
-    WR_TRY(dev_alloc(ctx, wm, sizeof(uint32_t) * std::max<int64_t>(N, 1)));
-    WR_TRY(dev_alloc(ctx, st.s_raw, sizeof(unsigned long long) * m * n));
-    WR_TRY(dev_alloc(ctx, st.counter, sizeof(int)));
-    WR_TRY(dev_alloc(ctx, st.err, sizeof(int)));
-    WR_CUDA(cudaMemsetAsync(st.s_raw.ptr, 0, st.s_raw.bytes, s));
-    WR_CUDA(cudaMemsetAsync(st.counter.ptr, 0, sizeof(int), s));
-    WR_CUDA(cudaMemsetAsync(st.err.ptr, 0, sizeof(int), s));
-    if (N > 0) {
-        k_to_mont_vec<<<blocks_for(N, 256), 256, 0, s>>>(N, w, wm.as<uint32_t>(), st.mp);
-        WR_LAUNCHED(ctx);
-        WR_TRY(launch_gram(ctx, st, N, wm.as<uint32_t>(), t, 1, 0, tstride, yoff));
+    // the bulk copies of the weights start on 16-byte boundaries
+    DevBuf wcopy;
+    if (N > 0 && reinterpret_cast<uintptr_t>(w) % 16 != 0) {
+        WR_TRY(dev_alloc(ctx, wcopy, sizeof(uint32_t) * (size_t)N + 16));
+        uint32_t *wa = reinterpret_cast<uint32_t *>((reinterpret_cast<uintptr_t>(wcopy.ptr) + 15) & ~uintptr_t(15));
+        WR_CUDA(cudaMemcpyAsync(wa, w, sizeof(uint32_t) * (size_t)N, cudaMemcpyDeviceToDevice, s));
+        w = wa;
     }
-    k_reduce_seq<<<blocks_for((int64_t)m * n, 256), 256, 0, s>>>((int64_t)m * n, st.s_raw.as<unsigned long long>(),
-                                                                G, st.mp);
+    // s_raw (m n sums), term counter, error flag
+    DevBuf ws;
+    const size_t nS = sizeof(unsigned long long) * (size_t)m * n;
+    WR_TRY(dev_alloc(ctx, ws, nS + 2 * sizeof(int)));
+    WR_CUDA(cudaMemsetAsync(ws.ptr, 0, ws.bytes, s));
+    unsigned long long *s_raw = ws.as<unsigned long long>();
+    int *counter = reinterpret_cast<int *>(ws.as<unsigned char>() + nS), *err = counter + 1;
+    const ModP mp = make_modp(p);
+    if (N > 0) {
+        // the kernels' weights are in Montgomery form; w as it is gives the products
+        // over R, and the reduction below multiplies by R
+        Resolved r;
+        r.m = m;
+        r.n = n;
+        r.nv = nv;
+        r.L = 1;
+        GramItems g{};
+        g.item[0] = GramItem{N, w, t, s_raw, 0, mp};
+        WR_TRY(launch_grams(ctx, r, g, 1, 1, tstride, yoff, counter, err));
+    }
+    k_reduce_scaled<<<blocks_for((int64_t)m * n, 256), 256, 0, s>>>(m * n, s_raw, G, mp.r1, mp);
     WR_LAUNCHED(ctx);
     int herr = 0;
-    WR_CUDA(cudaMemcpyAsync(&herr, st.err.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
+    WR_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     WR_CUDA(cudaStreamSynchronize(s));
     if (herr) return fail(WR_ETIMEDOUT, "tensor-core projection: a bounded wait ran out");
     return WR_OK;
