@@ -115,6 +115,26 @@ __host__ __device__ __forceinline__ uint32_t red64(uint64_t x, const ModP &m) {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// thread block clusters
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// store to the same shared-memory address of block `rank` of the cluster
+__device__ __forceinline__ void st_cluster(uint32_t *p, uint32_t rank, uint32_t v) {
+    uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p)), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(r), "r"(v) : "memory");
+}
+
 // d = a b + c in one 32x32 -> 64-bit multiply-add
 __device__ __forceinline__ unsigned long long madw(uint32_t a, uint32_t b, unsigned long long c) {
     unsigned long long d;
@@ -646,6 +666,12 @@ wr_status resolve(const wr_matrix *mat, const wr_params *prm, Resolved &r);
 
 wr_status run_sequence_resolved(wr_ctx *ctx, const wr_matrix *mat, Resolved r, int64_t L, uint32_t *d_S,
                                 double *setup_ms, double *seq_ms, SeqFeed *feed = nullptr, StateOut *out = nullptr);
+// the loop of a small matrix on one cluster (wr_seq_small.cu): `apps` applications from
+// application `base` on, T in global memory before and after
+bool seq_small_fits(const wr_ctx *ctx, const Sell &first, const Sell &second, const Resolved &r);
+wr_status launch_seq_small(wr_ctx *ctx, const Sell &first, const Sell &second, const Resolved &r, const ModP &mp, uint32_t *T,
+                           const uint32_t *scale1, const uint32_t *scale2, const uint32_t *gw1, const uint32_t *gw2,
+                           unsigned long long *s_raw, int64_t base, int apps, int64_t L);
 // whether the generic projection pairs X with Y in one block (m = n)
 bool pairs_generic(const wr_ctx *ctx, const Resolved &r);
 

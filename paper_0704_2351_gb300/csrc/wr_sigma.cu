@@ -358,25 +358,6 @@ __host__ __device__ inline LcLayout lc_layout(int m, int q, int b, int CS, int M
     return l;
 }
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t cluster_size() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-// store to the same shared-memory address of block `rank` of the cluster
-__device__ __forceinline__ void st_cluster(uint32_t *p, uint32_t rank, uint32_t v) {
-    uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p)), r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(r), "r"(v) : "memory");
-}
-
 // A row times the order's transform in registers (lane: column j and, CPL = 2,
 // column j + 32; f[k][t] = F[t][column k], d[k] its diagonal): x[k] the row's
 // residues of the lane's columns, g the row's residue at pivot column t = the

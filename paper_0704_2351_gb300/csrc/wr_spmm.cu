@@ -901,7 +901,11 @@ wr_status run_sequence_resolved(wr_ctx *ctx, const wr_matrix *mat, Resolved r, i
     cudaGraphExec_t exec = nullptr;
     cudaGraph_t graph = nullptr;
     int64_t graph_launches = 0;  // kernel nodes in one replay
-    if (iters >= G) {
+    // a small matrix: groups of applications in one launch each (unless the context asks
+    // for what only the passes do: their events, the side stream, the tensor cores)
+    const bool small = !ctx->profiling && !st.side && ctx->tensor_proj != 1 && !st.slabs1 && !st.slabs2 &&
+                       seq_small_fits(ctx, *st.first, *st.second, r);
+    if (iters >= G && !small) {
         const int64_t before = ctx->launches;
         WR_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
         wr_status cst = WR_OK;
@@ -932,7 +936,11 @@ wr_status run_sequence_resolved(wr_ctx *ctx, const wr_matrix *mat, Resolved r, i
         // a snapshot of the block ends the group at its application count
         const int64_t lim = (out && out->d_snap && out->snap_at > done) ? std::min(out->snap_at, iters) : iters;
         const int64_t todo = std::min(G, lim - done);
-        if (todo == G && exec && !(ctx->profiling && group % PROF_EVERY == 0)) {
+        if (small) {
+            loop_st = launch_seq_small(ctx, *st.first, *st.second, r, st.mp, st.T.as<uint32_t>(), st.D2.as<uint32_t>(),
+                                       st.d1sq.as<uint32_t>(), st.w2.as<uint32_t>(), st.xh.as<uint32_t>(),
+                                       st.s_raw.as<unsigned long long>(), done, (int)todo, L);
+        } else if (todo == G && exec && !(ctx->profiling && group % PROF_EVERY == 0)) {
             cudaError_t ce = cudaGraphLaunch(exec, s);
             if (ce != cudaSuccess) loop_st = cuda_fail(ce, "cudaGraphLaunch");
             ctx->launches += graph_launches;
