@@ -28,7 +28,12 @@
 // rewrite them as digit tiles in the MMA's swizzled layout, and a ninth warp
 // issues the MMAs, commits them to an mbarrier and requests the next rows, so
 // that issuing never holds up the conversion; operand tiles are
-// double-buffered.  Every wait is bounded: after WAIT_NS the block records an
+// double-buffered.  The accumulator is double too: a drain waits for its group's last
+// MMA, some 2,000 cycles after that tile was converted, so the converters first convert
+// the next group's first tile and the MMAs run on in the other accumulator.  What bounds
+// the kernel is the conversion (shared loads, digits, shared stores, the fence: one chain
+// a tile, two blocks a SM).  The X X and X Y products of an application at 1.9M rows x 32:
+// 277 us with one accumulator, 238 us so.  Every wait is bounded: after WAIT_NS the block records an
 // error, waits (bounded) for its copies and MMAs in flight, frees its tensor
 // memory and returns.
 #include <cuda_runtime.h>
@@ -58,7 +63,8 @@ struct GramShape {
     static constexpr uint32_t BBYTES = (uint32_t)TN * 128u;
     static constexpr uint32_t OPB = ABYTES + BBYTES;       // one operand stage
     static constexpr uint32_t RAWB = (uint32_t)GT_KT * RB; // one raw tile
-    static constexpr uint32_t TMEM_COLS = TN < 32 ? 32 : TN;
+    static constexpr uint32_t TMEM_COLS = 2 * TN;          // two accumulators (groups of tiles in turn)
+    static_assert(TMEM_COLS >= 32 && TMEM_COLS <= 256, "two blocks a SM share 512 columns");
     static constexpr uint32_t WB = (uint32_t)GT_KT * 4;   // one tile's weights
     // raw tiles in flight per block (two blocks a SM): five for rows of up to
     // 128 bytes (32 KB in flight a block, what the shared memory of two
@@ -81,15 +87,11 @@ __device__ __forceinline__ uint32_t digit_h2(uint32_t x0, uint32_t x1) {
     return r;
 }
 
-// byte offsets in a swizzled tile of the 16-byte chunk c of the 4 digit rows
-// row0 + i * stride (the same for every tile a thread converts)
-__device__ __forceinline__ void digit_offsets(int row0, int stride, int c, uint32_t (&off)[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; i++) off[i] = tc::sw128_chunk((uint32_t)(row0 + i * stride), (uint32_t)c);
-}
-
-// the 4 digit rows of 8 consecutive K values into their chunks (off)
-__device__ __forceinline__ void put_digits(unsigned char *tile, const uint32_t (&off)[4], const uint32_t (&x)[8]) {
+// the 4 digit rows (row0 + I * STRIDE, STRIDE a multiple of the 8 rows of an atom) of 8
+// consecutive K values into their chunks; off: byte offset in the swizzled tile of row0's
+template <int STRIDE>
+__device__ __forceinline__ void put_digits(unsigned char *tile, uint32_t off, const uint32_t (&x)[8]) {
+    static_assert(STRIDE % 8 == 0, "digit rows in the same place of their atoms");
 #define WR_DIGIT_ROW(I)                                                                              \
     {                                                                                                \
         uint4 q;                                                                                     \
@@ -97,7 +99,7 @@ __device__ __forceinline__ void put_digits(unsigned char *tile, const uint32_t (
         q.y = digit_h2<I>(x[2], x[3]);                                                               \
         q.z = digit_h2<I>(x[4], x[5]);                                                               \
         q.w = digit_h2<I>(x[6], x[7]);                                                               \
-        *reinterpret_cast<uint4 *>(tile + off[I]) = q;                                               \
+        *reinterpret_cast<uint4 *>(tile + off + (I) * STRIDE * 128) = q;                                               \
     }
     WR_DIGIT_ROW(0)
     WR_DIGIT_ROW(1)
@@ -116,10 +118,11 @@ __device__ __forceinline__ void put_digits(unsigned char *tile, const uint32_t (
 // warp on conv[stage]); warp 8's first lane issues (wait on conv[stage],
 // the four MMAs of the tile, the commit to mma[stage], the bulk copies of the
 // tile GT_NS ahead into the raw stage just converted), so that the issue
-// never holds up a converter.  Every GT_DRAIN tiles the converters drain the
-// accumulator (warp w: digit row w % 4 of the left factor, half w / 4 of the
-// right factor's columns) and arrive on drained, which the issuer waits for
-// before the next group overwrites the accumulator.  All waits are bounded
+// never holds up a converter.  Groups of GT_DRAIN tiles take the two accumulators
+// in turn; the converters drain a group's (warp w: digit row w % 4 of the left
+// factor, half w / 4 of the right factor's columns) after converting the next
+// group's first tile, when its MMAs are done, and arrive on drained, which the
+// issuer waits for before the group after that overwrites it.  All waits are bounded
 // mbarrier waits; a wait that runs out sets a shared flag that every role
 // polls, and the issuer then lets the copies and MMAs in flight finish.
 template <int NB, int RB>
@@ -142,15 +145,15 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
     uint64_t *bar_raw = reinterpret_cast<uint64_t *>(wts + S::NS * GT_KT);
     uint64_t *bar_mma = bar_raw + S::NS;   // [2] MMAs of an operand stage done
     uint64_t *bar_conv = bar_mma + 2;      // [2] operand stage converted
-    uint64_t *bar_drain = bar_conv + 2;    // accumulator drained
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar_drain + 1);
+    uint64_t *bar_drain = bar_conv + 2;    // [2] accumulator drained
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar_drain + 2);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool issuer = warp == GT_CONV / 32;
     const int64_t tiles = (N + GT_KT - 1) / GT_KT;
     const int64_t t_begin = tiles * blockIdx.x / gridDim.x;
-    const int64_t ntile = tiles * (blockIdx.x + 1) / gridDim.x - t_begin;
+    const int ntile = (int)(tiles * (blockIdx.x + 1) / gridDim.x - t_begin);
 
     // (everything up to pdl_wait overlaps the pass before)
     // both operand stages start at zero: digit rows of absent columns stay zero
@@ -162,7 +165,8 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
         tc::mbar_init(&bar_mma[1], 1);
         tc::mbar_init(&bar_conv[0], GT_CONV / 32);
         tc::mbar_init(&bar_conv[1], GT_CONV / 32);
-        tc::mbar_init(bar_drain, GT_CONV / 32);
+        tc::mbar_init(&bar_drain[0], GT_CONV / 32);
+        tc::mbar_init(&bar_drain[1], GT_CONV / 32);
         *abort_flag = 0;
         tc::fence_mbar_init();
     }
@@ -182,8 +186,8 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
         return;
     }
 
-    int64_t issued = 0, committed = 0;  // (issuer) raw tiles requested, MMA commits
-    auto issue = [&](int64_t tl) {
+    int issued = 0, committed = 0;  // (issuer) raw tiles requested, MMA commits
+    auto issue = [&](int tl) {
         const int s = (int)(tl % S::NS);
         const int64_t r0 = (t_begin + tl) * GT_KT;
         const uint32_t rows = (uint32_t)min64(GT_KT, N - r0);
@@ -202,13 +206,15 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
     if (issuer) {
         if (lane == 0) {
             for (; issued < ntile && issued < S::NS; issued++) issue(issued);
-            for (int64_t tl = 0; tl < ntile; tl++) {
+            for (int tl = 0; tl < ntile; tl++) {
                 const int so = (int)(tl & 1), g = (int)(tl % GT_DRAIN);
                 if (*abort_flag) break;
                 bool ok = tc::mbar_wait(&bar_conv[so], (uint32_t)((tl >> 1) & 1), GT_WAIT_NS);
-                // a new group overwrites the accumulator: the last one's drain must be done
-                if (ok && g == 0 && tl > 0)
-                    ok = tc::mbar_wait(bar_drain, (uint32_t)(((tl / GT_DRAIN) - 1) & 1), GT_WAIT_NS);
+                // a new group overwrites the accumulator of the group before the last: its
+                // drain must be done
+                const int gq = tl / GT_DRAIN;
+                if (ok && g == 0 && gq >= 2)
+                    ok = tc::mbar_wait(&bar_drain[gq & 1], (uint32_t)(((gq >> 1) - 1) & 1), GT_WAIT_NS);
                 if (!ok) {
                     *abort_flag = 1;
                     break;
@@ -218,8 +224,8 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
                 const uint32_t a0 = tc::smem_addr(opA), b0 = tc::smem_addr(opB);
 #pragma unroll
                 for (int ks = 0; ks < GT_KT / 16; ks++)
-                    tc::mma_f16(tmem, tc::sdesc_k_sw128(a0 + 32u * ks), tc::sdesc_k_sw128(b0 + 32u * ks), IDESC,
-                                 (ks > 0 || g > 0) ? 1u : 0u);
+                    tc::mma_f16(tmem + (uint32_t)(gq & 1) * S::TN, tc::sdesc_k_sw128(a0 + 32u * ks),
+                                tc::sdesc_k_sw128(b0 + 32u * ks), IDESC, (ks > 0 || g > 0) ? 1u : 0u);
                 tc::mma_commit(&bar_mma[so]);
                 committed++;
                 // the raw stage of this tile has been converted: refill it
@@ -236,87 +242,105 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
         // column a = lane; right factor chunk tid / NB, column tid % NB
         const int ca = warp, a = lane, cb = tid / NB, b = tid % NB;
         const bool do_l = a < m, do_r = tid < 8 * NB && b < n;
-        uint32_t offL[4], offR[4];
-        digit_offsets(a, 32, ca, offL);
-        digit_offsets(b, NB, cb & 7, offR);
-        for (int64_t tl = 0; tl < ntile; tl++) {
-            const int sr = (int)(tl % S::NS), so = (int)(tl & 1);
-            const int g = (int)(tl % GT_DRAIN);
-            if (*abort_flag) break;
-            unsigned char *opA = base + so * S::OPB, *opB = opA + S::ABYTES;
-            // the raw rows have landed; the operand stage's previous MMAs are done
-            bool ok = tc::mbar_wait(&bar_raw[sr], (uint32_t)((tl / S::NS) & 1), GT_WAIT_NS);
-            if (ok && tl >= 2) ok = tc::mbar_wait(&bar_mma[so], (uint32_t)(((tl >> 1) - 1) & 1), GT_WAIT_NS);
-            if (!ok) {
-                *abort_flag = 1;
-                break;
-            }
-            const int64_t r0 = (t_begin + tl) * GT_KT;
-            const int rows = (int)min64(GT_KT, N - r0);
-            const uint32_t *rw = reinterpret_cast<const uint32_t *>(raw + sr * S::RAWB);
-            const uint32_t *ws = wts + sr * GT_KT;
-            const int wrows = rows & ~3;
-            if (rows == GT_KT) {
-                // a whole tile: every row and weight is in shared memory
-                if (do_l) {
-                    uint32_t x[8];
+        const uint32_t offL = tc::sw128_chunk((uint32_t)a, (uint32_t)ca);
+        const uint32_t offR = tc::sw128_chunk((uint32_t)b, (uint32_t)(cb & 7));
+        // the accumulator of group gq into the sums (the commit of its last tile covers
+        // every earlier MMA)
+        auto drain = [&](int gq) -> bool {
+            const int last = min((gq + 1) * GT_DRAIN, ntile) - 1;
+            if (!tc::mbar_wait(&bar_mma[last & 1], (uint32_t)((last >> 1) & 1), GT_WAIT_NS)) return false;
+            tc::tc_fence_after();
+            const uint32_t at = tmem + (uint32_t)(gq & 1) * S::TN + ((uint32_t)((warp & 3) * 32) << 16) +
+                                (uint32_t)((warp >> 2) * HB);
 #pragma unroll
-                    for (int u = 0; u < 8; u++) x[u] = mont_mul(ws[8 * ca + u], rw[(8 * ca + u) * RW + a], mp);
-                    put_digits(opA, offL, x);
-                }
-                if (do_r) {
-                    uint32_t x[8];
+            for (int j = 0; j < 4; j++) {
+                constexpr int DC = HB < 8 ? HB : 8;  // columns a load: the sums leave few registers
 #pragma unroll
-                    for (int u = 0; u < 8; u++) x[u] = rw[(8 * cb + u) * RW + yoff + b];
-                    put_digits(opB, offR, x);
-                }
-            } else {
-                if (do_l) {
-                    // left factor, weighted (the last weights past a 16-byte group by plain loads)
-                    uint32_t x[8];
+                for (int h = 0; h < HB; h += DC) {
+                    uint32_t v[DC];
+                    tc::tmem_ldn<DC>(at + (uint32_t)(j * NB + h), v);
+                    tc::tmem_ld_wait();
 #pragma unroll
-                    for (int u = 0; u < 8; u++) {
-                        const int rr = 8 * ca + u;
-                        const uint32_t wv = rr < wrows ? ws[rr] : (rr < rows ? __ldg(w + r0 + rr) : 0u);
-                        x[u] = rr < rows ? mont_mul(wv, rw[rr * RW + a], mp) : 0u;
-                    }
-                    put_digits(opA, offL, x);
-                }
-                if (do_r) {
-                    uint32_t x[8];
-#pragma unroll
-                    for (int u = 0; u < 8; u++) {
-                        const int rr = 8 * cb + u;
-                        x[u] = rr < rows ? rw[rr * RW + yoff + b] : 0u;
-                    }
-                    put_digits(opB, offR, x);
+                    for (int b = 0; b < DC; b++)
+                        acc[j][h + b] += __float2int_rn(__uint_as_float(v[b]) * 0x1p48f);
                 }
             }
-            tc::fence_proxy_async_smem();
+            tc::tc_fence_before();
             __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&bar_conv[so]);
-            if (g == GT_DRAIN - 1 || tl == ntile - 1) {
-                // drain: the accumulator of this group into the int64 sums
-                // (the commit of this tile covers every earlier MMA)
-                if (!tc::mbar_wait(&bar_mma[so], (uint32_t)((tl >> 1) & 1), GT_WAIT_NS)) {
+            if (lane == 0) tc::mbar_arrive(&bar_drain[gq & 1]);
+            return true;
+        };
+        // X = Y with 32 columns: a thread's left and right residues are the same
+        const bool same = NB == 32 && yoff == 0;
+        for (int tl = 0; tl <= ntile; tl++) {
+            const int sr = (int)(tl % S::NS), so = (int)(tl & 1);
+            const int g = tl % GT_DRAIN;
+            if (*abort_flag) break;
+            if (tl < ntile) {
+                unsigned char *opA = base + so * S::OPB, *opB = opA + S::ABYTES;
+                // the raw rows have landed; the operand stage's previous MMAs are done
+                bool ok = tc::mbar_wait(&bar_raw[sr], (uint32_t)((tl / S::NS) & 1), GT_WAIT_NS);
+                if (ok && tl >= 2) ok = tc::mbar_wait(&bar_mma[so], (uint32_t)(((tl >> 1) - 1) & 1), GT_WAIT_NS);
+                if (!ok) {
                     *abort_flag = 1;
                     break;
                 }
-                tc::tc_fence_after();
-                const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
-                const int hf = warp >> 2;
+                const int64_t r0 = (t_begin + tl) * GT_KT;
+                const int rows = (int)min64(GT_KT, N - r0);
+                const uint32_t *rw = reinterpret_cast<const uint32_t *>(raw + sr * S::RAWB);
+                const uint32_t *ws = wts + sr * GT_KT;
+                const int wrows = rows & ~3;
+                const bool full = rows == GT_KT;
+                uint32_t x[8];
+                if (do_r) {
+                    const uint32_t *src = rw + 8 * cb * RW + yoff + b;
+                    if (full) {
 #pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    uint32_t v[HB];
-                    tc::tmem_ldn<HB>(tmem + lanes + (uint32_t)(j * NB + hf * HB), v);
-                    tc::tmem_ld_wait();
+                        for (int u = 0; u < 8; u++) x[u] = src[u * RW];
+                    } else {
 #pragma unroll
-                    for (int b = 0; b < HB; b++) acc[j][b] += __float2int_rn(__uint_as_float(v[b]) * 0x1p48f);
+                        for (int u = 0; u < 8; u++) x[u] = 8 * cb + u < rows ? src[u * RW] : 0u;
+                    }
+                    put_digits<NB>(opB, offR, x);
                 }
-                tc::tc_fence_before();
+                if (do_l) {
+                    // weighted; X = Y with 32 columns: this thread's residues are those above
+                    if (!same || !do_r) {
+                        const uint32_t *src = rw + 8 * ca * RW + a;
+                        if (full) {
+#pragma unroll
+                            for (int u = 0; u < 8; u++) x[u] = src[u * RW];
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < 8; u++) x[u] = 8 * ca + u < rows ? src[u * RW] : 0u;
+                        }
+                    }
+                    // (the last weights past a 16-byte group by plain loads)
+#pragma unroll
+                    for (int h = 0; h < 8; h += 4) {
+                        const int rr = 8 * ca + h;
+                        uint4 wv;
+                        if (rr + 4 <= wrows) {
+                            wv = *reinterpret_cast<const uint4 *>(ws + rr);
+                        } else {
+                            wv.x = rr < rows ? __ldg(w + r0 + rr) : 0u;
+                            wv.y = rr + 1 < rows ? __ldg(w + r0 + rr + 1) : 0u;
+                            wv.z = rr + 2 < rows ? __ldg(w + r0 + rr + 2) : 0u;
+                            wv.w = 0u;  // (a whole group ends at a row that is there)
+                        }
+                        x[h] = mont_mul(wv.x, x[h], mp);
+                        x[h + 1] = mont_mul(wv.y, x[h + 1], mp);
+                        x[h + 2] = mont_mul(wv.z, x[h + 2], mp);
+                        x[h + 3] = mont_mul(wv.w, x[h + 3], mp);
+                    }
+                    put_digits<32>(opA, offL, x);
+                }
+                tc::fence_proxy_async_smem();
                 __syncwarp();
-                if (lane == 0) tc::mbar_arrive(bar_drain);
+                if (lane == 0) tc::mbar_arrive(&bar_conv[so]);
             }
+            // the group before, whose MMAs ran while this tile was converted
+            if (tl > 0 && (g == 0 || tl == ntile) && !drain((tl - 1) / GT_DRAIN)) *abort_flag = 1;
         }
     }
 
@@ -326,10 +350,10 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
         // record the error, let the copies and MMAs in flight finish (bounded)
         if (issuer && lane == 0) {
             atomicExch(err, GT_ERR_TIMEOUT);
-            for (int64_t tl = max64(0, issued - S::NS); tl < issued; tl++)
+            for (int tl = max(0, issued - S::NS); tl < issued; tl++)
                 tc::mbar_wait(&bar_raw[tl % S::NS], (uint32_t)((tl / S::NS) & 1), GT_WAIT_NS);
             if (committed > 0) {
-                const int64_t last = committed - 1;
+                const int last = committed - 1;
                 tc::mbar_wait(&bar_mma[last & 1], (uint32_t)((last >> 1) & 1), GT_WAIT_NS);
             }
         }

@@ -64,3 +64,28 @@ def test_more_rows_than_a_blocks_sums_hold(wr):
         out.append(G.cpu().clone())
     wr.wr_destroy(ctx)
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("m,stride,yoff", [(32, 32, 0), (20, 32, 0), (32, 64, 32), (16, 32, 16), (8, 8, 0)])
+@pytest.mark.parametrize("groups", [1, 2, 3, 5])
+def test_groups_of_tiles_in_both_accumulators(wr, m, stride, yoff, groups):
+    """Blocks of one to a few groups of four tiles, and of a tile more or less."""
+    p = 2147483629
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m + groups)
+    ctx = wr.wr_create(0)
+    for tiles in (4 * groups - 1, 4 * groups, 4 * groups + 1):
+        N = 2 * sms * 64 * tiles - 7
+        t = torch.randint(0, p, (N, stride), generator=g, device="cuda", dtype=torch.int32)
+        t[: N // 4] = p - 1
+        w = torch.randint(0, p, (N,), generator=g, device="cuda", dtype=torch.int32)
+        G = torch.empty((m, m), dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        out = []
+        for mode in (0, 1):
+            wr.wr_set_tensor_projection(ctx, mode)
+            wr.wr_gram_device(ctx, p, N, m, m, t, stride, yoff, w, G)
+            out.append(G.cpu().clone())
+        assert torch.equal(out[0], out[1]), tiles
+    wr.wr_destroy(ctx)
