@@ -246,8 +246,8 @@ __global__ void __launch_bounds__(256)
 // Orders per chunk unless the context sets it (wr_set_sigma_chunk): the window and
 // product launches are spread over more orders by a longer chunk, the local kernel's
 // row work per order grows with it.  Measured: q = 16, 11,252 orders 58 / 53 ms
-// for 32 / 64; q = 32, 2,254 orders 20.0 / 19.6 / 23.1 ms for 16 / 32 / 64; q = 64,
-// 4,098 orders (256-order leaves) 126 / 122 / 135 ms for 8 / 16 / 32.
+// for 32 / 64; q = 32, 2,254 orders 23.1 / 17.4 / 18.5 ms for 8 / 32 / 64; q = 64,
+// 4,098 orders (256-order leaves) 101 / 96 / 105 ms for 8 / 16 / 32.
 inline int sigma_chunk_default(int q) {
     return q <= 16 ? 64 : (q <= 32 ? 32 : 16);
 }
@@ -259,10 +259,9 @@ inline int sigma_chunk_default(int q) {
 // 180,000 matrix: 1,777 ms with the M-Basis chunk by chunk, 1,622 / 1,607 in
 // PM-Basis segments with 2,048- / 4,096-order leaves).  For q > 32 those passes
 // cost more per order, so PM-Basis with short leaves takes over early: at q =
-// 64, 4,098 orders, 125 / 122 / 132 ms for leaves of 128 / 256 / 512 orders, and
-// against the M-Basis alone 16.8 / 15.8 ms at 600 orders, 27.8 / 29.3 at 1,000,
-// 42.3 / 49.5 at 1,500, 58.5 / 75.5 at 2,040.  wr_set_sigma_leaf chooses the leaf
-// explicitly.
+// 64, 4,098 orders, 98 / 96 / 105 ms for leaves of 128 / 256 / 512 orders, and
+// against the M-Basis alone 12.9 / 12.0 ms at 600 orders, 21.4 / 22.9 at 1,000,
+// 32.7 / 39.9 at 1,500.  wr_set_sigma_leaf chooses the leaf explicitly.
 constexpr int64_t SIGMA_LEAF_DEFAULT = 4096;
 constexpr int64_t SIGMA_PM_MIN_L = 16384;
 constexpr int64_t SIGMA_LEAF_WIDE = 256;
@@ -299,15 +298,16 @@ __device__ __forceinline__ void named_arrive(int id, int nthreads) {
 // Roles in a block: the first warps (EW of them) eliminate, the others multiply
 // rows.  Per order i
 //   elim    Gauss-Jordan by rows on the m x q discrepancy, columns in (degree,
-//           index) order, 4 column slots x MR rows over the EW warps, q / 4
-//           residues a lane.  A column is frozen (written to FR) at its turn; if it
+//           index) order, 4 or 8 column slots x MR rows over the EW warps.  A column is frozen (written to FR) at its turn; if it
 //           is nonzero outside the pivot rows so far it becomes pivot k, its first
 //           such row r_k the pivot row, and every other row of the later columns
 //           becomes d_k row - A[row][pc] row_k (fraction-free).  Row r_t then holds
 //           the coefficients of the pivot columns, times prod_{t <= i < k} d_i, so
 //           with pre_t = d_0 .. d_{t-1}: s_j = pre_k(j), F[t][j] = -pre_t FR[j][r_t]
 //           (t < k(j), the pivots before j) -- no inverse, and no transform
-//           carried beside the matrix.
+//           carried beside the matrix.  With several warps the columns go by groups
+//           of one per slot: within a group step by step, the later columns take the
+//           group's whole transform as one product.
 //   rows    first the block's rows of orders i and i + 1 (the next discrepancy:
 //           pivot columns take order i's value, the others order i + 1's), written
 //           to all blocks; then, beside the next elimination, the other rows.
@@ -319,29 +319,40 @@ __device__ __forceinline__ void named_arrive(int id, int nthreads) {
 // Multiplying column c by x moves no data: window column c is read at row
 // ip - sh[c], and Ml column c holds its coefficient s at row base[c] + s.
 //
-// Bound by the chain of one order: m pivot steps of a shared store, a barrier of EW
-// warps, a load, a ballot, two shuffles and one two-product Montgomery
-// reduction.  Measured per order (GB300): q = 16 9.6 -> 2.4 us, q = 32 70 -> 4.7 us,
-// q = 64 68 -> 17 us (one block, one elimination warp that also carried the
-// transform, or sixteen warps with all rows of the chunk on one SM, before).
+// Bound by the chain of one order (elimination, hand-over, the next discrepancy's rows,
+// the cluster barrier) and, at q = 64, by issue: an order is 47,000 warp instructions a
+// block, a wide multiply-add taking a scheduler five cycles.  Hence the elimination
+// by groups of columns, one copy of the row product's code, sums reduced by three
+// multiplications, and 16 blocks where 8 rows a block kept the row warps busy longer
+// than the elimination.  An odd pitch for the discrepancy and the transform: with lanes
+// a row apart, pitch q put the elimination's loads and the transform's stores on one
+// bank (4,700 of 32,000 cycles an order at q = 64).  Measured per order (GB300): q = 16
+// 9.6 -> 2.3 us, q = 32 70 -> 4.2 us, q = 64 68 -> 11 us (17 with 8 blocks and 32 steps on
+// every later column; at first one block, one elimination warp that also carried the
+// transform, or sixteen warps with all rows of the chunk on one SM).  A warp of its own
+// for the bookkeeping, beside the elimination, gained nothing: the chain runs through
+// the rows (sigma-basis of 11,252 orders at q = 16 52.8 ms without, 53.8 with).
 constexpr int LC_SNAP = 228;   // words of an order's snapshot
 constexpr int LC_INTS = 1392;  // words of the bookkeeping arrays
 __host__ __device__ constexpr int lc_threads(int MR) { return MR == 32 ? 512 : (MR == 16 ? 384 : 256); }
 // elimination warps: one for MR = 8 (4 column slots, handed round by shuffles), else 8 column slots
 __host__ __device__ constexpr int lc_ew(int MR) { return MR == 8 ? 1 : MR / 4; }
+// words of a row warp's pivot residues: 32, or 16 groups of 2 lanes with 8 each
+__host__ __device__ constexpr int lc_gs_words(int MR) { return MR == 8 ? 128 : 32; }
 
-// Blocks per cluster for q columns (8 is the largest portable size): q = 16 84 / 82
-// ms for 4 / 8, q = 32 49 / 43, q = 64 413 / 400 (the whole sigma-basis with the
-// earlier window and product kernels); up to 8 columns 4 and 8 measure the same
+// Blocks per cluster for q columns (8 is the largest portable size, 16 the largest): the
+// whole sigma-basis with 8 / 16 blocks: q = 32, 2,254 orders 19.6 / 17.4 ms; q = 64, 4,098
+// orders 113 / 97 ms; q = 16, 11,252 orders, 4 / 8 blocks 84 / 82 ms with the earlier
+// kernels, 16 as 8; up to 8 columns 4 and 8 measure the same
 inline int local_cluster(int q) {
-    return q > 8 ? 8 : 4;
+    return q > 16 ? 16 : q > 8 ? 8 : 4;
 }
 
 struct LcLayout {  // word offsets of the dynamic shared memory (ints and residues are both words)
     int ma, mx;    // most rows of a window order / of an Ml coefficient in a block
-    int Es, Ml, qt, disc, F, dg, FR, ints, total;
+    int Es, Ml, qt, disc, F, dg, FR, gs, ints, total;
 };
-__host__ __device__ inline LcLayout lc_layout(int m, int q, int b, int CS, int MR) {
+__host__ __device__ inline LcLayout lc_layout(int m, int q, int b, int CS, int MR, int QC) {
     LcLayout l;
     l.ma = (m + CS - 1) / CS;
     l.mx = (q + CS - 1) / CS;
@@ -349,23 +360,35 @@ __host__ __device__ inline LcLayout lc_layout(int m, int q, int b, int CS, int M
     l.Es = o; o += b * l.ma * q;
     l.Ml = o; o += (2 * b + 1) * l.mx * q;
     l.qt = o; o += l.ma * q;
-    l.disc = o; o += 2 * m * q;
-    l.F = o; o += 2 * m * q;
+    l.disc = o; o += 2 * m * (QC + 1);
+    l.F = o; o += 2 * MR * (QC + 1);  // (rows from m on stay zero)
     l.dg = o; o += 2 * 64;
     l.FR = o; o += q * (MR + 1);
+    o = (o + 3) & ~3;  // (16-byte loads)
+    l.gs = o; o += (lc_threads(MR) / 32 - lc_ew(MR)) * lc_gs_words(MR);
     l.ints = o; o += LC_INTS;
     l.total = o;
     return l;
 }
 
+// (a0 + a1) 2^-32 mod p: folded, each is at most (c + 1)(2^32 - 1) <= 2^63 (c = 2^32 mod
+// p), so their sum fits, and folded again it is below p 2^32 (3 multiplications; the
+// general reduction mod p takes 8)
+__device__ __forceinline__ uint32_t redc_sum(unsigned long long a0, unsigned long long a1, uint32_t fc,
+                                             const ModP &mp) {
+    const unsigned long long t = fold1(fold1(a0, fc) + fold1(a1, fc), fc);
+    const uint32_t u = (uint32_t)(madw((uint32_t)t * mp.pneg, mp.p, t) >> 32);
+    return min(u, u - mp.p);
+}
+
 // A row times the order's transform in registers (lane: column j and, CPL = 2,
-// column j + 32; f[k][t] = F[t][column k], d[k] its diagonal): x[k] the row's
-// residues of the lane's columns, g the row's residue at pivot column t = the
-// lane's index in its group of W2 lanes.  Two accumulators a column (even and odd
+// column j + 32; f[k][t] = F[t][column k], d[k] its diagonal, both in Montgomery form): x[k] the row's
+// residues of the lane's columns, gs the row's residues at the pivot columns (shared
+// memory, read 4 at a time by the whole group).  Two accumulators a column (even and odd
 // t), each folded after FOLDK of its own products.
 template <int TM, int CPL, int FOLDK>
-__device__ __forceinline__ void row_times(const uint32_t (&f)[CPL][TM], const uint32_t (&d)[CPL], int np, int W2,
-                                          const uint32_t (&x)[CPL], uint32_t g, uint32_t (&out)[CPL], uint32_t fc,
+__device__ __forceinline__ void row_times(const uint32_t (&f)[CPL][TM], const uint32_t (&d)[CPL], int m,
+                                          const uint32_t (&x)[CPL], const uint32_t *gs, uint32_t (&out)[CPL], uint32_t fc,
                                           const ModP &mp) {
     unsigned long long a0[CPL], a1[CPL];
 #pragma unroll
@@ -373,13 +396,14 @@ __device__ __forceinline__ void row_times(const uint32_t (&f)[CPL][TM], const ui
         a0[k] = (unsigned long long)d[k] * x[k];
         a1[k] = 0ull;
     }
-    // (f[k][t] = 0 from t = np on: whole groups of 8 without branches)
+    // (f[k][t] = 0 from the number of pivots on: whole groups of 8, and branches that only
+    // depend on a kernel argument)
 #pragma unroll
     for (int t0 = 0; t0 < TM; t0 += 8) {
-        if (TM == 8 || t0 < np) {
-            uint32_t v[8];
-#pragma unroll
-            for (int u = 0; u < 8; u++) v[u] = __shfl_sync(0xffffffffu, g, t0 + u, W2);
+        if (TM == 8 || t0 < m) {
+            const uint4 va = *reinterpret_cast<const uint4 *>(gs + t0);
+            const uint4 vb = *reinterpret_cast<const uint4 *>(gs + t0 + 4);
+            const uint32_t v[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
 #pragma unroll
             for (int u = 0; u < 8; u++) {
                 const int t = t0 + u;
@@ -396,9 +420,8 @@ __device__ __forceinline__ void row_times(const uint32_t (&f)[CPL][TM], const ui
             }
         }
     }
-    // folded, each is below p 2^32 + 2^32 <= 2^63: their sum fits
 #pragma unroll
-    for (int k = 0; k < CPL; k++) out[k] = red64(fold1(a0[k], fc) + fold1(a1[k], fc), mp);
+    for (int k = 0; k < CPL; k++) out[k] = redc_sum(a0[k], a1[k], fc, mp);
 }
 
 // The update of a pivot step on the lane's residues from k0 on: A[k] <- d A[k] -
@@ -426,15 +449,16 @@ __global__ void __launch_bounds__(lc_threads(MR), 1)
     constexpr int CL = EW * 32 / MR;        // column slots of the elimination
     constexpr int KR = QC / CL;             // residues a lane of the elimination (q <= QC)
     constexpr int TM = MR;                  // most pivots of an order
+    constexpr int PQ = QC + 1;              // odd pitch: the elimination's lanes are rows
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ uint32_t sm[];
     const int CS = (int)cluster_size(), rank = (int)cluster_rank();
-    const LcLayout l = lc_layout(m, q, bb, CS, MR);
+    const LcLayout l = lc_layout(m, q, bb, CS, MR, QC);
     uint32_t *Es = sm + l.Es;      // [bb][ma][q]
     uint32_t *Ml = sm + l.Ml;      // [2 bb + 1][mx][q]
     uint32_t *qt = sm + l.qt;      // [ma][q]
-    uint32_t *disc = sm + l.disc;  // [2][m][q], written by every block
-    uint32_t *Fs = sm + l.F;       // [2][m][q]
+    uint32_t *disc = sm + l.disc;  // [2][m][PQ], written by every block
+    uint32_t *Fs = sm + l.F;       // [2][MR][PQ]
     uint32_t *dgs = sm + l.dg;     // [2][64]
     uint32_t *FR = sm + l.FR;      // [q][MR + 1] frozen columns by position
     int *deg = (int *)(sm + l.ints);  // [64] degrees, local degrees (before and after the transform), offsets
@@ -443,8 +467,7 @@ __global__ void __launch_bounds__(lc_threads(MR), 1)
     int *rk = posc + 64;           // [64] position of each column
     int *kj = rk + 64;             // [64] pivots before the position's turn
     uint32_t *scum = (uint32_t *)(kj + 64);  // [64] column scales of the chunk (Montgomery form)
-    uint32_t *preN = scum + 64;    // [33] pre_t in normal form
-    uint32_t *preM = preN + 36;    // [33] pre_t in Montgomery form
+    uint32_t *preM = scum + 64;    // [33] pre_t in Montgomery form
     int *pr = (int *)(preM + 36);  // [32] pivot rows
     int *snap = pr + 32;           // [2][LC_SNAP]: sh, base, isp [64 each], pc [32], np, D
     int *dmx = snap + 2 * LC_SNAP; // [8]
@@ -454,9 +477,8 @@ __global__ void __launch_bounds__(lc_threads(MR), 1)
     int *degl_n = pmax + 36;       // [64]
     uint32_t *sck = (uint32_t *)(degl_n + 64);  // [64] the order's column scales (Montgomery form)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int mq = m * q;
+    const int mq = m * PQ;
     const uint32_t fc = mp.r1;  // 2^32 mod p
-    const int ma = (m - rank + CS - 1) / CS, mx = (q - rank + CS - 1) / CS;  // rows of this block (may be 0)
 
     for (int x = tid; x < bb * l.ma * q; x += NT) {
         const int c = x % q, al = x / q % l.ma, i = x / (q * l.ma), a = rank + CS * al;
@@ -467,7 +489,8 @@ __global__ void __launch_bounds__(lc_threads(MR), 1)
         }
         Es[x] = e;
     }
-    for (int x = tid; x < mq; x += NT) disc[x] = subm(E[x], qtop_g[x], mp);
+    for (int x = tid; x < 2 * MR * PQ; x += NT) Fs[x] = 0u;
+    for (int x = tid; x < m * q; x += NT) disc[x / q * PQ + x % q] = subm(E[x], qtop_g[x], mp);
     for (int x = tid; x < l.ma * q; x += NT) {
         const int a = rank + CS * (x / q);
         qt[x] = a < m ? qtop_g[a * q + x % q] : 0u;
@@ -524,13 +547,13 @@ __global__ void __launch_bounds__(lc_threads(MR), 1)
         // path below writes, through FR; returns the number of pivots.
         auto slow = [&](int i) -> int {
             const uint32_t *dc = disc + (i & 1) * mq;
-            uint32_t *F = Fs + (i & 1) * mq, *dg = dgs + (i & 1) * 64;
+            uint32_t *F = Fs + (i & 1) * MR * PQ, *dg = dgs + (i & 1) * 64;
             int *sn = snap + (i & 1) * LC_SNAP;
             uint32_t A[KR], y[KR];
 #pragma unroll
             for (int k = 0; k < KR; k++) {
                 const int pos = CL * k + slot;
-                A[k] = to_mont(dc[am * q + posc[min(pos, q - 1)]], mp);
+                A[k] = to_mont(dc[am * PQ + posc[min(pos, q - 1)]], mp);
                 if (pos >= q || a >= m) A[k] = 0u;
             }
             for (int c = tid; c < 64; c += NE) {
@@ -599,17 +622,14 @@ __global__ void __launch_bounds__(lc_threads(MR), 1)
             }
             esync();
             // the pivots' columns, local degrees and scales
-            for (int t = tid; t <= np; t += NE) {
-                preN[t] = from_mont(preM[t], mp);
-                if (t < np) {
-                    const int c = posc[ppos[t]];
-                    sn[192 + t] = c;
-                    pdl[t] = degl[c];
-                    sn[128 + c] = 1;
-                }
+            for (int t = tid; t < np; t += NE) {
+                const int c = posc[ppos[t]];
+                sn[192 + t] = c;
+                pdl[t] = degl[c];
+                sn[128 + c] = 1;
             }
             esync();
-            // publish the transform (normal form) and the local degree bounds
+            // publish the transform (Montgomery form) and the local degree bounds
             for (int c0 = 0; c0 < q; c0 += NE / parts) {
                 const int j = c0 + tid / parts;
                 if (j < q) {
@@ -617,16 +637,16 @@ __global__ void __launch_bounds__(lc_threads(MR), 1)
                     const uint32_t *fj = FR + pj * (MR + 1);
                     int dl = 0;
 #pragma unroll 4
-                    for (int t = part; t < np; t += parts) {
-                        const uint32_t x = mont_mul(fj[pr[t]], preN[t], mp);
+                    for (int t = part; t < m; t += parts) {  // (rows from np on: zero)
+                        const bool is = t < np;
+                        const uint32_t x = mont_mul(fj[is ? pr[t] : 0], is ? preM[t] : 0u, mp);
                         const uint32_t v = t < kk ? x : 0u;
-                        F[t * q + j] = v != 0u ? mp.p - v : 0u;
+                        F[t * PQ + j] = v != 0u ? mp.p - v : 0u;
                         dl = max(dl, v != 0u ? pdl[t] : 0);
                     }
                     if (dl > 0) atomicMax(&dln[j], dl);
                     if (part == 0) {
-                        dg[j] = preN[kk];
-                        sck[j] = preM[kk];
+                        dg[j] = sck[j] = preM[kk];
                     }
                 }
             }
@@ -634,71 +654,125 @@ __global__ void __launch_bounds__(lc_threads(MR), 1)
         };
         for (int i = 0; i < bb; i++) {
             const uint32_t *dc = disc + (i & 1) * mq;
-            uint32_t *F = Fs + (i & 1) * mq, *dg = dgs + (i & 1) * 64;
+            uint32_t *F = Fs + (i & 1) * MR * PQ, *dg = dgs + (i & 1) * 64;
             int *sn = snap + (i & 1) * LC_SNAP;
             uint32_t A[KR], y[KR];
             int col[KR];  // the lane's columns
 #pragma unroll
             for (int k = 0; k < KR; k++) {
                 col[k] = posc[min(CL * k + slot, q - 1)];
-                A[k] = to_mont(dc[am * q + col[k]], mp);
+                A[k] = to_mont(dc[am * PQ + col[k]], mp);
                 if (CL * k + slot >= q || a >= m) A[k] = 0u;
             }
             int np = m;
+            // the snapshot's pivots, if nothing vanishes (else the slow path writes its own)
+            for (int c = tid; c < q; c += NE) sn[128 + c] = rk[c] < m ? 1 : 0;
+            if (tid < m) sn[192 + tid] = posc[tid];
+            if (tid == 0) {
+                sn[224] = m;
+                sn[225] = D;
+            }
             // Straight through: position t becomes pivot t with row t its pivot row, as it
             // does unless residues vanish.  Registers keep a column's values from its turn
             // on, so a lane holds row a of every column it has: F and the scales come from
             // registers, with pre_a kept as the lane's own.
             uint32_t pre = mp.r1, pre_a = mp.r1;
             bool bad = m > q;
+            if constexpr (EW == 1) {
 #pragma unroll
-            for (int g = 0; g < MR / CL; g++) {
+                for (int g = 0; g < MR / CL; g++) {
 #pragma unroll
-                for (int s = 0; s < CL; s++) {
-                    const int t = CL * g + s;
-                    if (t < m) {  // (the same for all)
-                        uint32_t v, d;
+                    for (int s = 0; s < CL; s++) {
+                        const int t = CL * g + s;
+                        if (t < m) {  // (the same for all)
 #pragma unroll
-                        for (int k = g; k < KR; k++) y[k] = __shfl_sync(FULL, A[k], t, MR);
-                        if constexpr (EW == 1) {
-                            v = __shfl_sync(FULL, A[g], s * MR + a);
-                            d = __shfl_sync(FULL, A[g], s * MR + t);
-                        } else {
-                            uint32_t *fr = FR + (t & 1) * MR;  // (two slots: a barrier apart)
-                            if (slot == s) fr[a] = A[g];
-                            esync();
-                            v = fr[a];
-                            d = fr[t];
+                            for (int k = g; k < KR; k++) y[k] = __shfl_sync(FULL, A[k], t, MR);
+                            const uint32_t v = __shfl_sync(FULL, A[g], s * MR + a);
+                            const uint32_t d = __shfl_sync(FULL, A[g], s * MR + t);
+                            bad |= d == 0u;
+                            const uint32_t nv = v != 0u ? mp.p - v : 0u;
+                            const uint32_t keep = A[g];
+                            pivot_step(A, y, g, d, nv, a != t, mp.p, mp.pneg);
+                            if (slot <= s) A[g] = keep;
+                            pre_a = a == t ? pre : pre_a;
+                            pre = mont_mul(pre, d, mp);
                         }
-                        bad |= d == 0u;
-                        const uint32_t nv = v != 0u ? mp.p - v : 0u;
-                        const uint32_t keep = A[g];
-                        pivot_step(A, y, g, d, nv, a != t, mp.p, mp.pneg);
-                        if (slot <= s) A[g] = keep;
-                        pre_a = a == t ? pre : pre_a;
-                        pre = mont_mul(pre, d, mp);
+                    }
+                }
+            } else {
+                // A group of CL columns (one of each slot) at a time.  Its steps change one
+                // residue r of a lane: its column's until the column's turn, from then on the
+                // coefficients G of that pivot row in the group's transform.  The later
+                // columns take the whole transform at once,
+                //   row a <- (a a pivot row of the group ? 0 : sg) row a + sum_t G_t[a] row t,
+                // sg the product of the group's pivots: 9 products and one reduction instead
+                // of 8 steps of two products and a reduction each.
+#pragma unroll
+                for (int g = 0; g < MR / CL; g++) {
+                    const int ns = min(CL, m - CL * g);
+                    if (ns > 0) {  // (the same for all)
+                        uint32_t r = A[g], sg = mp.r1, sg_a = mp.r1;
+#pragma unroll 1
+                        for (int s = 0; s < ns; s++) {
+                            const int t = CL * g + s;
+                            uint32_t *fr = FR + (t & 1) * MR;  // (two slots: a barrier apart)
+                            uint32_t yr[1] = {__shfl_sync(FULL, r, t, MR)};
+                            if (slot == s) {
+                                fr[a] = r;
+                                A[g] = r;
+                                yr[0] = sg;
+                                r = a == t ? sg : 0u;
+                            }
+                            esync();
+                            const uint32_t v = fr[a], d = fr[t];
+                            bad |= d == 0u;
+                            const uint32_t nv = v != 0u ? mp.p - v : 0u;
+                            uint32_t rr[1] = {r};
+                            pivot_step(rr, yr, 0, d, nv, a != t, mp.p, mp.pneg);
+                            r = rr[0];
+                            sg_a = a == t ? sg : sg_a;
+                            sg = mont_mul(sg, d, mp);
+                        }
+                        uint32_t *Gs = FR + 2 * MR;  // [CL][MR] (q >= 10 columns of MR + 1 words)
+                        if (slot >= ns) A[g] = r;
+                        Gs[slot * MR + a] = slot < ns ? r : 0u;
+                        if (a / CL == g && a < m) pre_a = mont_mul(pre, sg_a, mp);
+                        const uint32_t dg0 = a / CL == g && a < m ? 0u : sg;
+                        pre = mont_mul(pre, sg, mp);
+                        esync();
+                        uint32_t G[CL];
+#pragma unroll
+                        for (int u = 0; u < CL; u++) G[u] = Gs[u * MR + a];
+#pragma unroll
+                        for (int k = g + 1; k < KR; k++) {
+                            unsigned long long a0 = (unsigned long long)dg0 * A[k], a1 = 0ull;
+#pragma unroll
+                            for (int u = 0; u < CL; u++) {
+                                const uint32_t yk = __shfl_sync(FULL, A[k], min(CL * g + u, MR - 1), MR);
+                                if ((u & 1) == 0) {
+                                    a0 = madw(G[u], yk, a0);
+                                    if ((u / 2 + 2) % FOLDK == 0) a0 = fold1(a0, fc);
+                                } else {
+                                    a1 = madw(G[u], yk, a1);
+                                    if (((u + 1) / 2) % FOLDK == 0) a1 = fold1(a1, fc);
+                                }
+                            }
+                            A[k] = redc_sum(a0, a1, fc, mp);
+                        }
                     }
                 }
             }
             if (!bad) {
-                const uint32_t pa = from_mont(pre_a, mp), pm = from_mont(pre, mp);
 #pragma unroll
                 for (int k = 0; k < KR; k++) {
                     const int pos = CL * k + slot, kk = min(pos, m);
                     if (pos < q && a < m) {
-                        const uint32_t v = mont_mul(A[k], pa, mp);
-                        F[a * q + col[k]] = a < kk && v != 0u ? mp.p - v : 0u;
+                        const uint32_t v = mont_mul(A[k], pre_a, mp);
+                        F[a * PQ + col[k]] = a < kk && v != 0u ? mp.p - v : 0u;
                         if (a == (pos < m ? pos : 0)) {
-                            dg[col[k]] = pos < m ? pa : pm;
-                            sck[col[k]] = pos < m ? pre_a : pre;
+                            dg[col[k]] = sck[col[k]] = pos < m ? pre_a : pre;
                         }
                     }
-                }
-                for (int c = tid; c < q; c += NE) sn[128 + c] = rk[c] < m ? 1 : 0;
-                if (tid < m) sn[192 + tid] = posc[tid];
-                if (tid == 0) {
-                    sn[224] = m;
-                    sn[225] = D;
                 }
             } else {
                 np = slow(i);
@@ -747,13 +821,15 @@ __global__ void __launch_bounds__(lc_threads(MR), 1)
         int W2 = 1;
         while (W2 < q && W2 < 32) W2 <<= 1;
         const int rpw = 32 / W2, grp = lane / W2, col = lane % W2;
-        const int NG = NWK * rpw, gg = ow * rpw + grp;  // row groups, this group's first row
+        const int NG = NWK * rpw;          // rows at a time
+        uint32_t *gs = sm + l.gs + (ow * rpw + grp) * max(W2, TM);  // the group's pivot residues
+        const int wq = l.ma * q, xq = l.mx * q;
         bool cok[CPL];
 #pragma unroll
         for (int k = 0; k < CPL; k++) cok[k] = col + 32 * k < q;
         for (int i = 0; i < bb; i++) {
             named_sync(BAR_T0 + (i & 1), NE + 32 * NWK);
-            const uint32_t *F = Fs + (i & 1) * mq, *dg = dgs + (i & 1) * 64;
+            const uint32_t *F = Fs + (i & 1) * MR * PQ, *dg = dgs + (i & 1) * 64;
             const int *sn = snap + (i & 1) * LC_SNAP;
             const int np = sn[224], D = sn[225];
             uint32_t f[CPL][TM], d[CPL];
@@ -767,98 +843,63 @@ __global__ void __launch_bounds__(lc_threads(MR), 1)
                 bsc[k] = cok[k] ? sn[64 + j] : 0;
                 isp[k] = cok[k] && sn[128 + j] != 0;
 #pragma unroll
-                for (int t = 0; t < TM; t++) f[k][t] = (t < np && cok[k]) ? F[t * q + j] : 0u;
+                for (int t = 0; t < TM; t++) f[k][t] = F[t * PQ + (cok[k] ? j : 0)];
             }
             // lane t of a group fetches the row's residue at pivot column t
             const bool pok = col < np;
             const int pc = pok ? sn[192 + col] : 0;
             const int shp = pok ? sn[pc] : 0, bsp = pok ? sn[64 + pc] : 0;
-            // one row: rp[k] the lane's columns, gp its pivot column (when ok); x[k] the new residues
-            auto row = [&](bool ok, uint32_t *const (&rp)[CPL], const uint32_t *gp, uint32_t (&x)[CPL]) {
-                uint32_t v[CPL];
+            // word offsets of the lane's columns (ad*) and its pivot column (pd*) in row 0 of
+            // the window, of Ml and of Qtop
+            int adW[CPL], adM[CPL];
 #pragma unroll
-                for (int k = 0; k < CPL; k++) v[k] = ok && cok[k] ? *rp[k] : 0u;
-                const uint32_t g = ok && pok ? *gp : 0u;
-                row_times<TM, CPL, FOLDK>(f, d, np, W2, v, g, x, fc, mp);
-                __syncwarp();
-            };
-            auto es_at = [&](int ip, int al, int s, int c) { return Es + ((size_t)(ip - s) * l.ma + al) * q + c; };
-            // the next discrepancy: rows i and i + 1, to every block
-            if (i + 1 < bb) {
-                uint32_t *dn = disc + ((i + 1) & 1) * mq;
-                for (int r0 = ow * rpw; r0 < 2 * ma; r0 += NG) {
-                    // row i of a (its pivot columns) or row i + 1 (the others)
-                    const int al = (r0 + grp) >> 1, h = (r0 + grp) & 1;
-                    const bool ok = al < ma;
-                    uint32_t *rp[CPL], x[CPL];
+            for (int k = 0; k < CPL; k++) {
+                adW[k] = l.Es + col + 32 * k - shc[k] * wq;
+                adM[k] = l.Ml + col + 32 * k + bsc[k] * xq;
+            }
+            const int pdW = l.Es + pc - shp * wq, pdM = l.Ml + pc + bsp * xq, pdQ = l.qt + pc;
+            // Pass 0: the next discrepancy, window rows i and i + 1, to every block.  Pass 1,
+            // beside the next elimination: the window's later rows, Qtop (the next one keeps
+            // the pivot columns of Qtop T), Ml's coefficients 0 .. D.  One loop over all the
+            // rows (those past m or q are zero and stay so): one copy of the product's code.
+            uint32_t *dn = disc + ((i + 1) & 1) * mq;
+#pragma unroll 1
+            for (int ps = 0; ps < 2; ps++) {
+                const int w0 = (i + 2 * ps) * l.ma;
+                const int nw = ps == 0 ? (i + 1 < bb ? 2 * l.ma : 0) : max(bb - i - 2, 0) * l.ma;
+                const int nq = nw + (ps == 0 ? 0 : l.ma);
+                const int nr = nq + (ps == 0 || np == 0 ? 0 : (D + 1) * l.mx);
+#pragma unroll 1
+                for (int r0 = ow * rpw; r0 < nr; r0 += NG) {
+                    const int r = r0 + grp;
+                    const bool ok = r < nr, inw = r < nw, inm = r >= nq;
+                    const int row = (inw ? w0 + r : (inm ? r - nq : r - nw)) * q;
+                    uint32_t *rp[CPL], v[CPL], x[CPL];
 #pragma unroll
-                    for (int k = 0; k < CPL; k++) rp[k] = es_at(i + h, al, shc[k], col + 32 * k);
-                    row(ok, rp, es_at(i + h, al, shp, pc), x);
+                    for (int k = 0; k < CPL; k++) {
+                        rp[k] = sm + row + (inw ? adW[k] : (inm ? adM[k] : l.qt + col + 32 * k));
+                        v[k] = ok && cok[k] ? *rp[k] : 0u;
+                    }
+                    if (pok) gs[col] = ok ? sm[row + (inw ? pdW : (inm ? pdM : pdQ))] : 0u;
+                    __syncwarp();
+                    row_times<TM, CPL, FOLDK>(f, d, m, v, gs, x, fc, mp);
+                    __syncwarp();
+                    const int h = r >= l.ma ? 1 : 0, ar = rank + CS * (r - h * l.ma);  // (pass 0)
 #pragma unroll
                     for (int k = 0; k < CPL; k++) {
                         if (ok && cok[k]) {
-                            *rp[k] = x[k];
-                            if (isp[k] == (h == 0)) {
-                                uint32_t *dst = dn + (rank + CS * al) * q + col + 32 * k;
+                            *rp[k] = inw || inm || isp[k] ? x[k] : 0u;
+                            // row i's pivot columns, row i + 1's others
+                            if (ps == 0 && ar < m && isp[k] == (h == 0)) {
+                                uint32_t *dst = dn + ar * PQ + col + 32 * k;
                                 for (int b = 0; b < CS; b++) st_cluster(dst, (uint32_t)b, x[k]);
                             }
                         }
                     }
                 }
+                __syncwarp();
+                if (ps == 0) cluster_arrive();
             }
-            __syncwarp();
-            cluster_arrive();
-            // window orders i + 2 .. bb - 1
-            if (np > 0 && ma > 0) {
-                const int rows = (bb - i - 2) * ma;
-                const int stepi = NG / ma, stepa = NG - stepi * ma;
-                int ip = i + 2 + gg / ma, al = gg % ma;
-                for (int r0 = ow * rpw; r0 < rows; r0 += NG) {
-                    const bool ok = r0 + grp < rows;
-                    uint32_t *rp[CPL], x[CPL];
-#pragma unroll
-                    for (int k = 0; k < CPL; k++) rp[k] = es_at(ip, al, shc[k], col + 32 * k);
-                    row(ok, rp, es_at(ip, al, shp, pc), x);
-#pragma unroll
-                    for (int k = 0; k < CPL; k++)
-                        if (ok && cok[k]) *rp[k] = x[k];
-                    ip += stepi;
-                    al += stepa;
-                    if (al >= ma) { al -= ma; ip++; }
-                }
-            }
-            // Qtop; the next one keeps the pivot columns of Qtop T
-            for (int r0 = ow * rpw; r0 < ma; r0 += NG) {
-                const int al = r0 + grp;
-                const bool ok = al < ma;
-                uint32_t *rp[CPL], x[CPL];
-#pragma unroll
-                for (int k = 0; k < CPL; k++) rp[k] = qt + al * q + col + 32 * k;
-                row(ok, rp, qt + al * q + pc, x);
-#pragma unroll
-                for (int k = 0; k < CPL; k++)
-                    if (ok && cok[k]) *rp[k] = isp[k] ? x[k] : 0u;
-            }
-            // Ml coefficients 0 .. D
-            if (np > 0 && mx > 0) {
-                const int rows = (D + 1) * mx;
-                const int steps = NG / mx, stepx = NG - steps * mx;
-                int s = gg / mx, xl = gg % mx;
-                for (int r0 = ow * rpw; r0 < rows; r0 += NG) {
-                    const bool ok = r0 + grp < rows;
-                    uint32_t *rp[CPL], x[CPL];
-#pragma unroll
-                    for (int k = 0; k < CPL; k++) rp[k] = Ml + ((size_t)(bsc[k] + s) * l.mx + xl) * q + col + 32 * k;
-                    row(ok, rp, Ml + ((size_t)(bsp + s) * l.mx + xl) * q + pc, x);
-#pragma unroll
-                    for (int k = 0; k < CPL; k++)
-                        if (ok && cok[k]) *rp[k] = x[k];
-                    s += steps;
-                    xl += stepx;
-                    if (xl >= mx) { xl -= mx; s++; }
-                }
-            }
-            __syncwarp();
             cluster_wait();
         }
     }
@@ -1045,8 +1086,47 @@ static wr_status mbasis_run(wr_ctx *ctx, const uint32_t *d_S, int64_t L, int m, 
 
     // chunk size b and tiles: every kernel's shared memory must fit
     const size_t budget = std::min<size_t>(ctx->smem_optin, 227 * 1024) - 1024;
-    const int MR = m <= 8 ? 8 : (m <= 16 ? 16 : 32), CS = local_cluster(q);
-    auto local_need = [&](int b) { return sizeof(uint32_t) * (size_t)lc_layout(m, q, b, CS, MR).total; };
+    const int MR = m <= 8 ? 8 : (m <= 16 ? 16 : 32);
+    int CS = local_cluster(q);
+    const int QC = MR == 8 ? (q <= 16 ? 16 : (q <= 32 ? 32 : 40)) : (q <= 32 ? 32 : (MR == 16 ? 48 : 64));
+    const bool big = p > (1u << 30);  // fold1_products: 4 products, else 12
+    using LocalFn = void (*)(int, int, int, const uint32_t *, uint32_t *, int32_t *, uint32_t *, int32_t *, int *,
+                             uint32_t *, int, ModP);
+    LocalFn kloc = nullptr;
+#define WR_LOCAL(MRV, CPLV, QCV) kloc = big ? k_local<MRV, CPLV, QCV, 4> : k_local<MRV, CPLV, QCV, 12>
+    if (MR == 8) { if (QC == 16) WR_LOCAL(8, 1, 16); else if (QC == 32) WR_LOCAL(8, 1, 32); else WR_LOCAL(8, 2, 40); }
+    else if (MR == 16) { if (QC == 32) WR_LOCAL(16, 1, 32); else WR_LOCAL(16, 2, 48); }
+    else { if (QC == 32) WR_LOCAL(32, 1, 32); else WR_LOCAL(32, 2, 64); }
+#undef WR_LOCAL
+    WR_CUDA(cudaFuncSetAttribute(kloc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
+    auto local_config = [&](size_t smem, cudaLaunchAttribute &at) {
+        cudaLaunchConfig_t lc{};
+        at = cudaLaunchAttribute{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)CS;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        lc.gridDim = dim3((unsigned)CS);
+        lc.blockDim = dim3((unsigned)lc_threads(MR));
+        lc.dynamicSmemBytes = smem;
+        lc.stream = s;
+        lc.attrs = &at;
+        lc.numAttrs = 1;
+        return lc;
+    };
+    if (CS > 8) {
+        // more than the portable size: where the device can place such a cluster at all
+        cudaLaunchAttribute at;
+        int fit = 0;
+        if (cudaFuncSetAttribute(kloc, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            [&] {
+                const cudaLaunchConfig_t lc = local_config(budget, at);
+                return cudaOccupancyMaxActiveClusters(&fit, kloc, &lc);
+            }() != cudaSuccess || fit < 1) {
+            cudaGetLastError();
+            CS = 8;
+        }
+    }
+    auto local_need = [&](int b) { return sizeof(uint32_t) * (size_t)lc_layout(m, q, b, CS, MR, QC).total; };
     int bmax = ctx->sigma_chunk > 0 ? std::min(ctx->sigma_chunk, 64) : sigma_chunk_default(q);
     while (bmax > 1 && local_need(bmax) > budget) bmax--;
     if (local_need(bmax) > budget) return fail(WR_EINVAL, "block sizes too large for shared memory");
@@ -1063,21 +1143,11 @@ static wr_status mbasis_run(wr_ctx *ctx, const uint32_t *d_S, int64_t L, int m, 
         WR_CUDA(cudaMemcpyAsync(scale.ptr, one.data(), sizeof(uint32_t) * q, cudaMemcpyHostToDevice, s));
         WR_CUDA(cudaStreamSynchronize(s));
     }
-    const bool big = p > (1u << 30);  // fold1_products: 4 products, else 12
     auto *ktoep = NC == 16 ? (big ? k_toeplitz<16, 4> : k_toeplitz<16, 8>)
                   : NC == 32 ? (big ? k_toeplitz<32, 4> : k_toeplitz<32, 8>)
                              : (big ? k_toeplitz<64, 4> : k_toeplitz<64, 8>);
     DevBuf Esum;
     WR_TRY(dev_alloc(ctx, Esum, sizeof(uint32_t) * (size_t)bmax * m * q));
-    using LocalFn = void (*)(int, int, int, const uint32_t *, uint32_t *, int32_t *, uint32_t *, int32_t *, int *,
-                             uint32_t *, int, ModP);
-    LocalFn kloc = nullptr;
-#define WR_LOCAL(MRV, CPLV, QCV) kloc = big ? k_local<MRV, CPLV, QCV, 4> : k_local<MRV, CPLV, QCV, 12>
-    if (MR == 8) { if (q <= 16) WR_LOCAL(8, 1, 16); else if (q <= 32) WR_LOCAL(8, 1, 32); else WR_LOCAL(8, 2, 40); }
-    else if (MR == 16) { if (q <= 32) WR_LOCAL(16, 1, 32); else WR_LOCAL(16, 2, 48); }
-    else { if (q <= 32) WR_LOCAL(32, 1, 32); else WR_LOCAL(32, 2, 64); }
-#undef WR_LOCAL
-    WR_CUDA(cudaFuncSetAttribute(kloc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget));
 
     uint32_t *Pcur = d_P, *Pnext = P2.as<uint32_t>();
     int64_t Dbound = 1;
@@ -1156,17 +1226,8 @@ static wr_status mbasis_run(wr_ctx *ctx, const uint32_t *d_S, int64_t L, int m, 
         }
         if (prof) WR_CUDA(cudaEventRecord(pe[1], s));
         {
-            cudaLaunchConfig_t lc{};
-            cudaLaunchAttribute at{};
-            at.id = cudaLaunchAttributeClusterDimension;
-            at.val.clusterDim.x = (unsigned)CS;
-            at.val.clusterDim.y = at.val.clusterDim.z = 1;
-            lc.gridDim = dim3((unsigned)CS);
-            lc.blockDim = dim3((unsigned)lc_threads(MR));
-            lc.dynamicSmemBytes = local_need(bb);
-            lc.stream = s;
-            lc.attrs = &at;
-            lc.numAttrs = 1;
+            cudaLaunchAttribute at;
+            const cudaLaunchConfig_t lc = local_config(local_need(bb), at);
             WR_CUDA(cudaLaunchKernelEx(&lc, kloc, m, q, bb, Ewin, qtop.as<uint32_t>(), d_deg, Ml.as<uint32_t>(),
                                        degl.as<int32_t>(), dmax.as<int>(), scale.as<uint32_t>(), dbase, mp));
         }

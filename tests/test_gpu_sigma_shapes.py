@@ -65,3 +65,15 @@ def test_discrepancies_that_lose_rank_in_some_orders(wr, ctx, m, n):
     _check(wr, ctx, S, p)
     S[:, m - 1] = S[:, 0]  # one row of X twice: never full rank
     _check(wr, ctx, S, p)
+
+
+@pytest.mark.parametrize("m,n", [(9, 9), (12, 6), (15, 20), (17, 17), (23, 10), (24, 24), (25, 7), (30, 31)])
+@pytest.mark.parametrize("p", [1073741789, 2147483647])
+def test_groups_of_pivot_columns(wr, ctx, m, n, p):
+    """m around multiples of the elimination's groups of eight, both primes' folds, and
+    residues at the ends of their range."""
+    rng = np.random.default_rng(m)
+    S = rng.choice(np.array([p - 1, p - 2, 1, p // 2, 12345]), size=(20, m, n)).astype(np.uint32)
+    _check(wr, ctx, S, p)
+    S = rng.integers(p - 50, p, size=(35, m, n)).astype(np.uint32)
+    _check(wr, ctx, S, p)
