@@ -220,9 +220,9 @@ wr_status wr_set_projection_overlap(wr_ctx *ctx, int32_t on);
  * dot-product step): 1 = the tensor cores, 0 = 64-bit integer multiply-adds,
  * -1 (default) = the tensor cores for blocks of 16 columns and more (m, n >=
  * 16), the integer path below.  The tensor-core path is exact: every residue
- * is split into four balanced 8-bit digits (bf16 values), tcgen05 MMAs sum the
- * 16 digit products per residue product in fp32 over at most 512 rows (every
- * partial sum an integer below 2^23), and the sums are drained into int64 and
+ * is its four bytes (each an fp16 subnormal), tcgen05 MMAs sum the 16 digit
+ * products per residue product in fp32 over at most 256 rows (every partial
+ * sum below 2^24 units), and the sums are drained into int32 sums and
  * recombined mod p.  The result is the same bit for bit either way. */
 wr_status wr_set_tensor_projection(wr_ctx *ctx, int32_t mode);
 /* Column slabs of the SpMM passes (Section 4 names reordering for locality;

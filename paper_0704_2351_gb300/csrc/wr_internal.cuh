@@ -552,7 +552,7 @@ wr_status validate_csr(wr_ctx *ctx, int64_t rows, int64_t cols, int64_t nnz, con
                        const int32_t *d_colidx, const int32_t *d_vals, bool *wide);
 wr_status exclusive_scan_i64(wr_ctx *ctx, const int64_t *d_in, int64_t *d_out, int64_t n);
 
-// Several jobs on one matrix in one SpMM pass (wr_multi.cu): the block holds
+// Several jobs on one matrix in one SpMM pass (run_sequence_multi): the block holds
 // `jobs` slices of 2^jw_log columns side by side, slice g reduced modulo
 // mp[g] and scaled by scale[g] in the epilogue (the exact int64 row sums do
 // not depend on the prime).

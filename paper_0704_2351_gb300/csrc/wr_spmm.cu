@@ -626,7 +626,7 @@ static int64_t max_split(const Sell &S, const std::vector<Sell> *slabs) {
 }
 
 // A Gram projection S_raw[tmul * counter + toff] += sum_r w_r t[r][0..m)^T
-// t[r][yoff..yoff+n): on the tensor cores (bf16 digit products, exact) when
+// t[r][yoff..yoff+n): on the tensor cores (fp16 digit products, exact) when
 // the context asks for them, or automatically for blocks of 16 columns and
 // more; otherwise with 64-bit integer multiply-adds.  Same result either way.
 static bool use_tc_gram(const wr_ctx *ctx, int m, int n, int tstride, int yoff) {
