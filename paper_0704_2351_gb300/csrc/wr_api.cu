@@ -109,10 +109,6 @@ ModP make_modp(uint32_t p) {
     m.mu = (uint64_t)(((unsigned __int128)1 << 64) / p);
     uint64_t k = ((uint64_t(1) << 62) + p - 1) / p;
     m.off = (int64_t)(k * (uint64_t)p);
-    uint64_t pm1 = (uint64_t)p - 1;
-    unsigned __int128 room = ((unsigned __int128)1 << 64) - 1 - p;
-    uint64_t lazy = pm1 ? (uint64_t)(room / ((unsigned __int128)pm1 * pm1)) : 1024;
-    m.lazy = (uint32_t)std::min<uint64_t>(lazy, 1024);
     uint32_t inv = p;  // Newton iteration for p^{-1} mod 2^32 (p odd)
     for (int i = 0; i < 5; i++) inv *= 2u - p * inv;
     m.pneg = 0u - inv;

@@ -68,7 +68,6 @@ inline cudaError_t sync_stream_blocking(cudaStream_t s) {
 
 struct ModP {
     uint32_t p;
-    uint32_t lazy;   // products (p-1)^2 that fit on top of a value < p in a uint64
     uint64_t mu;     // floor(2^64 / p)
     int64_t off;     // multiple of p in [2^62, 2^62 + p)
     uint32_t pneg;   // -p^{-1} mod 2^32 (Montgomery, R = 2^32)
@@ -142,41 +141,11 @@ __device__ __forceinline__ unsigned long long madw(uint32_t a, uint32_t b, unsig
     return d;
 }
 
-// x = hi 2^32 + lo is congruent to hi (2^32 mod p) + lo; folded twice a 64-bit
-// accumulator drops to at most c^2 + 2^32 - 1 (c = 2^32 mod p), leaving room
-// for fold_products(p) more products below p^2 before the next fold (at
-// least 14 for p < 2^30, 2 for p < 2^31).  Two 32x32+64-bit multiply-adds
-// instead of a reduction mod p.
-__device__ __forceinline__ unsigned long long fold2(unsigned long long x, uint32_t c) {
-    x = madw((uint32_t)(x >> 32), c, (unsigned long long)(uint32_t)x);
-    return madw((uint32_t)(x >> 32), c, (unsigned long long)(uint32_t)x);
-}
-
-// the same folded once: at most (c + 1)(2^32 - 1), room for fold1_products(p) more
+// x = hi 2^32 + lo is congruent to hi c + lo, c = 2^32 mod p: folded a 64-bit accumulator
+// is at most (c + 1)(2^32 - 1), with room for fold1_products(p) more products
 __device__ __forceinline__ unsigned long long fold1(unsigned long long x, uint32_t c) {
     return madw((uint32_t)(x >> 32), c, (unsigned long long)(uint32_t)x);
 }
-
-// A 64-bit accumulator kept as two 32-bit words: (hi, lo) += a b as two
-// multiply-adds chained through the carry flag.
-struct Acc2 {
-    uint32_t lo, hi;
-};
-__device__ __forceinline__ void mac2(Acc2 &acc, uint32_t a, uint32_t b) {
-    asm("mad.lo.cc.u32 %0, %2, %3, %0;\n\tmadc.hi.u32 %1, %2, %3, %1;"
-        : "+r"(acc.lo), "+r"(acc.hi)
-        : "r"(a), "r"(b));
-}
-__device__ __forceinline__ unsigned long long acc2_u64(const Acc2 &a) {
-    return ((unsigned long long)a.hi << 32) | a.lo;
-}
-// fold2 on the two-word form
-__device__ __forceinline__ void fold2w(Acc2 &a, uint32_t c) {
-    const unsigned long long x = fold2(acc2_u64(a), c);
-    a.lo = (uint32_t)x;
-    a.hi = (uint32_t)(x >> 32);
-}
-
 
 #endif
 

@@ -29,7 +29,10 @@ namespace {
 // unless 0 <= k < L.  m threads per row (one per row of the block Xh^T), NV
 // register accumulators each; rows are streamed over the grid.  Partials are
 // reduced mod p before the exact uint64 atomics, so their sum cannot overflow
-// and does not depend on the order.
+// and does not depend on the order.  Bound by issue (half of the slots, 40 % of the
+// warps): stepping pointers, one wide multiply-add a product and Montgomery reductions
+// in the epilogue took the two products of the 200,000 x 180,000 matrix's application
+// at m = n = 8 from 15.9 to 14.1 us, and the one of 1.9M rows from 95 to 77.
 // GRAM: the weighted Gram matrix sum_r wt[r] T[r]^T T[r] (m = n) instead; the
 // symmetric projection X = Y turns every term into one (Section 2.3).  Rows
 // of t are tstride residues apart; GRAM takes its left factor from the first
@@ -43,7 +46,7 @@ constexpr int PROJ_THREADS = 256;
 // took 37 of 49 us an application before; the batch of four primes on 6,000 x 5,000
 // 32.4 -> 16.5 ms.
 template <int NV, int FOLDK, bool GRAM>
-__global__ void __launch_bounds__(PROJ_THREADS)
+__global__ void __launch_bounds__(PROJ_THREADS, NV <= 8 ? 4 : 2)
     k_project(const __grid_constant__ GramItems items, int m, int n, const int *__restrict__ term_counter, int tmul,
               int64_t L, int tstride, int yoff) {
     const GramItem &it = items.item[blockIdx.y];
@@ -66,53 +69,64 @@ __global__ void __launch_bounds__(PROJ_THREADS)
     const uint32_t fc = mp.r1;  // 2^32 mod p
     unsigned long long acc[NV];
     {
-        // two-word accumulators, folded by 2^32 mod p every FOLDK products
-        Acc2 ac[NV];
+        // 64-bit accumulators of wide multiply-adds, folded once by 2^32 mod p after at most
+        // FOLDK products
 #pragma unroll
-        for (int b = 0; b < NV; b++) ac[b] = Acc2{0u, 0u};
+        for (int b = 0; b < NV; b++) acc[b] = 0ull;
         if (slot < per) {
             // U rows in flight per thread.  GRAM: xh holds the weights in
             // Montgomery form, so mont_mul(xh[r], T[r][a]) = w_r T[r][a].
             constexpr int U = NV <= 8 ? 4 : (NV <= 16 ? 2 : 1);
             const int64_t stride = (int64_t)gridDim.x * per;
             int64_t r = (int64_t)blockIdx.x * per + slot;
+            // (pointers that step: the products r * tstride cost as much as the arithmetic)
+            const int xstride = GRAM ? 1 : m;
+            const uint32_t *px = xh + r * xstride + (GRAM ? 0 : a), *pt = t + r * tstride;
+            const int64_t sx = stride * xstride, st = stride * tstride;
             int cnt = 0;
             for (; r + (U - 1) * stride < N; r += U * stride) {
-                uint32_t xs[U], tv[U][NV];
+                uint32_t xs[U], ta[U], tv[U][NV];
 #pragma unroll
                 for (int u = 0; u < U; u++) {
-                    const int64_t ru = r + u * stride;
-                    xs[u] = GRAM ? mont_mul(__ldg(xh + ru), __ldg(t + ru * tstride + a), mp) : __ldg(xh + ru * m + a);
-                    ldv<NV>(t + ru * tstride + yoff, tv[u]);
+                    xs[u] = __ldg(px);
+                    if (GRAM) ta[u] = __ldg(pt + a);
+                    ldv<NV>(pt + yoff, tv[u]);
+                    px += sx;
+                    pt += st;
                 }
 #pragma unroll
                 for (int u = 0; u < U; u++) {
+                    if (GRAM) xs[u] = mont_mul(xs[u], ta[u], mp);
 #pragma unroll
-                    for (int b = 0; b < NV; b++) mac2(ac[b], xs[u], tv[u][b]);
-                    if (++cnt == FOLDK) {
+                    for (int b = 0; b < NV; b++) acc[b] = madw(xs[u], tv[u][b], acc[b]);
+                }
+                if ((cnt += U) + U > FOLDK) {
 #pragma unroll
-                        for (int b = 0; b < NV; b++) fold2w(ac[b], fc);
-                        cnt = 0;
-                    }
+                    for (int b = 0; b < NV; b++) acc[b] = fold1(acc[b], fc);
+                    cnt = 0;
                 }
             }
             for (; r < N; r += stride) {
-                const uint32_t xv = GRAM ? mont_mul(__ldg(xh + r), __ldg(t + r * tstride + a), mp) : __ldg(xh + r * m + a);
+                const uint32_t xv = GRAM ? mont_mul(__ldg(px), __ldg(pt + a), mp) : __ldg(px);
                 uint32_t tv[NV];
-                ldv<NV>(t + r * tstride + yoff, tv);
+                ldv<NV>(pt + yoff, tv);
+                px += sx;
+                pt += st;
 #pragma unroll
-                for (int b = 0; b < NV; b++) mac2(ac[b], xv, tv[b]);
+                for (int b = 0; b < NV; b++) acc[b] = madw(xv, tv[b], acc[b]);
                 if (++cnt == FOLDK) {
 #pragma unroll
-                    for (int b = 0; b < NV; b++) fold2w(ac[b], fc);
+                    for (int b = 0; b < NV; b++) acc[b] = fold1(acc[b], fc);
                     cnt = 0;
                 }
             }
         }
-#pragma unroll
-        for (int b = 0; b < NV; b++) acc[b] = red64(acc2_u64(ac[b]), mp);
     }
     if (pow2) {
+        // (folded, below p 2^32: a Montgomery reduction is a third of a general one; its
+        // factor 2^-32, twice, is made up for once per entry below)
+#pragma unroll
+        for (int b = 0; b < NV; b++) acc[b] = mont_redc(fold1(acc[b], fc), mp);
         // lanes of a warp with the same a hold the same (a, b) entries:
         // butterfly over the slot bits (offsets m, 2m, ..., 16)
         for (int off = m; off < 32; off <<= 1)
@@ -120,16 +134,19 @@ __global__ void __launch_bounds__(PROJ_THREADS)
             for (int b = 0; b < NV; b++) acc[b] += __shfl_xor_sync(0xffffffffu, acc[b], off);
         if (lane < m)
 #pragma unroll
-            for (int b = 0; b < NV; b++) red32[(warp * m + lane) * NV + b] = red64(acc[b], mp);
+            for (int b = 0; b < NV; b++) red32[(warp * m + lane) * NV + b] = mont_redc(acc[b], mp);
         __syncthreads();
         unsigned long long *dst = s_raw + (size_t)k_term * m * n;
         for (int e = tid; e < m * n; e += PROJ_THREADS) {
             const int aa = e / n, b = e % n;
             unsigned long long v = 0;
             for (int w = 0; w < PROJ_THREADS / 32; w++) v += red32[(w * m + aa) * NV + b];
+            v = to_mont(to_mont(red64(v, mp), mp), mp);
             if (v) atomicAdd(dst + e, v);
         }
     } else {
+#pragma unroll
+        for (int b = 0; b < NV; b++) acc[b] = red64(acc[b], mp);
         for (int i = tid; i < m * NV; i += PROJ_THREADS) red[i] = 0;
         __syncthreads();
         if (slot < per) {
@@ -490,9 +507,9 @@ template <int NV, bool GRAM>
 void launch_project_t(wr_ctx *ctx, dim3 grid, const GramItems &items, int count, int m, int n, const int *term_counter,
                       int tmul, int64_t L, int tstride, int yoff) {
     if (tstride <= 0) tstride = NV;
-    bool small = true;  // p < 2^30 for every item: sums folded every 14 products, else every 2
-    for (int i = 0; i < count; i++) small = small && items.item[i].mp.lazy >= 16;
-    launch_dep(ctx, small ? k_project<NV, 14, GRAM> : k_project<NV, 2, GRAM>, grid, dim3(PROJ_THREADS), 0, items, m, n,
+    bool small = true;  // p <= 2^30 for every item: sums folded after 12 products, else after 4
+    for (int i = 0; i < count; i++) small = small && items.item[i].mp.p <= (1u << 30);
+    launch_dep(ctx, small ? k_project<NV, 12, GRAM> : k_project<NV, 4, GRAM>, grid, dim3(PROJ_THREADS), 0, items, m, n,
                term_counter, tmul, L, tstride, yoff);
 }
 

@@ -89,3 +89,26 @@ def test_groups_of_tiles_in_both_accumulators(wr, m, stride, yoff, groups):
             out.append(G.cpu().clone())
         assert torch.equal(out[0], out[1]), tiles
     wr.wr_destroy(ctx)
+
+
+@pytest.mark.parametrize("m,stride,yoff", [(1, 1, 0), (2, 4, 2), (3, 4, 0), (5, 16, 8), (8, 8, 0), (12, 16, 0), (16, 32, 16),
+                                           (32, 32, 0)])
+@pytest.mark.parametrize("p", [3, 65521, 1073741789, 2147483647])
+def test_integer_products(wr, m, stride, yoff, p):
+    """The multiply-add path: both folds, rows around its batches of rows, widths that
+    divide a warp and others."""
+    ctx = wr.wr_create(0)
+    wr.wr_set_tensor_projection(ctx, 0)
+    rng = np.random.default_rng(m)
+    for N in (1, 31, 300, 20011, 60000):
+        t = rng.integers(0, p, size=(N, stride))
+        t[: N // 2] = p - 1
+        w = rng.integers(0, p, size=N)
+        w[: N // 3] = p - 1
+        dt = torch.from_numpy(t.astype(np.uint32).view(np.int32)).cuda()
+        dw = torch.from_numpy(w.astype(np.uint32).view(np.int32)).cuda()
+        G = torch.empty((m, m), dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        wr.wr_gram_device(ctx, p, N, m, m, dt, stride, yoff, dw, G)
+        assert np.array_equal(G.cpu().numpy().astype(np.int64), _ref(t, w, m, m, yoff, p)), N
+    wr.wr_destroy(ctx)
