@@ -113,6 +113,14 @@ __host__ __device__ __forceinline__ uint32_t red64(uint64_t x, const ModP &m) {
 // kernels read the matrix layouts only.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A word that an earlier kernel of such a chain may still be writing while this one is
+// resident: a plain load after pdl_wait.  (const __restrict__ and __ldg become
+// ld.global.nc, defined only for memory that nobody writes during the kernel.)
+__device__ __forceinline__ uint32_t ld_plain(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 
 // thread block clusters
 __device__ __forceinline__ uint32_t cluster_rank() {

@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(AS_THREADS)
     for (int x = threadIdx.x; x < rows * nv; x += AS_THREADS) {
         const int rl = x / nv, b = x % nv;
         const int64_t r = r0 + rl, g = nmap ? (int64_t)nmap[r] : r;
-        out[r * nv + b] = b < width ? mulm(ds[rl], in[g * width + b], mp) : 0;
+        out[r * nv + b] = b < width ? mulm(ds[rl], ld_plain(in + g * width + b), mp) : 0;
     }
 }
 
@@ -294,7 +294,7 @@ __global__ void k_unpad(int64_t N, int width, int nv, const uint32_t *__restrict
     int64_t r = i / width;
     int b = (int)(i % width);
     const int64_t g = nmap ? (int64_t)nmap[r] : r;
-    out[g * width + b] = in[r * nv + b];
+    out[g * width + b] = ld_plain(in + r * nv + b);
 }
 
 // The iterated block in the matrix's row order, unscaled (T = D1 V): from the

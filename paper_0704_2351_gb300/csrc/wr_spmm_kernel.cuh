@@ -112,17 +112,20 @@ __device__ __forceinline__ void mac(int64_t (&acc)[W], int a, const uint32_t (&v
 // The gathers of a batch: volatile loads keep their program order, so a batch
 // of U gathers is in flight before its first product (left to itself the
 // compiler interleaves loads and products to stay at 32 registers, with two or
-// three gathers in flight).
+// three gathers in flight).  Plain loads, not the non-coherent ones: under a
+// dependent launch (launch_dep) this kernel is resident while the one before it
+// still writes the block, and ld.global.nc is defined only for memory that nobody
+// writes during the kernel.
 template <int W>
 __device__ __forceinline__ void gather(const uint32_t *p, uint32_t (&v)[W]) {
     if constexpr (W == 1) {
-        asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v[0]) : "l"(p));
+        asm volatile("ld.global.u32 %0, [%1];" : "=r"(v[0]) : "l"(p));
     } else if constexpr (W == 2) {
-        asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "l"(p));
+        asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "l"(p));
     } else {
 #pragma unroll
         for (int k = 0; k < W / 4; k++)
-            asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
+            asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
                          : "=r"(v[4 * k]), "=r"(v[4 * k + 1]), "=r"(v[4 * k + 2]), "=r"(v[4 * k + 3])
                          : "l"(p + 4 * k));
     }
@@ -145,7 +148,7 @@ __device__ __forceinline__ void job_of(const MultiEpi &me, int col0, ModP &mp, c
 }
 
 // The scale residue of output row tgt (0 for a split or absent row), loaded
-// ahead of the row's gathers.
+// ahead of the row's gathers (a plain load, as the gathers).
 template <bool MULTI>
 __device__ __forceinline__ uint32_t row_scale(uint32_t tgt, const uint32_t *scale, const MultiEpi &me, int col0) {
     if (tgt & VROW_SPLIT) return 0u;  // (VROW_EMPTY has the bit set)
@@ -153,7 +156,7 @@ __device__ __forceinline__ uint32_t row_scale(uint32_t tgt, const uint32_t *scal
         ModP mp;
         job_of(me, col0, mp, scale);
     }
-    return __ldg(scale + tgt);
+    return ld_plain(scale + tgt);
 }
 
 // part: 0 the whole pass (y = scale (A x)); with column slabs of the matrix
@@ -456,7 +459,7 @@ __global__ void k_finalize_split(int64_t nsplit, int nv, const int32_t *__restri
     uint32_t *yr = y + (size_t)r * nv + b;
     uint32_t v = red_s64((int64_t)s, mp);
     if (part >= 2) v = addm(v, *yr, mp);
-    if (part == 0 || part == 3) v = mulm(scale[r], v, mp);
+    if (part == 0 || part == 3) v = mulm(ld_plain(scale + r), v, mp);
     *yr = v;
 }
 
