@@ -111,7 +111,7 @@ __device__ __forceinline__ void put_digits(unsigned char *tile, uint32_t off, co
 // G into s_raw[k] (k = tmul * counter + toff; skipped unless 0 <= k < L): the
 // per-block result reduced mod p, then added with exact uint64 atomics.
 // w: the N weights in Montgomery form (mont_mul(w_r, x) = w_r x mod p); t and w
-// 16-byte aligned (bulk copies).
+// 16-byte aligned (bulk copies), col a multiple of 4.
 //
 // Roles: warps 0-7 convert (tile tl: wait for its raw rows and for the MMAs
 // that last read its operand stage, write the digit tiles, one arrival per
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
     using S = GramShape<NB, RB>;
     const GramItem &it = items.item[blockIdx.y];
     const int64_t N = it.rows;
-    const uint32_t *__restrict__ w = it.w, *__restrict__ t = it.t;
+    const uint32_t *__restrict__ w = it.w, *__restrict__ t = it.t + it.col;
     const ModP mp = it.mp;
     pdl_launch();
     constexpr int RW = RB / 4;      // residues per raw row
@@ -192,8 +192,10 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
         const int64_t r0 = (t_begin + tl) * GT_KT;
         const uint32_t rows = (uint32_t)min64(GT_KT, N - r0);
         const uint32_t wrows = rows & ~3u;  // whole 16-byte groups of weights; the rest by plain loads
-        tc::mbar_arrive_expect_tx(&bar_raw[s], rows * (uint32_t)RB + wrows * 4u);
-        tc::bulk_g2s(raw + s * S::RAWB, t + r0 * RW, rows * (uint32_t)RB, &bar_raw[s]);
+        // rows from column col on, whole rows apart: the last row ends col words early
+        const uint32_t bytes = rows * (uint32_t)RB - (r0 + rows == N ? (uint32_t)it.col * 4u : 0u);
+        tc::mbar_arrive_expect_tx(&bar_raw[s], bytes + wrows * 4u);
+        tc::bulk_g2s(raw + s * S::RAWB, t + r0 * RW, bytes, &bar_raw[s]);
         if (wrows) tc::bulk_g2s(wts + s * GT_KT, w + r0, wrows * 4u, &bar_raw[s]);
     };
 

@@ -573,15 +573,16 @@ bool sigma_uses_pm(const wr_ctx *ctx, int64_t L, int m, int n, bool early = fals
 void copy_settings(const wr_ctx *parent, wr_ctx *child);
 wr_status blackbox_apply(wr_ctx *ctx, const wr_matrix *mat, const wr_params &prm,
                          const uint32_t *d_in, uint32_t *d_out, int64_t width);
-// Gram products of one launch: item y adds sum_r w_r t[r][0..m)^T t[r][yoff..yoff+n)
-// mod p over its rows (w in Montgomery form) to s_raw[k], k = tmul * counter + toff
-// (skipped unless 0 <= k < L).
+// Gram products of one launch: item y adds sum_r w_r t[r][col..col+m)^T
+// t[r][col+yoff..col+yoff+n) mod p over its rows (w in Montgomery form) to s_raw[k],
+// k = tmul * counter + toff (skipped unless 0 <= k < L).  t is the start of the block's
+// rows (a job's slice of a wider block starts at column col: nothing past the rows is read).
 constexpr int GRAM_MAX_ITEMS = 2 * 4;  // both sides of an application for up to MULTI_MAX_JOBS jobs
 struct GramItem {
     int64_t rows;
     const uint32_t *w, *t;
     unsigned long long *s_raw;
-    int toff;
+    int col, toff;
     ModP mp;
 };
 struct GramItems {

@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(PROJ_THREADS, NV <= 8 ? 4 : 2)
               int64_t L, int tstride, int yoff) {
     const GramItem &it = items.item[blockIdx.y];
     const int64_t N = it.rows;
-    const uint32_t *__restrict__ xh = it.w, *__restrict__ t = it.t;
+    const uint32_t *__restrict__ xh = it.w, *__restrict__ t = it.t + it.col;
     unsigned long long *__restrict__ s_raw = it.s_raw;
     const ModP mp = it.mp;
     pdl_launch();
@@ -663,14 +663,14 @@ static wr_status launch_gram(wr_ctx *ctx, SeqState &st, int64_t rows, const uint
                              int tmul, int toff, int tstride, int yoff, const int *counter = nullptr) {
     if (rows <= 0) return WR_OK;
     GramItems g{};
-    g.item[0] = GramItem{rows, w, t, st.s_raw.as<unsigned long long>(), toff, st.mp};
+    g.item[0] = GramItem{rows, w, t, st.s_raw.as<unsigned long long>(), 0, toff, st.mp};
     return launch_grams(ctx, st.r, g, 1, tmul, tstride, yoff, counter ? counter : st.counter.as<int>(), st.err.as<int>());
 }
 
 // S_raw[counter + 0] += Xh^T T (the generic projection, one term per application)
 static wr_status launch_generic(wr_ctx *ctx, SeqState &st, int64_t L) {
     GramItems g{};
-    g.item[0] = GramItem{st.r.N, st.xh.as<uint32_t>(), st.T.as<uint32_t>(), st.s_raw.as<unsigned long long>(), 0, st.mp};
+    g.item[0] = GramItem{st.r.N, st.xh.as<uint32_t>(), st.T.as<uint32_t>(), st.s_raw.as<unsigned long long>(), 0, 0, st.mp};
     return launch_project(ctx, g, 1, st.r.m, st.r.n, st.r.nv, st.counter.as<int>(), false, 1, L, st.r.nvs, 0);
 }
 
@@ -796,8 +796,8 @@ static wr_status seq_iteration(wr_ctx *ctx, SeqState &st, cudaEvent_t *ev) {
     if (st.r.gram || st.r.paired) {
         // both Gram products of the application in one launch
         GramItems g{};
-        g.item[0] = GramItem{st.r.M, st.w2.as<uint32_t>(), st.Wb.as<uint32_t>(), st.s_raw.as<unsigned long long>(), -1, st.mp};
-        g.item[1] = GramItem{st.r.N, st.xh.as<uint32_t>(), st.T.as<uint32_t>(), st.s_raw.as<unsigned long long>(), 0, st.mp};
+        g.item[0] = GramItem{st.r.M, st.w2.as<uint32_t>(), st.Wb.as<uint32_t>(), st.s_raw.as<unsigned long long>(), 0, -1, st.mp};
+        g.item[1] = GramItem{st.r.N, st.xh.as<uint32_t>(), st.T.as<uint32_t>(), st.s_raw.as<unsigned long long>(), 0, 0, st.mp};
         WR_TRY(launch_grams(ctx, st.r, g, 2, 2, nv, st.r.paired ? st.r.nv : 0, st.counter.as<int>(), st.err.as<int>()));
     } else {
         WR_TRY(launch_generic(ctx, st, st.r.L));
@@ -1070,7 +1070,7 @@ wr_status gram_device(wr_ctx *ctx, uint32_t p, int64_t N, int m, int n, const ui
         r.nv = nv;
         r.L = 1;
         GramItems g{};
-        g.item[0] = GramItem{N, w, t, s_raw, 0, mp};
+        g.item[0] = GramItem{N, w, t, s_raw, 0, 0, mp};
         WR_TRY(launch_grams(ctx, r, g, 1, 1, tstride, yoff, counter, err));
     }
     k_reduce_scaled<<<blocks_for((int64_t)m * n, 256), 256, 0, s>>>(m * n, s_raw, G, mp.r1, mp);
@@ -1249,8 +1249,8 @@ wr_status run_sequence_multi(wr_ctx *ctx, const wr_matrix *mat, const std::vecto
         for (int g = 0; g < G; g++) {
             Job &j = jobs[g];
             unsigned long long *sr = j.s_raw.as<unsigned long long>();
-            if (w_side && M > 0) it.item[k++] = GramItem{M, j.w2.as<uint32_t>(), Wb.as<uint32_t>() + g * jw, sr, -1, j.mp};
-            if (N > 0) it.item[k++] = GramItem{N, j.xh.as<uint32_t>(), T.as<uint32_t>() + g * jw, sr, 0, j.mp};
+            if (w_side && M > 0) it.item[k++] = GramItem{M, j.w2.as<uint32_t>(), Wb.as<uint32_t>(), sr, g * jw, -1, j.mp};
+            if (N > 0) it.item[k++] = GramItem{N, j.xh.as<uint32_t>(), T.as<uint32_t>(), sr, g * jw, 0, j.mp};
         }
         return k > 0 ? launch_grams(ctx, rs[0], it, k, 2, W, r0.nv, counter.as<int>(), err.as<int>()) : WR_OK;
     };
