@@ -486,6 +486,7 @@ static wr_status ensure_twiddles(wr_ctx *ctx, int lg) {
     if (ctx->ntt_lg >= lg) return WR_OK;
     const int LG = std::max(lg, 14);
     const int64_t half = (int64_t)1 << (LG - 1);
+    ctx->ntt_lg = 0;  // (the old table goes back first: none is there until this one is whole)
     WR_TRY(dev_alloc(ctx, ctx->ntt_tw, sizeof(uint32_t) * (size_t)(2 * NTT_NPRIMES) * half));
     for (int i = 0; i < NTT_NPRIMES; i++) {
         const uint32_t P = NTT_PRIMES[i];
