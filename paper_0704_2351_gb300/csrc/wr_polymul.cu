@@ -243,8 +243,9 @@ __host__ __device__ inline NttSteps ntt_steps(int lc) {
 __device__ __forceinline__ int ntt_pad(int e) { return e + (e >> 5); }
 
 // One step: h0 the lowest bit it touches.  SRC / DST: 0 shared memory, 1 the
-// tile in natural order, 2 the tile in the transform's order.
-template <int R, bool FWD, int SRC, int DST>
+// tile in natural order, 2 the tile in the transform's order.  SHORT: transforms past
+// the end are left out.
+template <int R, bool FWD, bool SHORT, int SRC, int DST>
 __device__ __forceinline__ void ntt_step(uint32_t *sm, uint32_t *__restrict__ g, int valid, int lc, int h0, uint32_t top,
                                          const uint32_t *__restrict__ tw, uint32_t P, uint32_t pneg) {
     constexpr int NG = 16 >> R;  // groups per thread
@@ -255,6 +256,7 @@ __device__ __forceinline__ void ntt_step(uint32_t *sm, uint32_t *__restrict__ g,
         const int gp = gi & ((1 << (lc - R)) - 1);  // group within its transform
         const int pbase = ((gi >> (lc - R)) << lc) + gp;
         const uint32_t blk = (top << (lc - h0 - R)) + (uint32_t)((base & ((1 << lc) - 1)) >> (h0 + R));
+        if (SHORT && base >> lc << lc >= valid) continue;
         uint32_t v[1 << R];
 #pragma unroll
         for (int i = 0; i < (1 << R); i++) {
@@ -274,7 +276,10 @@ __device__ __forceinline__ void ntt_step(uint32_t *sm, uint32_t *__restrict__ g,
     }
 }
 
-template <bool FWD>
+// SHORT: a launch of a single tile that is not full (a product of a few short
+// polynomials: 1 x 1 x 1, 100 coefficients, 118 -> 106 us; the test cost launches of
+// many tiles 2 %, so their last tile takes the empty transforms along).
+template <bool FWD, bool SHORT>
 __global__ void __launch_bounds__(NTT_TILE_THREADS, 2)
     k_ntt_tile(uint32_t *__restrict__ a, int64_t words, int lg, int lc, const uint32_t *__restrict__ tw, uint32_t P,
                uint32_t pneg) {
@@ -291,9 +296,9 @@ __global__ void __launch_bounds__(NTT_TILE_THREADS, 2)
         if (k > 0) __syncthreads();
 #define WR_NTT_STEP(SRC, DST)                                                                    \
     {                                                                                            \
-        if (R == 4) ntt_step<4, FWD, SRC, DST>(sm, g, valid, lc, h0, top, tw, P, pneg);          \
-        else if (R == 3) ntt_step<3, FWD, SRC, DST>(sm, g, valid, lc, h0, top, tw, P, pneg);     \
-        else ntt_step<2, FWD, SRC, DST>(sm, g, valid, lc, h0, top, tw, P, pneg);                 \
+        if (R == 4) ntt_step<4, FWD, SHORT, SRC, DST>(sm, g, valid, lc, h0, top, tw, P, pneg);          \
+        else if (R == 3) ntt_step<3, FWD, SHORT, SRC, DST>(sm, g, valid, lc, h0, top, tw, P, pneg);     \
+        else ntt_step<2, FWD, SHORT, SRC, DST>(sm, g, valid, lc, h0, top, tw, P, pneg);                 \
     }
         if (k == 0) WR_NTT_STEP((FWD ? 1 : 2), 0)
         else if (k + 1 < st.n) WR_NTT_STEP(0, 0)
@@ -522,7 +527,8 @@ static wr_status ntt_run(wr_ctx *ctx, uint32_t *a, int64_t npoly, int lg, const 
     };
     auto tiles = [&]() -> wr_status {
         const int64_t words = npoly << lg;
-        k_ntt_tile<FWD><<<(unsigned)((words + (1 << NTT_TILE_LOG) - 1) >> NTT_TILE_LOG), NTT_TILE_THREADS, 0, st>>>(
+        auto *k = words < (1 << NTT_TILE_LOG) ? k_ntt_tile<FWD, true> : k_ntt_tile<FWD, false>;
+        k<<<(unsigned)((words + (1 << NTT_TILE_LOG) - 1) >> NTT_TILE_LOG), NTT_TILE_THREADS, 0, st>>>(
             a, words, lg, lc, tw, mP.p, mP.pneg);
         WR_LAUNCHED(ctx);
         return WR_OK;
@@ -617,8 +623,11 @@ static wr_status polymat_mul_run(wr_ctx *ctx, const uint32_t *A, int64_t na, con
         WR_TRY(ntt_run<true>(ctx, bufB.as<uint32_t>(), nB, lg, tw, mP[i]));
         // the tile of C that a block covers: 16 x 16, or less where C is smaller
         // (the block then takes more groups of points)
+        // (few entries of C and a long sum: four k a stage, 1 x 64 x 1, 1,000 coefficients
+        // 253 -> 241 us; two for up to 8, 2 x 5 x 7, 30,000 coefficients 264 and 271)
         uint32_t *pA = bufA.as<uint32_t>(), *pB = bufB.as<uint32_t>(), *pC = bufC[i].as<uint32_t>();
-        if (r <= 4 && t <= 8) WR_TRY((pointwise_run<1, 1, 2>(ctx, pA, pB, pC, r, s, t, Lz, mP[i])));
+        if (r <= 4 && t <= 8 && s <= 8) WR_TRY((pointwise_run<1, 1, 2>(ctx, pA, pB, pC, r, s, t, Lz, mP[i])));
+        else if (r <= 4 && t <= 8) WR_TRY((pointwise_run<1, 1, 4>(ctx, pA, pB, pC, r, s, t, Lz, mP[i])));
         else if (t <= 8) WR_TRY((pointwise_run<2, 1, 4>(ctx, pA, pB, pC, r, s, t, Lz, mP[i])));
         else if (r <= 8) WR_TRY((pointwise_run<2, 2, 4>(ctx, pA, pB, pC, r, s, t, Lz, mP[i])));
         else WR_TRY((pointwise_run<4, 2, 8>(ctx, pA, pB, pC, r, s, t, Lz, mP[i])));
