@@ -134,7 +134,6 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
     const int64_t N = it.rows;
     const uint32_t *__restrict__ w = it.w, *__restrict__ t = it.t + it.col;
     const ModP mp = it.mp;
-    pdl_launch();
     constexpr int RW = RB / 4;      // residues per raw row
     constexpr int HB = NB / 2;      // right-factor columns a draining thread holds
     constexpr uint32_t IDESC = tc::idesc_f16_f32(128, S::TN);
@@ -155,7 +154,6 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
     const int64_t t_begin = tiles * blockIdx.x / gridDim.x;
     const int ntile = (int)(tiles * (blockIdx.x + 1) / gridDim.x - t_begin);
 
-    // (everything up to pdl_wait overlaps the pass before)
     // both operand stages start at zero: digit rows of absent columns stay zero
     for (uint32_t i = (uint32_t)tid * 16u; i < 2u * S::OPB; i += GT_THREADS * 16u)
         *reinterpret_cast<uint4 *>(base + i) = make_uint4(0u, 0u, 0u, 0u);
@@ -179,8 +177,7 @@ __global__ void __launch_bounds__(GT_THREADS, 2)
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    pdl_wait();
-    const int64_t k_term = term_counter ? (int64_t)tmul * *term_counter + it.toff : (int64_t)it.toff;
+    const int64_t k_term = (int64_t)tmul * *term_counter + it.toff;
     if (k_term < 0 || k_term >= L) {  // the same for every block of the item
         if (warp == 0) tc::tmem_dealloc(tmem, S::TMEM_COLS);
         return;
@@ -415,8 +412,8 @@ wr_status launch_gram_tc_t(wr_ctx *ctx, const GramItems &items, int count, int m
     const unsigned grid =
         (unsigned)std::min<int64_t>(tiles, std::max<int64_t>(std::max(1, 2 * ctx->num_sms / count), (tiles + most - 2) / (most - 1)));
     if (grid == 0) return WR_OK;
-    launch_dep(ctx, k_gram_tc<NB, RB>, dim3(grid, (unsigned)count), dim3(GT_THREADS), S::SMEM, items, m, n, yoff,
-               term_counter, tmul, L, err);
+    k_gram_tc<NB, RB><<<dim3(grid, (unsigned)count), GT_THREADS, S::SMEM, ctx->stream>>>(items, m, n, yoff, term_counter, tmul, L,
+                                                                                        err);
     WR_LAUNCHED(ctx);
     return WR_OK;
 }

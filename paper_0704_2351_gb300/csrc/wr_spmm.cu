@@ -54,8 +54,6 @@ __global__ void __launch_bounds__(PROJ_THREADS, NV <= 8 ? 4 : 2)
     const uint32_t *__restrict__ xh = it.w, *__restrict__ t = it.t + it.col;
     unsigned long long *__restrict__ s_raw = it.s_raw;
     const ModP mp = it.mp;
-    pdl_launch();
-    pdl_wait();
     const int64_t k_term = (int64_t)tmul * *term_counter + it.toff;
     if (k_term < 0 || k_term >= L) return;  // the same for every thread
     // red32[w][a][b]: per-warp sums reduced mod p (m divides 32); red: one
@@ -176,8 +174,6 @@ __global__ void k_reduce_seq(int64_t count, const unsigned long long *__restrict
 // permutation of A~'s rows and columns, X and Y)
 __global__ void k_derive_diag(uint64_t seed, uint64_t tag, int64_t len, uint32_t p,
                               uint32_t *__restrict__ out, const uint32_t *__restrict__ map) {
-    pdl_launch();
-    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < len) {
         const uint64_t gi = map ? (uint64_t)map[i] : (uint64_t)i;
@@ -193,8 +189,6 @@ __global__ void k_prepare(int64_t N, int m, int n, int nv, uint64_t seed, uint64
                           int ycol0, int gram, int paired, const uint32_t *__restrict__ d1, uint32_t *__restrict__ t0,
                           uint32_t *__restrict__ xh, uint32_t *__restrict__ d1sq, const uint32_t *__restrict__ nmap,
                           ModP mp, int trow) {
-    pdl_launch();
-    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const uint64_t gi = nmap ? (uint64_t)nmap[i] : (uint64_t)i;  // index of the draws
@@ -230,8 +224,6 @@ __global__ void k_prepare(int64_t N, int m, int n, int nv, uint64_t seed, uint64
 // out = d^{-1} R mod p, elementwise (the Gram weights D2^{-1} of the odd terms of
 // the symmetric projection: S_2k+1 = W^T D2^{-1} W with W = D2 A D1 V_k)
 __global__ void k_inv_diag(int64_t len, const uint32_t *__restrict__ d, uint32_t *__restrict__ out, ModP mp) {
-    pdl_launch();
-    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < len) out[i] = to_mont(invm(d[i], mp), mp);  // Montgomery form for the Gram projection
 }
@@ -275,8 +267,6 @@ __global__ void __launch_bounds__(AS_THREADS)
 __global__ void k_scale_pad(int64_t N, int width, int nv, const uint32_t *__restrict__ in,
                             const uint32_t *__restrict__ d1, uint32_t *__restrict__ out,
                             const uint32_t *__restrict__ nmap, ModP mp) {
-    pdl_launch();
-    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N * nv) return;
     int64_t r = i / nv;
@@ -376,8 +366,7 @@ wr_status launch_spmm_t(wr_ctx *ctx, const SellView &A, const uint32_t *x, uint3
     if (finalize && A.nsplit > 0) {
         int64_t cnt = A.nsplit * NV;
         if (me && me->jobs > 1)
-            launch_dep(ctx, k_finalize_split_multi, dim3(blocks_for(cnt, 256)), dim3(256), 0, A.nsplit, NV, A.split_row,
-                       acc64, y, *me);
+            k_finalize_split_multi<<<blocks_for(cnt, 256), 256, 0, ctx->stream>>>(A.nsplit, NV, A.split_row, acc64, y, *me);
         else
             launch_dep(ctx, k_finalize_split, dim3(blocks_for(cnt, 256)), dim3(256), 0, A.nsplit, NV, A.split_row, acc64,
                        y, scale, mp, part);
@@ -509,8 +498,8 @@ void launch_project_t(wr_ctx *ctx, dim3 grid, const GramItems &items, int count,
     if (tstride <= 0) tstride = NV;
     bool small = true;  // p <= 2^30 for every item: sums folded after 12 products, else after 4
     for (int i = 0; i < count; i++) small = small && items.item[i].mp.p <= (1u << 30);
-    launch_dep(ctx, small ? k_project<NV, 12, GRAM> : k_project<NV, 4, GRAM>, grid, dim3(PROJ_THREADS), 0, items, m, n,
-               term_counter, tmul, L, tstride, yoff);
+    auto *k = small ? k_project<NV, 12, GRAM> : k_project<NV, 4, GRAM>;
+    k<<<grid, PROJ_THREADS, 0, ctx->stream>>>(items, m, n, term_counter, tmul, L, tstride, yoff);
 }
 
 // Per item, gram = false: S_raw[k] += w^T t (w: rows x m).  gram = true: S_raw[k] +=
@@ -713,13 +702,11 @@ static wr_status seq_setup(wr_ctx *ctx, const wr_matrix *mat, const Resolved &r,
         WR_LAUNCHED(ctx);
     }
     if (r.N > 0) {
-        launch_dep(ctx, k_derive_diag, dim3(blocks_for(r.N, 256)), dim3(256), 0, r.seed, TAG_D1, r.N, r.p,
-                   st.D1.as<uint32_t>(), r.nmap);
+        k_derive_diag<<<blocks_for(r.N, 256), 256, 0, s>>>(r.seed, TAG_D1, r.N, r.p, st.D1.as<uint32_t>(), r.nmap);
         WR_LAUNCHED(ctx);
     }
     if (r.M > 0) {
-        launch_dep(ctx, k_derive_diag, dim3(blocks_for(r.M, 256)), dim3(256), 0, r.seed, TAG_D2, r.M, r.p,
-                   st.D2.as<uint32_t>(), r.mmap);
+        k_derive_diag<<<blocks_for(r.M, 256), 256, 0, s>>>(r.seed, TAG_D2, r.M, r.p, st.D2.as<uint32_t>(), r.mmap);
         WR_LAUNCHED(ctx);
     }
     if (r.N > 0) {

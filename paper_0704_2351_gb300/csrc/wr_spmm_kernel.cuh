@@ -466,8 +466,6 @@ __global__ void k_finalize_split(int64_t nsplit, int nv, const int32_t *__restri
 // the same for a multi-job block: column b is reduced with its job's modulus and scale
 __global__ void k_finalize_split_multi(int64_t nsplit, int nv, const int32_t *__restrict__ split_row,
                                        unsigned long long *__restrict__ acc64, uint32_t *__restrict__ y, MultiEpi me) {
-    pdl_launch();
-    pdl_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nsplit * nv) return;
     int64_t sid = i / nv;
