@@ -80,14 +80,22 @@ ModP make_modp(uint32_t p);
 // Products of at most (p-1)^2 that fit in a 64-bit accumulator on top of what
 // fold1 by c = 2^32 mod p leaves (at most (c + 1)(2^32 - 1)): at least 12 for
 // p <= 2^30, where c < p; at least 4 below 2^31 (there c is 2^32 - 3p < 2^30 or
-// 2^32 - 2p, which leaves 2p 2^32 >= 4 p^2).
-inline int fold1_products(uint32_t p) {
+// 2^32 - 2p, which leaves 2p 2^32 >= 4 p^2).  Kernels fold after FOLD_SMALL products
+// where that many fit, else after FOLD_BIG.
+constexpr int FOLD_SMALL = 12, FOLD_BIG = 4;
+constexpr int fold1_products(uint32_t p) {
     const unsigned __int128 c = ((unsigned __int128)1 << 32) % p;
     const unsigned __int128 after = (c + 1) * (((unsigned __int128)1 << 32) - 1);
     const unsigned __int128 room = (((unsigned __int128)1 << 64) - 1) - after;
     const unsigned __int128 prod = (unsigned __int128)(p - 1) * (p - 1);
-    return prod ? (int)std::min<unsigned __int128>(room / prod, 1000) : 1000;
+    return prod == 0 || room / prod > 1000 ? 1000 : (int)(room / prod);
 }
+static_assert(fold1_products(65537) >= FOLD_SMALL && fold1_products(858993463) >= FOLD_SMALL &&
+                  fold1_products(1073741789) >= FOLD_SMALL,
+              "p <= 2^30");
+static_assert(fold1_products(1431655765) >= FOLD_BIG && fold1_products(1431655777) >= FOLD_BIG &&
+                  fold1_products(2147483629) >= FOLD_BIG && fold1_products(2147483647) == FOLD_BIG,
+              "p < 2^31");
 
 __host__ __device__ __forceinline__ uint64_t mulhi64(uint64_t a, uint64_t b) {
 #ifdef __CUDA_ARCH__

@@ -37,6 +37,11 @@ namespace {
 
 constexpr int NTT_NPRIMES = 3;
 constexpr uint32_t NTT_PRIMES[NTT_NPRIMES] = {998244353u, 469762049u, 2013265921u};  // 119 2^23+1, 7 2^26+1, 15 2^27+1
+// products between folds in the pointwise sums (P < 2^30, else)
+constexpr int PW_FOLD_SMALL = 16, PW_FOLD_BIG = 4;
+static_assert(fold1_products(NTT_PRIMES[0]) >= PW_FOLD_SMALL && fold1_products(NTT_PRIMES[1]) >= PW_FOLD_SMALL &&
+                  fold1_products(NTT_PRIMES[2]) >= PW_FOLD_BIG,
+              "folded sums");
 constexpr int NTT_MAX_LOG = 23;  // 2^23 divides every p_i - 1
 
 uint64_t hpow(uint64_t a, uint64_t e, uint64_t m) {
@@ -546,7 +551,7 @@ template <int WR, int WC, int KC>
 static wr_status pointwise_run(wr_ctx *ctx, const uint32_t *A, const uint32_t *B, uint32_t *C, int r, int s, int t,
                                int64_t Lz, const ModP &mP) {
     using S = PwShape<WR, WC, KC>;
-    auto *k = mP.p < (1u << 30) ? k_ntt_pointwise<WR, WC, KC, 16> : k_ntt_pointwise<WR, WC, KC, 4>;
+    auto *k = mP.p < (1u << 30) ? k_ntt_pointwise<WR, WC, KC, PW_FOLD_SMALL> : k_ntt_pointwise<WR, WC, KC, PW_FOLD_BIG>;
     WR_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM));
     const int64_t tiles = (int64_t)((r + S::TR - 1) / S::TR) * ((t + S::TC - 1) / S::TC);
     const dim3 g((unsigned)((Lz + 32 * S::FG - 1) / (32 * S::FG)), (unsigned)tiles);

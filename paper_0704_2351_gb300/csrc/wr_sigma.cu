@@ -102,6 +102,8 @@ __global__ void k_quiet(const uint32_t *__restrict__ E, int bb, int m, int n, in
 // shared memory, window 141 and product 131 us); q = 16, 11,252 orders, 64 a chunk
 // 69 us (window 85, product 154 us).
 constexpr int TP_THREADS = 256, TP_K = 16;
+constexpr int TP_FOLD = 8;  // (whole groups of a chunk's 16)
+static_assert(TP_FOLD <= FOLD_SMALL && TP_K % TP_FOLD == 0 && TP_K % FOLD_BIG == 0, "folds of a chunk");
 
 template <int NC>
 struct Toep {
@@ -1089,11 +1091,11 @@ static wr_status mbasis_run(wr_ctx *ctx, const uint32_t *d_S, int64_t L, int m, 
     const int MR = m <= 8 ? 8 : (m <= 16 ? 16 : 32);
     int CS = local_cluster(q);
     const int QC = MR == 8 ? (q <= 16 ? 16 : (q <= 32 ? 32 : 40)) : (q <= 32 ? 32 : (MR == 16 ? 48 : 64));
-    const bool big = p > (1u << 30);  // fold1_products: 4 products, else 12
+    const bool big = fold1_products(p) < FOLD_SMALL;
     using LocalFn = void (*)(int, int, int, const uint32_t *, uint32_t *, int32_t *, uint32_t *, int32_t *, int *,
                              uint32_t *, int, ModP);
     LocalFn kloc = nullptr;
-#define WR_LOCAL(MRV, CPLV, QCV) kloc = big ? k_local<MRV, CPLV, QCV, 4> : k_local<MRV, CPLV, QCV, 12>
+#define WR_LOCAL(MRV, CPLV, QCV) kloc = big ? k_local<MRV, CPLV, QCV, FOLD_BIG> : k_local<MRV, CPLV, QCV, FOLD_SMALL>
     if (MR == 8) { if (QC == 16) WR_LOCAL(8, 1, 16); else if (QC == 32) WR_LOCAL(8, 1, 32); else WR_LOCAL(8, 2, 40); }
     else if (MR == 16) { if (QC == 32) WR_LOCAL(16, 1, 32); else WR_LOCAL(16, 2, 48); }
     else { if (QC == 32) WR_LOCAL(32, 1, 32); else WR_LOCAL(32, 2, 64); }
@@ -1143,9 +1145,9 @@ static wr_status mbasis_run(wr_ctx *ctx, const uint32_t *d_S, int64_t L, int m, 
         WR_CUDA(cudaMemcpyAsync(scale.ptr, one.data(), sizeof(uint32_t) * q, cudaMemcpyHostToDevice, s));
         WR_CUDA(cudaStreamSynchronize(s));
     }
-    auto *ktoep = NC == 16 ? (big ? k_toeplitz<16, 4> : k_toeplitz<16, 8>)
-                  : NC == 32 ? (big ? k_toeplitz<32, 4> : k_toeplitz<32, 8>)
-                             : (big ? k_toeplitz<64, 4> : k_toeplitz<64, 8>);
+    auto *ktoep = NC == 16 ? (big ? k_toeplitz<16, FOLD_BIG> : k_toeplitz<16, TP_FOLD>)
+                  : NC == 32 ? (big ? k_toeplitz<32, FOLD_BIG> : k_toeplitz<32, TP_FOLD>)
+                             : (big ? k_toeplitz<64, FOLD_BIG> : k_toeplitz<64, TP_FOLD>);
     DevBuf Esum;
     WR_TRY(dev_alloc(ctx, Esum, sizeof(uint32_t) * (size_t)bmax * m * q));
 

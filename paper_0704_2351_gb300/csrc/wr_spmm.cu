@@ -496,9 +496,9 @@ template <int NV, bool GRAM>
 void launch_project_t(wr_ctx *ctx, dim3 grid, const GramItems &items, int count, int m, int n, const int *term_counter,
                       int tmul, int64_t L, int tstride, int yoff) {
     if (tstride <= 0) tstride = NV;
-    bool small = true;  // p <= 2^30 for every item: sums folded after 12 products, else after 4
-    for (int i = 0; i < count; i++) small = small && items.item[i].mp.p <= (1u << 30);
-    auto *k = small ? k_project<NV, 12, GRAM> : k_project<NV, 4, GRAM>;
+    bool small = true;
+    for (int i = 0; i < count; i++) small = small && fold1_products(items.item[i].mp.p) >= FOLD_SMALL;
+    auto *k = small ? k_project<NV, FOLD_SMALL, GRAM> : k_project<NV, FOLD_BIG, GRAM>;
     k<<<grid, PROJ_THREADS, 0, ctx->stream>>>(items, m, n, term_counter, tmul, L, tstride, yoff);
 }
 
