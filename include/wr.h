@@ -160,11 +160,17 @@ wr_status wr_set_sigma_leaf(wr_ctx *ctx, int64_t orders);
  * forces one (0 = tuned or default).  Results never depend on it. */
 wr_status wr_set_autotune(wr_ctx *ctx, int32_t on);
 /* Route the context's device allocations through the caller's allocator
- * (both callbacks, or NULL, NULL for the default stream-ordered pool).
+ * (both callbacks, or NULL, NULL for the default: one stream-ordered pool per
+ * device, shared by its contexts, which keeps up to 2 GiB of freed memory for
+ * the next call while any of them lives; wr_trim_memory gives it back).
  * Matrices keep the allocator they were loaded with until wr_matrix_free;
  * batch and server slots inherit the context's callbacks, which may then be
  * called from the library's worker threads. */
 wr_status wr_set_allocator(wr_ctx *ctx, wr_alloc_fn alloc, wr_free_fn release, void *user);
+/* Give the freed memory that the device's pool keeps back to the device (for
+ * other libraries of the process, say).  Waits for the context's stream; memory
+ * in use (matrices, calls running on other contexts) stays. */
+wr_status wr_trim_memory(wr_ctx *ctx);
 wr_status wr_set_lane_width(wr_ctx *ctx, int32_t residues);
 /* wr_rank pipeline (on by default): the sigma-basis trails the sequence on a
  * second stream driven by a second host thread.  M-Basis orders k .. k+b-1
@@ -504,7 +510,8 @@ typedef struct {
  * host thread; a queued request is admitted, in arrival order, as soon as a
  * slot is idle and its device-memory estimate (wr_rank_device_bytes) fits
  * beside the requests already resident (hbm_budget; 0 = no limit; a request
- * above the budget is refused at submission with WR_EINVAL).  Requests that
+ * above the budget is refused at submission with WR_EINVAL; freed memory that
+ * the device's pool keeps, up to 2 GiB, is not counted).  Requests that
  * arrive while others are on the GPU therefore start at once and overlap with
  * them on the device; each result is bit-identical to the same request run
  * alone.  Latency is measured from wr_submit to the result being ready. */

@@ -274,6 +274,14 @@ extern "C" wr_status wr_set_allocator(wr_ctx *ctx, wr_alloc_fn alloc, wr_free_fn
     return WR_OK;
 }
 
+extern "C" wr_status wr_trim_memory(wr_ctx *ctx) {
+    if (!ctx) return fail(WR_EINVAL, "null context");
+    WR_CUDA(cudaSetDevice(ctx->device));
+    WR_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (ctx->pool && ctx->pool->pool) WR_CUDA(cudaMemPoolTrimTo(ctx->pool->pool, 0));
+    return WR_OK;
+}
+
 extern "C" wr_status wr_set_autotune(wr_ctx *ctx, int32_t on) {
     if (!ctx) return fail(WR_EINVAL, "null context");
     ctx->autotune = on != 0;

@@ -83,6 +83,7 @@ _sig = {
     "wr_set_sigma_leaf": ([vp, i64], ctypes.c_int),
     "wr_set_autotune": ([vp, i32], ctypes.c_int),
     "wr_set_allocator": ([vp, vp, vp, vp], ctypes.c_int),
+    "wr_trim_memory": ([vp], ctypes.c_int),
     "wr_set_lane_width": ([vp, i32], ctypes.c_int),
     "wr_set_paired_projection": ([vp, i32], ctypes.c_int),
     "wr_set_tensor_projection": ([vp, i32], ctypes.c_int),
@@ -254,6 +255,10 @@ def wr_set_allocator(ctx: int, alloc=None, release=None, user=None) -> None:
 
 
 _allocators = {}
+
+
+def wr_trim_memory(ctx: int) -> None:
+    _check(_lib.wr_trim_memory(vp(ctx)))
 
 
 def wr_set_autotune(ctx: int, on: bool) -> None:
