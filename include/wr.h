@@ -120,7 +120,11 @@ wr_status wr_create(wr_ctx **out, int device, void *cuda_stream);
 void wr_destroy(wr_ctx *ctx);
 /* Message of the last failing call made by this thread ("" if none). */
 const char *wr_last_error(void);
-/* Turn per-kernel CUDA-event sampling of the SpMM passes on (1) or off (0). */
+/* Turn per-kernel CUDA-event sampling of the SpMM passes on (1) or off (0).
+ * With it on every sequence runs as passes, an eighth of them launched one by one
+ * between events; the sequence of a small matrix, which otherwise runs in one
+ * cluster of thread blocks (64 applications a launch), then does so too, and
+ * wr_last_timings describes the passes.  Results do not depend on it. */
 wr_status wr_set_profiling(wr_ctx *ctx, int on);
 wr_status wr_last_timings(const wr_ctx *ctx, wr_timings *out);
 /* Orders per chunk of the blocked sigma-basis (1..64; 0 = automatic).  The
