@@ -389,8 +389,8 @@ size_t max_dynamic(const wr_ctx *ctx) { return std::min<size_t>(ctx->smem_optin,
 // Matrices and blocks that the small loop takes: packed entries, both blocks and a block's
 // entries in shared memory, two terms per application, and sizes whose pass is
 // shorter than the launches it saves: the limit is the shared memory, near which an
-// application of 6,500 x 6,000 with scalar blocks takes 8.1 us against 10.5 and one of
-// 1,000 x 900 with blocks of 4 6.9 against 10.6.  (Symmetric blocks of 16, whose products
+// application of 6,500 x 6,000 with scalar blocks takes 7.1 us against 10.5 and one of
+// 1,000 x 900 with blocks of 4 6.2 against 10.6.  (Symmetric blocks of 16, whose products
 // the passes take to the tensor cores, meet earlier: 257 terms of 500 x 450 1.62 ms
 // against 2.00, of 800 x 720 2.50 against 2.02; of 8, 1,500 x 1,350 1.55 against 1.68,
 // 2,000 x 1,800 1.91 against 1.69.)

@@ -255,15 +255,21 @@ inline int sigma_chunk_default(int q) {
 }
 // PM-Basis by default for sequences longer than SIGMA_PM_MIN_L (q <= 32), with
 // leaves of SIGMA_LEAF_DEFAULT orders: the M-Basis's window and product passes grow
-// with the square of the length (11,252 orders at q = 16: 53 ms, 57 with 2,048-order
-// leaves; 45,002 orders: 387 ms, 198 / 201 / 221 with leaves of 2,048 / 4,096 /
-// 8,192), and trailing a sequence they take its SMs (the rank of the 200,000 x
-// 180,000 matrix: 1,777 ms with the M-Basis chunk by chunk, 1,622 / 1,607 in
-// PM-Basis segments with 2,048- / 4,096-order leaves).  For q > 32 those passes
+// with the square of the length.  M-Basis alone / PM-Basis, ms: q = 2 17,000 orders 34.0 /
+// 35.1, 30,000 62.1 / 60.6, 130,000 337 / 264; q = 4 17,000 39.7 / 39.9, 130,000 478 / 303;
+// q = 8 17,000 50.5 / 49.4, 130,000 842 / 378; q = 16 11,252 53 / 57 (2,048-order leaves),
+// 45,002 387 / 201 (leaves of 2,048 / 8,192: 198 / 221); q = 32 17,000 355 / 174.  Trailing a
+// sequence they take its SMs (the rank of the 200,000 x 180,000 matrix: 1,926 ms with the
+// M-Basis chunk by chunk; in PM-Basis segments 1,711, 1,729 to 1,813 and 1,917 with 2,048-,
+// 4,096- and 8,192-order leaves, the sequence by itself varying by 5 % with the tuner's pick;
+// symmetric 1,520 against 1,391, 1,394 to 1,405 and 1,492).  For q > 32 those passes
 // cost more per order, so PM-Basis with short leaves takes over early: at q =
 // 64, 4,098 orders, 98 / 96 / 105 ms for leaves of 128 / 256 / 512 orders, and
-// against the M-Basis alone 12.9 / 12.0 ms at 600 orders, 21.4 / 22.9 at 1,000,
-// 32.7 / 39.9 at 1,500.  wr_set_sigma_leaf chooses the leaf explicitly.
+// against the M-Basis alone 12.9 / 12.0 ms at 600 orders, 22.4 / 21.3 at 1,030,
+// 44.9 / 34.9 at 1,700; q = 33 10.0 / 11.0 at 1,030, 18.6 / 18.2 at 1,700, 24.5 / 22.5 at 2,100;
+// q = 40 (8 x 32) 9.0 / 10.4, 16.2 / 17.2, 20.7 / 21.1, (20 x 20) 14.6 / 15.4, 27.3 / 25.4,
+// 36.0 / 31.7; q = 48 24.4 / 16.8, 31.8 / 27.6, 42.8 / 34.7.  wr_set_sigma_leaf chooses the
+// leaf explicitly.
 constexpr int64_t SIGMA_LEAF_DEFAULT = 4096;
 constexpr int64_t SIGMA_PM_MIN_L = 16384;
 constexpr int64_t SIGMA_LEAF_WIDE = 256;

@@ -425,9 +425,14 @@ static wr_status tune_lane_width(wr_ctx *ctx, const Sell &S, int nv, int *out) {
     cudaEvent_t e0, e1;
     WR_CUDA(cudaEventCreate(&e0));
     WR_CUDA(cudaEventCreate(&e1));
-    // one warm-up and three timed launches a candidate: 2, 4 and 8 residues a lane,
-    // then the streaming hints with the best of them.  (1 residue a lane was slowest
-    // on every matrix measured, by a third and more.)
+    // one warm-up and three timed launches a candidate: 2, 4 and 8 residues a lane, then
+    // the streaming hints with the best of them.  Sequences with 1 / 2 / 4 / 8 residues
+    // forced, ms: 200,000 x 180,000 power law, rows of 4 3.22 / 3.08 / 3.46; of 8 4.35 /
+    // 3.61 / 3.63 / 5.10; of 16 6.74 / 5.29 / 4.55 / 5.78; of 32 12.8 / 9.0 / 7.9 / 8.3;
+    // 500,000 x 450,000, rows of 4 2.90 / 2.69 / 2.62, of 16 6.65 / 4.93 / 4.35 / 5.06; 1.9M x
+    // 1.95M, rows of 32 38.0 / 27.1 / 24.6 / 25.6.  (Rows of 2 run up to 4 % faster with 1
+    // residue, 100,000 to 400,000 rows; its launches would cost a matrix that is applied
+    // once more than that.)
     float best = 0.0f;
     auto time_one = [&](int variant) -> wr_status {
         for (int k = 0; k < 4; k++) {

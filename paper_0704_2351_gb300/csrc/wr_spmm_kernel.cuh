@@ -216,8 +216,9 @@ __device__ __forceinline__ void row_out(uint32_t tgt, const int64_t (&acc)[W], u
 // 64 a thread for 16-byte lanes (32 resident warps x 8 gathers of 16 bytes a
 // lane), 51 for narrower ones.  Measured per pass on GB300, against one loop
 // that the compiler kept at 32 registers with two or three gathers in flight:
-// 1.9M x 1.95M, 37M entries, rows of 32 residues from a 250 MB block 740 ->
-// 586 us (3.47 GB of DRAM traffic at 5.8-6.1 TB/s, 87 % of the copy rate);
+// 1.9M x 1.95M, 40.7M entries, rows of 32 residues from a 250 MB block 740 ->
+// 608 us on two GPUs, 586 on a third (3.47 GB of DRAM traffic at 5.6-6.1 TB/s,
+// 83-89 % of the copy rate);
 // 500,000 x 450,000, rows of 32 from 58 MB 97 -> 79 us; 200,000 x 180,000
 // power-law, rows of 16 22.9 and 27.2 -> 21.6 and 26.7 us, rows of 8 18.5 and
 // 20.2 -> 17.0 and 20.0 us.  72 registers (7 blocks) and 56 with spills (9 and
