@@ -5,8 +5,8 @@
 // stream on the caller's device) driven by one host thread, so the captured
 // sequence loops and the sigma-basis kernels of different jobs are in flight
 // on the device at the same time: small matrices that cannot fill 152 SMs on
-// their own share the GPU, and the single-block M-Basis chunks of several jobs
-// run side by side.  A job's kernels, launch shapes and arithmetic do not
+// their own share the GPU, and the M-Basis chunks of several jobs (a cluster of
+// 4 to 16 blocks each) run side by side.  A job's kernels, launch shapes and arithmetic do not
 // depend on what runs beside it, so its result is bit-identical to the same
 // job run alone.
 #include <cuda_runtime.h>
