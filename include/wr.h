@@ -105,7 +105,8 @@ typedef struct {
 
 /* Device allocator callbacks (for example PyTorch's caching allocator):
  * alloc(bytes, stream, user) returns device memory usable on `stream` (the
- * context's stream) or NULL; release(ptr, bytes, stream, user) gives it back,
+ * context's stream; memory that is not 16-byte aligned is given back and
+ * asked for again with 16 bytes more) or NULL; release(ptr, bytes, stream, user) gives it back,
  * in stream order (work already queued on `stream` may still use it). */
 typedef void *(*wr_alloc_fn)(size_t bytes, void *stream, void *user);
 typedef void (*wr_free_fn)(void *ptr, size_t bytes, void *stream, void *user);

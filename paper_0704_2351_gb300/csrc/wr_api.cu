@@ -31,11 +31,11 @@ wr_status cuda_fail(cudaError_t e, const char *what) {
 
 void DevBuf::release() {
     if (ptr) {
-        if (free_fn) free_fn(ptr, bytes, (void *)stream, free_user);
+        if (free_fn) free_fn(static_cast<char *>(ptr) - skip, bytes + extra, (void *)stream, free_user);
         else cudaFreeAsync(ptr, stream);
     }
     ptr = nullptr;
-    bytes = 0;
+    bytes = skip = extra = 0;
 }
 
 DevPool::DevPool(int device) {
@@ -77,13 +77,27 @@ std::shared_ptr<DevPool> device_pool(int device) {
 // Device buffers come from the caller's allocator when one is set
 // (wr_set_allocator), else from the context's stream-ordered pool;
 // either way they are used on ctx->stream only and returned on it.
+constexpr size_t DEV_ALIGN = 16;  // 16-byte vector loads, asynchronous and bulk copies
 wr_status dev_alloc(wr_ctx *ctx, DevBuf &b, size_t bytes) {
     b.release();
     if (bytes == 0) bytes = 1;
     void *p = nullptr;
     if (ctx->alloc_fn) {
         p = ctx->alloc_fn(bytes, (void *)ctx->stream, ctx->alloc_user);
-        if (!p) return fail(WR_ENOMEM, "the caller's allocator returned no memory for " + std::to_string(bytes) + " bytes");
+        if (p && reinterpret_cast<uintptr_t>(p) % DEV_ALIGN != 0) {
+            // the kernels' widest accesses need DEV_ALIGN: room to move the start up
+            ctx->free_fn(p, bytes, (void *)ctx->stream, ctx->alloc_user);
+            b.extra = DEV_ALIGN;
+            p = ctx->alloc_fn(bytes + b.extra, (void *)ctx->stream, ctx->alloc_user);
+            if (p) {
+                b.skip = (DEV_ALIGN - reinterpret_cast<uintptr_t>(p) % DEV_ALIGN) % DEV_ALIGN;
+                p = static_cast<char *>(p) + b.skip;
+            }
+        }
+        if (!p) {
+            b.extra = 0;
+            return fail(WR_ENOMEM, "the caller's allocator returned no memory for " + std::to_string(bytes) + " bytes");
+        }
         b.free_fn = ctx->free_fn;
         b.free_user = ctx->alloc_user;
     } else {

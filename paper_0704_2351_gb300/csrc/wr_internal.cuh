@@ -264,11 +264,14 @@ struct DevBuf {
     cudaStream_t stream = nullptr;
     wr_free_fn free_fn = nullptr;  // caller's allocator (nullptr: cudaFreeAsync)
     void *free_user = nullptr;
+    size_t skip = 0;  // ptr past the start of the caller's memory of bytes + extra bytes
+    size_t extra = 0;
     DevBuf() = default;
     DevBuf(const DevBuf &) = delete;
     DevBuf &operator=(const DevBuf &) = delete;
     DevBuf(DevBuf &&o) noexcept
-        : ptr(o.ptr), bytes(o.bytes), stream(o.stream), free_fn(o.free_fn), free_user(o.free_user) {
+        : ptr(o.ptr), bytes(o.bytes), stream(o.stream), free_fn(o.free_fn), free_user(o.free_user), skip(o.skip),
+          extra(o.extra) {
         o.ptr = nullptr;
         o.bytes = 0;
     }
@@ -276,6 +279,7 @@ struct DevBuf {
         if (this != &o) {
             release();
             ptr = o.ptr; bytes = o.bytes; stream = o.stream; free_fn = o.free_fn; free_user = o.free_user;
+            skip = o.skip; extra = o.extra;
             o.ptr = nullptr;
             o.bytes = 0;
         }
